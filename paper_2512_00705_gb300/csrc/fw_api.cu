@@ -244,14 +244,48 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   return FW_OK;
 }
 
-static fw_status with_qctr(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
-                           cudaStream_t st) {
+// Queue counters come from a pool of the graph's own that keeps up to
+// kCounterPoolKeep bytes: the device's default pool gives its memory back at
+// every synchronisation, so that the first walk after one paid about 0.2 ms
+// for mapping it again.
+static constexpr unsigned long long kCounterPoolKeep = 4ull << 20;
+
+static void create_counter_pool(fw_graph* g) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = g->device;
+  if (cudaMemPoolCreate(&g->counter_pool, &props) != cudaSuccess) {
+    g->counter_pool = nullptr;
+    cudaGetLastError();  // not sticky; the default pool serves
+    return;
+  }
+  unsigned long long keep = kCounterPoolKeep;
+  cudaMemPoolSetAttribute(g->counter_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t st) {
+  const size_t bytes = sizeof(unsigned long long) * (size_t)count;
+  void** p = reinterpret_cast<void**>(out);
+  cudaError_t e = g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(*out, 0, bytes, st);
+  if (e != cudaSuccess) cudaFreeAsync(*out, st);
+  return e;
+}
+
+static fw_status with_qctr(const fw_graph* g, const Job* jobs, long long total, bool count, cudaStream_t st) {
+  bool need = true;
+  cudaError_t e = single_needs_queue(g, jobs[0], total, count, &need);
+  if (e != cudaSuccess) return cuda_error(e, "walk launch");
   unsigned long long* q = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&q), sizeof(unsigned long long), st);
-  if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(queue counter)");
-  e = cudaMemsetAsync(q, 0, sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = launch_walk(g, jobs, njobs, total, count, q, st);
-  cudaError_t e2 = cudaFreeAsync(q, st);
+  if (need) {
+    e = alloc_counters(g, 1, &q, st);
+    if (e != cudaSuccess) return cuda_error(e, "queue counter");
+  }
+  e = launch_walk(g, jobs, 1, total, count, q, st);
+  cudaError_t e2 = q ? cudaFreeAsync(q, st) : cudaSuccess;
   if (e != cudaSuccess) return cuda_error(e, "walk launch");
   if (e2 != cudaSuccess) return cuda_error(e2, "cudaFreeAsync(queue counter)");
   return FW_OK;
@@ -339,6 +373,7 @@ static void free_graph(fw_graph* g) {
   if (g->host_copy) cudaStreamDestroy(g->host_copy);
   for (cudaEvent_t ev : g->host_ev)
     if (ev) cudaEventDestroy(ev);
+  if (g->counter_pool) cudaMemPoolDestroy(g->counter_pool);
   delete g;
 }
 
@@ -371,6 +406,7 @@ extern "C" fw_status fw_graph_create(const int32_t* offsets, const int32_t* cols
   g->e = e;
   FW_TRY(cudaGetDevice(&g->device), "cudaGetDevice");
   FW_TRY(cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->device), "cudaDeviceGetAttribute");
+  create_counter_pool(g);
   const cudaMemcpyKind kind = ptr_kind == FW_PTR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const size_t eb = (size_t)(e > 0 ? e : 1);
   FW_TRY(cudaMalloc(&g->d_off, sizeof(int32_t) * ((size_t)n + 1)), "cudaMalloc(offsets)");
@@ -541,7 +577,7 @@ extern "C" fw_status fw_walk(const fw_graph* g, const int32_t* starts, int32_t n
   J.len = len;
   J.gbase = 0;
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
-  return with_qctr(g, &J, 1, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
+  return with_qctr(g, &J, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" fw_status fw_walk_ids(const fw_graph* g, const int32_t* starts, const uint32_t* walker_ids,
@@ -562,7 +598,7 @@ extern "C" fw_status fw_walk_ids(const fw_graph* g, const int32_t* starts, const
   J.len = len;
   J.gbase = 0;
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
-  return with_qctr(g, &J, 1, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
+  return with_qctr(g, &J, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // Rows of at least this many bytes are walked in chunks so that the copy of
@@ -637,7 +673,7 @@ extern "C" fw_status fw_walk_host(fw_graph* g, const int32_t* starts, int32_t nu
     Jc.len = len;
     Jc.gbase = 0;
     Jc.walker_base = J.walker_base + (uint32_t)lo;
-    s = with_qctr(g, &Jc, 1, (long long)(hi - lo), count, ws);
+    s = with_qctr(g, &Jc, (long long)(hi - lo), count, ws);
     if (s != FW_OK) break;
     e = cudaEventRecord(ev[c], ws);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(g->host_copy, ev[c], 0);
@@ -683,7 +719,7 @@ extern "C" fw_status fw_sample_hist(const fw_graph* g, int32_t v, int32_t v_prev
     J.walker_base = base0 + (uint32_t)done;
     J.num_walkers = (int32_t)chunk;
     J.len = 1;
-    s = with_qctr(g, &J, 1, chunk, count, reinterpret_cast<cudaStream_t>(stream));
+    s = with_qctr(g, &J, chunk, count, reinterpret_cast<cudaStream_t>(stream));
     if (s != FW_OK) return s;
     done += chunk;
   }

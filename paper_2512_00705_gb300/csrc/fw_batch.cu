@@ -57,10 +57,9 @@ extern "C" fw_status fw_walk_batch(const fw_graph* g, const fw_job* jobs, int32_
     if (s != FW_OK) return s;
     if (total == 0) continue;
     unsigned long long* q = nullptr;  // one walker queue per algorithm
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&q), sizeof(unsigned long long) * kQueueCounters, st);
-    if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(queue counter)");
-    e = cudaMemsetAsync(q, 0, sizeof(unsigned long long) * kQueueCounters, st);
-    if (e == cudaSuccess) e = launch_walk(g, tab.data(), (int)tab.size(), total, count, q, st);
+    cudaError_t e = alloc_counters(g, kQueueCounters, &q, st);
+    if (e != cudaSuccess) return cuda_error(e, "queue counter");
+    e = launch_walk(g, tab.data(), (int)tab.size(), total, count, q, st);
     cudaError_t e2 = cudaFreeAsync(q, st);
     if (e != cudaSuccess) return cuda_error(e, "batch launch");
     if (e2 != cudaSuccess) return cuda_error(e2, "cudaFreeAsync(queue counter)");

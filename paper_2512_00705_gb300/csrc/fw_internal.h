@@ -52,6 +52,7 @@ struct fw_graph {
   unsigned long long fingerprint = 0;
   double preprocess_ms = 0.0;
   size_t bytes = 0;
+  cudaMemPool_t counter_pool = nullptr;  // queue counters of launches (nullptr: the device's default pool)
   // staging of fw_walk_host
   std::mutex stage_mu;
   int32_t* d_stage_starts = nullptr;
@@ -80,10 +81,16 @@ fw_status make_job(const fw_graph* g, int32_t algo, const fw_params* params, uin
 
 // Launch the walk over `njobs` jobs (total walkers `total`; njobs <= kMaxJobs).
 // `qctr` points to zeroed device counters the launch uses as walker queues:
-// one for a single job, kAlgos (one per algorithm) for several.  Several
+// one for a single job (see single_needs_queue), kAlgos (one per algorithm) for several.  Several
 // jobs give one kernel launch per algorithm present.
 cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
                         unsigned long long* qctr, cudaStream_t stream);
+// Does a single-job launch need a queue counter?  Without one (every walker
+// has a lane of its own) launch_walk may be given qctr = nullptr.
+cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, bool* need);
+// `count` zeroed queue counters for one launch on `stream`, from the graph's
+// pool; release with cudaFreeAsync on the same stream after the launch.
+cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t stream);
 // Several jobs of any algorithms: one launch per algorithm present, on
 // `stream` one after another, or (side: kAlgos - 1 helper streams, ev:
 // kAlgos events) side by side, joined back into `stream`.  qctr: kAlgos

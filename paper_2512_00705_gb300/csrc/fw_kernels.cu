@@ -12,12 +12,12 @@
 namespace fw {
 
 
-template <bool COUNT, bool SHARE = false>
+template <bool COUNT, bool SPREAD = false, bool SHARE = false>
 static cudaError_t prime_single(int* b) {
-  cudaError_t e = walk_blocks_per_sm<1, COUNT, ALGO_WEIGHTED, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_NODE2VEC, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_METAPATH, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_PAGERANK2, SHARE>(b);
+  cudaError_t e = walk_blocks_per_sm<1, COUNT, ALGO_WEIGHTED, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_NODE2VEC, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_METAPATH, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_PAGERANK2, SPREAD, SHARE>(b);
   return e;
 }
 
@@ -26,6 +26,7 @@ cudaError_t prime_walk_occupancy() {
   cudaError_t e = prime_single<false>(&b);
   if (e == cudaSuccess) e = prime_single<true>(&b);
   if (e == cudaSuccess) e = prime_single<false, true>(&b);
+  if (e == cudaSuccess) e = prime_single<false, true, true>(&b);
   if (e == cudaSuccess) e = prime_walk_mixed_occupancy();
   return e;
 }
@@ -40,6 +41,23 @@ static cudaError_t launch_single(const fw_graph* g, const Job* jobs, long long t
     case ALGO_METAPATH: return launch_walk_t<1, COUNT, ALGO_METAPATH>(g, jobs, 1, total, qctr, stream);
     default: return launch_walk_t<1, COUNT, ALGO_PAGERANK2>(g, jobs, 1, total, qctr, stream);
   }
+}
+
+template <bool COUNT>
+static cudaError_t shape_single(const fw_graph* g, const Job* jobs, long long total, LaunchShape* s) {
+  switch (jobs[0].algo) {
+    case ALGO_WEIGHTED: return walk_shape<1, COUNT, ALGO_WEIGHTED>(g, jobs, 1, total, s);
+    case ALGO_NODE2VEC: return walk_shape<1, COUNT, ALGO_NODE2VEC>(g, jobs, 1, total, s);
+    case ALGO_METAPATH: return walk_shape<1, COUNT, ALGO_METAPATH>(g, jobs, 1, total, s);
+    default: return walk_shape<1, COUNT, ALGO_PAGERANK2>(g, jobs, 1, total, s);
+  }
+}
+
+cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, bool* need) {
+  LaunchShape s = {};
+  const cudaError_t e = count ? shape_single<true>(g, &job, total, &s) : shape_single<false>(g, &job, total, &s);
+  *need = !s.spread;
+  return e;
 }
 
 cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,

@@ -5,7 +5,8 @@
 // One warp runs the loop over one walker queue [Sec. 5.3]:
 //   * query fetch   lanes without a walker take the next global walker
 //                   indices with one warp-aggregated atomicAdd on the queue
-//                   counter; a table of jobs is one concatenated index space
+//                   counter (launches with a lane for every walker take them
+//                   by place instead, see LaunchShape); a table of jobs is one concatenated index space
 //                   (job j owns [gbase_j, gbase_j + W_j)).
 //   * plan          [Sec. 3.3, Sec. 4.1]: per walker-step the bound B and the
 //                   sum estimate give the eRJS / eRVS choice (or a forced mode).
@@ -22,6 +23,8 @@
 // All loops are bounded (trial cap, degree, walk length, hub wait limit); no
 // warp waits on another.
 #pragma once
+
+#include <algorithm>
 
 #include "fw_internal.h"
 
@@ -409,10 +412,11 @@ __device__ __forceinline__ int32_t hub_step(const DevGraph& g, const Job* sj, co
 // write rows until the queue is exhausted and the warp holds no walker.
 // `sj` (shared memory) is the queue's job table: its jobs' walkers form the
 // index space [0, total), job j owning [sj[j].gbase, sj[j].gbase + W_j).
-// ALG fixes the algorithm of every job at compile time; SHARE: hub steps
-// may be shared with the block's idle warps (see hub steps).
-template <bool COUNT, int ALG, bool SHARE>
-__device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total,
+// ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
+// has a lane for every walker, `wpw` walkers per warp, and no queue; SHARE:
+// hub steps may be shared with the block's idle warps (see hub steps).
+template <bool COUNT, int ALG, bool SPREAD, bool SHARE>
+__device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
   static_assert(ALG >= 0 && ALG < kAlgos, "the walk loop is compiled for one algorithm");
@@ -461,12 +465,19 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       const int leader = __ffs(nm) - 1;
       const unsigned cntw = __popc(nm);
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(qctr, (unsigned long long)cntw);
-      base = __shfl_sync(kFull, base, leader);
-      if (base + cntw >= (unsigned long long)total) exhausted = true;
+      long long end = total;
+      if (!SPREAD) {
+        if (lane == leader) base = atomicAdd(qctr, (unsigned long long)cntw);
+        base = __shfl_sync(kFull, base, leader);
+        if (base + cntw >= (unsigned long long)total) exhausted = true;
+      } else {  // warp 0 of every block first, then warp 1, ...
+        base = (unsigned)((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (unsigned)wpw;
+        end = min(end, (long long)base + wpw);
+        exhausted = true;
+      }
       if (need) {
         const long long gi = (long long)base + __popc(nm & lt_mask);
-        if (gi < total) {
+        if (gi < end) {
           int j = 0;
           while (j + 1 < njobs && sj[j + 1].gbase <= gi) ++j;
           const Job& J = sj[j];
@@ -871,9 +882,9 @@ __device__ __forceinline__ void load_jobs(const Job* src_jobs, int njobs, Job* s
 // Single-job (or one-algorithm) launch: the job table in shared memory, one
 // walk loop per warp over the launch's queue.  SHARE: idle warps linger to
 // help the block's hub steps.
-template <int NJ, bool COUNT, int ALG, bool SHARE = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false>
 __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(DevGraph g, JobTableN<NJ> tab, int njobs, long long total,
-                                                      unsigned long long* __restrict__ qctr,
+                                                      int wpw, unsigned long long* __restrict__ qctr,
                                                       unsigned* __restrict__ err, DevCounters* __restrict__ cnt) {
   __shared__ Job sj[NJ];
   __shared__ int32_t obuf[kStageSlots * kBlock];
@@ -887,17 +898,17 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(DevGraph g, Jo
   __syncthreads();
   LaneCounters lc;
   lc.zero();
-  walk_loop<COUNT, ALG, SHARE>(g, sj, njobs, total, qctr, err, obuf, &hb, lc);
+  walk_loop<COUNT, ALG, SPREAD, SHARE>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
   if (SHARE) hub_linger<COUNT, ALG>(g, sj, &hb, lc);
   if (COUNT) flush_counters(lc, cnt);
 }
 
-template <int NJ, bool COUNT, int ALG, bool SHARE = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false>
 inline cudaError_t walk_blocks_per_sm(int* out) {
   static std::atomic<int> cached{0};
   int b = cached.load();
   if (b == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SHARE>, kBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE>, kBlock, 0);
     if (e != cudaSuccess) return e;
     b = b > 0 ? b : 1;
     cached.store(b);
@@ -922,30 +933,68 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
   return rvs;
 }
 
+// The shape of one launch.  While every walker can have a lane of its own
+// (`spread`), walkers go to their warps by place, `wpw` to a warp (the other
+// lanes stay idle): a warp pays for the longest of its lanes' paths in every
+// iteration and scans its lanes' long rows one after another, so walkers are
+// spread over the resident warps before they share one -- wpw is the
+// smallest count with which they fit, and blocks fill before warps do.  No
+// queue counter is needed then.  More walkers than lanes: full warps that
+// fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
+// full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
+// x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
+// kernel variant of its own, because the same choice made inside the queued
+// kernel's fetch cost the whole-graph walks 1 to 3 %.
+struct LaunchShape {
+  int grid, wpw;
+  bool spread;
+  bool share;  // spread, with hub sharing
+};
+
+template <int NJ, bool COUNT, int ALG>
+inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, LaunchShape* s) {
+  constexpr int kWarps = kBlock / 32;
+  int bps = 1;
+  cudaError_t e = walk_blocks_per_sm<NJ, COUNT, ALG>(&bps);
+  if (e != cudaSuccess) return e;
+  long long blocks = (long long)g->num_sms * bps;
+  s->wpw = 32;
+  s->spread = s->share = false;
+  if (!COUNT) {
+    s->share = hub_share_pays(g, jobs, njobs, total, blocks * kBlock);
+    e = s->share ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps) : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
+    if (e != cudaSuccess) return e;
+    const long long spread_blocks = (long long)g->num_sms * bps;
+    s->spread = total <= spread_blocks * kBlock;
+    s->share = s->share && s->spread;
+    if (s->spread) {
+      blocks = spread_blocks;
+      s->wpw = (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
+    }
+  }
+  const long long per_block = s->spread ? s->wpw : kBlock;  // a spread launch takes a block for every warp while it can
+  s->grid = (int)std::min<long long>(blocks, std::max<long long>(1, (total + per_block - 1) / per_block));
+  return cudaSuccess;
+}
+
 template <int NJ, bool COUNT, int ALG>
 inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total,
                                  unsigned long long* qctr, cudaStream_t stream) {
-  int blocks_per_sm = 1;
-  cudaError_t oe = walk_blocks_per_sm<NJ, COUNT, ALG>(&blocks_per_sm);
-  if (oe != cudaSuccess) return oe;
+  LaunchShape s;
+  cudaError_t e = walk_shape<NJ, COUNT, ALG>(g, jobs, njobs, total, &s);
+  if (e != cudaSuccess) return e;
+  if (!s.spread && !qctr) return cudaErrorInvalidValue;
   JobTableN<NJ> tab;
   for (int i = 0; i < njobs; ++i) tab.jobs[i] = jobs[i];
-  const long long cap = (long long)g->num_sms * blocks_per_sm;
-  if (!COUNT && hub_share_pays(g, jobs, njobs, total, cap * kBlock)) {
-    int bs = 1;
-    oe = walk_blocks_per_sm<NJ, false, ALG, true>(&bs);
-    if (oe != cudaSuccess) return oe;
-    // one warp's worth of walkers per block: the other warps of each block are free to help
-    const long long want = (total + 31) / 32, cs = (long long)g->num_sms * bs;
-    const int grid = (int)(want < cs ? (want > 0 ? want : 1) : cs);
-    walk_kernel<NJ, false, ALG, true><<<grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, qctr, g->d_err,
-                                                                   g->d_cnt);
-  } else {
-    const long long want = (total + kBlock - 1) / kBlock;
-    const int grid = (int)(want < cap ? (want > 0 ? want : 1) : cap);
-    walk_kernel<NJ, COUNT, ALG><<<grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, qctr, g->d_err,
-                                                             g->d_cnt);
-  }
+  if (s.share)
+    walk_kernel<NJ, false, ALG, true, true><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw,
+                                                                           nullptr, g->d_err, g->d_cnt);
+  else if (s.spread)
+    walk_kernel<NJ, false, ALG, true><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, nullptr,
+                                                                     g->d_err, g->d_cnt);
+  else
+    walk_kernel<NJ, COUNT, ALG><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err,
+                                                               g->d_cnt);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }

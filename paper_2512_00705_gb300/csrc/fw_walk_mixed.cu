@@ -28,12 +28,12 @@ cudaError_t launch_group(int a, const fw_graph* g, const Job* jobs, int njobs, l
   }
 }
 
-template <bool COUNT, bool SHARE = false>
+template <bool COUNT, bool SPREAD = false, bool SHARE = false>
 cudaError_t prime_groups(int* b) {
-  cudaError_t e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_WEIGHTED, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_NODE2VEC, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_METAPATH, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_PAGERANK2, SHARE>(b);
+  cudaError_t e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_WEIGHTED, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_NODE2VEC, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_METAPATH, SPREAD, SHARE>(b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_PAGERANK2, SPREAD, SHARE>(b);
   return e;
 }
 
@@ -44,6 +44,7 @@ cudaError_t prime_walk_mixed_occupancy() {
   cudaError_t e = prime_groups<false>(&b);
   if (e == cudaSuccess) e = prime_groups<true>(&b);
   if (e == cudaSuccess) e = prime_groups<false, true>(&b);
+  if (e == cudaSuccess) e = prime_groups<false, true, true>(&b);
   return e;
 }
 

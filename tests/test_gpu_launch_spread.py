@@ -1,0 +1,54 @@
+"""Launch shapes: few walkers are spread over the resident warps (no queue),
+more walkers than lanes come from the queue; the rows are the same."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2512_00705_gb300 import flexiwalk as fw
+from paper_2512_00705_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+LEN = 3
+
+
+@pytest.fixture(scope="module")
+def walks():
+    g = synth.workload_graph("small")
+    G = fw.Graph(g)
+    lanes = torch.cuda.get_device_properties(0).multi_processor_count * 4 * 256  # 4 resident blocks of 256 threads
+    most = lanes + 33
+    starts = synth.random_starts(g.n, most, seed=5)
+    yield g, G, lanes, starts
+    G.close()
+
+
+@pytest.mark.parametrize("where", ["one", "block", "warps", "warps+1", "half", "lanes-1", "lanes", "lanes+1", "lanes+33"])
+@pytest.mark.parametrize("mode", ["exact", "rvs"])
+def test_rows_do_not_depend_on_the_launch_shape(walks, where, mode):
+    g, G, lanes, starts = walks
+    w = {"one": 1, "block": 31, "warps": lanes // 32, "warps+1": lanes // 32 + 1, "half": lanes // 2 + 7,
+         "lanes-1": lanes - 1, "lanes": lanes, "lanes+1": lanes + 1, "lanes+33": lanes + 33}[where]
+    dev = torch.from_numpy(starts[:w]).cuda()
+    out = G.walk(dev, LEN, "node2vec", p=2.0, q=0.5, mode=mode, seed=9).cpu().numpy()
+    if mode == "exact":
+        ref, _ = oracle.walk(g, starts[:w], LEN, "node2vec", 2.0, 0.5, seed=9)
+    else:  # the counting build takes its walkers from the queue at every size
+        ref = G.walk(dev, LEN, "node2vec", p=2.0, q=0.5, mode=mode, seed=9, flags=fw.FLAG_COUNTERS).cpu().numpy()
+    assert np.array_equal(out, ref)
+    G.check()
+
+
+def test_small_batch_spreads_each_job(walks):
+    g, G, lanes, starts = walks
+    jobs, outs = [], []
+    for j, w in enumerate([1, 63, 700, 5]):
+        dev = torch.from_numpy(starts[:w]).cuda()
+        out = torch.full((w, LEN + 1), -7, dtype=torch.int32, device="cuda")
+        jobs.append(fw.make_job(dev, LEN, "node2vec", out, p=2.0, q=0.5, mode="exact", seed=j))
+        outs.append((w, out, dev))
+    fw.fw_walk_batch(G.handle, jobs)
+    for j, (w, out, _) in enumerate(outs):
+        ref, _ = oracle.walk(g, starts[:w], LEN, "node2vec", 2.0, 0.5, seed=j)
+        assert np.array_equal(out.cpu().numpy(), ref)
