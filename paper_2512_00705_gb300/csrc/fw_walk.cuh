@@ -684,7 +684,8 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       }
     }
     // ------------------------------------------------------------ eRJS trials
-    if (widx >= 0 && plan == PLAN_RJS && pick == -2) {
+    int32_t ent = -2;  // position drawn by eRVS / exact in the row (grouped metapath: label segment); -1: dead end
+    if (widx >= 0 && pick == -2 && plan == PLAN_RJS) {
       Accept acc;
       if (rjs_trials<COUNT, ALG>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
                                  grp)) {
@@ -712,38 +713,24 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     }
     // ------------------------------------------------------------ single-lane eRVS / exact
     if (widx >= 0 && pick == -2 && plan == PLAN_RVS_T) {
+      const bool jump = !(J.flags & FW_FLAG_RVS_NOJUMP);
       if ((FW_ALGO(J) == ALGO_METAPATH) && grp) {
         StepCtx cg = c;
         cg.s = c.ps;
         cg.d = c.pe - c.ps;
-        const int32_t j = rvs_pick<1, COUNT, ALG, true>(g, J, cg, 0, !(J.flags & FW_FLAG_RVS_NOJUMP), lc);
-        pick = -1;
-        if (j >= 0) {  // the grouped record gives the node, its position in the row and its node record
-          int4 a, b;
-          ld_record(g.gerec + 2ll * (cg.s + j), a, b);
-          if (COUNT) lc.bytes += 32;
-          pick = b.z;
-          node = a.x;
-          nxt = make_int4(a.z, a.w, b.x, b.y);
-          nxt_n0 = nxt_n1 = 0;  // metapath plans without weight classes
-          nxt_ok = true;
-        }
+        ent = rvs_pick<1, COUNT, ALG, true>(g, J, cg, 0, jump, lc);
       } else {
-        pick = rvs_pick<1, COUNT, ALG>(g, J, c, 0, !(J.flags & FW_FLAG_RVS_NOJUMP), lc);
-        if (pick >= 0) node = __ldg(g.col + c.s + pick);
+        ent = rvs_pick<1, COUNT, ALG>(g, J, c, 0, jump, lc);
       }
-      h_in = -1.0f;
       if (COUNT) lc.rvs_steps++;
     }
     if (widx >= 0 && pick == -2 && plan == PLAN_EXACT_T) {
       const float u = u01(philox(make_uint4(c.wid, (uint32_t)c.step, 0u, 0u), J.key0, J.key1).x);
-      pick = exact_pick<1, COUNT, ALG>(g, J, c, 0, u, lc);
-      if (pick >= 0) node = __ldg(g.col + c.s + pick);
-      h_in = -1.0f;
+      ent = exact_pick<1, COUNT, ALG>(g, J, c, 0, u, lc);
       if (COUNT) lc.exact_steps++;
     }
     // ------------------------------------------------------------ warp hand-off
-    unsigned wm = __ballot_sync(kFull, widx >= 0 && pick == -2 && (plan == PLAN_RVS_W || plan == PLAN_EXACT_W));
+    unsigned wm = __ballot_sync(kFull, widx >= 0 && pick == -2 && ent == -2 && (plan == PLAN_RVS_W || plan == PLAN_EXACT_W));
     while (wm != 0u) {
       const int src = __ffs(wm) - 1;
       wm &= wm - 1u;
@@ -786,29 +773,33 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       } else {
         k = rvs_pick<32, COUNT, ALG>(g, JW, w, lane, !(JW.flags & FW_FLAG_RVS_NOJUMP), lc);
       }
-      if (lane == src && ALG == ALGO_METAPATH && wg) {
-        pick = -1;
-        if (k >= 0) {  // grouped position -> node, position in the row, node record
-          int4 a, b;
-          ld_record(g.gerec + 2ll * (w.ps + k), a, b);
-          if (COUNT) lc.bytes += 32;
-          pick = b.z;
-          node = a.x;
-          nxt = make_int4(a.z, a.w, b.x, b.y);
-          nxt_n0 = nxt_n1 = 0;  // metapath plans without weight classes
-          nxt_ok = true;
-        }
-        h_in = -1.0f;
-        if (COUNT) lc.rvs_steps++;
-      } else if (lane == src) {
-        pick = k;
-        if (k >= 0) node = __ldg(g.col + w.s + k);
-        h_in = -1.0f;
+      if (lane == src) {
+        ent = k;
         if (COUNT) {
           if (pl == PLAN_EXACT_W) lc.exact_steps++;
           else lc.rvs_steps++;
         }
       }
+    }
+    // ------------------------------------------------------------ entry drawn -> node and its record
+    // One 32-byte edge record gives the node, its node record and h of the
+    // edge, as an accepted trial does: the column, the node record and the
+    // search for v' of the next node2vec plan were up to six more dependent
+    // accesses per eRVS hop (GB300, s22 p = 1/4, q = 4: 55.9 -> 49.4 ms).
+    if (ent >= 0) {
+      const bool in_group = ALG == ALGO_METAPATH && grp;
+      int4 a, b;
+      ld_record((in_group ? g.gerec + 2ll * (c.ps + ent) : g.erec + 2ll * (c.s + ent)), a, b);
+      if (COUNT) lc.bytes += 32;
+      pick = in_group ? b.z : ent;
+      node = a.x;
+      nxt = make_int4(a.z, a.w, b.x, b.y);
+      nxt_n0 = in_group ? 0 : (int32_t)((uint32_t)b.z >> 8);  // grouped metapath plans without weight classes
+      nxt_n1 = in_group ? 0 : b.w;
+      nxt_ok = true;
+      h_in = J.weighted ? __int_as_float(a.y) : 1.0f;
+    } else if (ent == -1) {
+      pick = -1;
     }
     // ------------------------------------------------------------ commit
     if (widx >= 0 && pick != -2) {
