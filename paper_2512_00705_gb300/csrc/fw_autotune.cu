@@ -69,7 +69,9 @@ __global__ void profile_rjs_kernel(DevGraph g, Job J, int32_t count, int32_t str
       const float B = __fmul_rn(second ? J.wmax1 : (J.algo == ALGO_PAGERANK2 && c.vp >= 0 ? c.w1 : 1.0f), hm);
       Accept acc;
       LaneCounters lc;
-      found = rjs_trials<false>(g, J, c, B, false, 0.0f, -1, 0.0f, j, 1, acc, lc) ? 1u : 0u;
+      float beta = 0.0f, beta2 = 0.0f;
+      int32_t pos = -1;
+      found = rjs_trials<false>(g, J, c, B, false, beta, pos, 0.0f, j, 1, acc, lc, false, beta2, false) ? 1u : 0u;
       done = 1;
     }
   }

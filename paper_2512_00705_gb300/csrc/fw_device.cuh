@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "../../include/flexiwalk.h"
+
 namespace fw {
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -559,21 +561,33 @@ struct Accept {
 // (1 - 1/q) h(x) [x in N(v')] from the second: w~(x) in total.  The envelope
 // mass is (1/q) d + (1 - 1/q) d' < d, so fewer trials than the one-envelope
 // bound max(1, 1/q) h_MAX = h_MAX (B = h_MAX is passed in this case).
-template <bool COUNT, int ALG = -1>
+//
+// Lane eRVS (rvs: a reservoir step over a row that the walker's own lane
+// scans, rvs_pick<1>): "trial" t is the scan's position t, so such a lane
+// moves in step with its warp's eRJS lanes instead of stalling them for the
+// whole row: its record load and membership test are the trials' own, its
+// Philox block is (wid, hop, 6, 0) for position 0 and (wid, hop, 2, t)
+// after it, and only the outcome differs -- the key or the jump.  The scan's
+// state lives in `beta` (weight left before the next crossing), `beta2`
+// (best key, the reference of the jumps) and `pos_ret` (its position, -1:
+// none); true once the row is done.
+template <bool COUNT, int ALG = -1, bool LANE_RVS = false>
 __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, const StepCtx& c, float B, bool split,
-                                           float beta, int32_t pos_ret, float h_ret, int32_t t0, int32_t nt,
-                                           Accept& acc, LaneCounters& lc, bool csplit = false, float beta2 = 0.0f,
-                                           bool grp = false) {
+                                           float& beta, int32_t& pos_ret, float h_ret, int32_t t0, int32_t nt,
+                                           Accept& acc, LaneCounters& lc, bool csplit, float& beta2, bool grp,
+                                           bool lane_rvs = false) {
+  const bool rvs = LANE_RVS && lane_rvs;
   const uint32_t d = (uint32_t)c.d;
   const uint8_t want = (FW_ALGO(J) == ALGO_METAPATH) ? J.schema[c.step % J.schema_len] : 0;
   const bool second = (FW_ALGO(J) == ALGO_NODE2VEC) && c.vp >= 0 && J.second_order;
+  const bool pr2 = (FW_ALGO(J) == ALGO_PAGERANK2) && c.vp >= 0;
   uint32_t probes = 0;
   bool found = false;
   for (int32_t t = t0; t < t0 + nt; ++t) {
-    const uint4 x = philox(make_uint4(c.wid, (uint32_t)c.step, 1u, (uint32_t)t), J.key0, J.key1);
-    if (COUNT) lc.rjs_trials++;
+    const uint4 x = philox(make_uint4(c.wid, (uint32_t)c.step, rvs ? (t == 0 ? 6u : 2u) : 1u, (uint32_t)t), J.key0, J.key1);
+    if (COUNT && !rvs) lc.rjs_trials++;
     const float ucomp = u01(x.w);
-    if (beta > 0.0f && ucomp < beta) {
+    if (!rvs && beta > 0.0f && ucomp < beta) {
       if (FW_ALGO(J) == ALGO_PAGERANK2) {
         uint32_t pb = 0;
         acc.node = common_pick(g, J, c, __fmul_rn(u01(x.z), h_ret), acc.k, acc.h, pb);
@@ -588,7 +602,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
       break;
     }
     int4 a, b;  // {col, h, target row start, target degree}, {target h_MAX, target h_SUM, label, 0}
-    if ((FW_ALGO(J) == ALGO_METAPATH) && grp) {
+    if ((FW_ALGO(J) == ALGO_METAPATH) && grp && !rvs) {
       // metapath inside the required label's segment [c.ps, c.pe) of the grouped
       // arrays, every entry of w = 1, ordered by weight class: slot t of the
       // class envelope (class_slots) proposes an entry of class c in proportion
@@ -642,7 +656,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
       }
       continue;
     }
-    if ((FW_ALGO(J) == ALGO_NODE2VEC) && csplit && ucomp < beta2) {
+    if ((FW_ALGO(J) == ALGO_NODE2VEC) && csplit && ucomp < beta2) {  // never set for lane eRVS
       // component 2: X uniform over N(v'), accepted iff X in N(v) and U h_MAX < h(v, X)
       uint32_t k2;
       if (!lemire_index(x.x, x.y, (uint32_t)(c.pe - c.ps), k2)) continue;
@@ -671,7 +685,10 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
     uint32_t ku;
     float Bc = B;  // bound of the proposed entry's class
     const int4* er;
-    if (c.n0 >= 0) {
+    if (rvs) {
+      ku = (uint32_t)t;
+      er = (FW_ALGO(J) == ALGO_METAPATH) && grp ? g.gerec + 2ll * (c.ps + t) : g.erec + 2ll * (c.s + t);
+    } else if (c.n0 >= 0) {
       // three weight classes of bounds B, B / 2, B / 4 (h <= h_MAX / 2^c in class c): slot t of
       // 4 n0 + 2 n1 + n2 proposes an entry of class c in proportion to its bound
       const uint32_t n0 = (uint32_t)c.n0, n1 = (uint32_t)c.n1;
@@ -697,6 +714,48 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
     const int32_t u = a.x;
     const float hk = J.weighted ? __int_as_float(a.y) : 1.0f;
     const float UB = __fmul_rn(u01(x.z), Bc);
+    // the transition weight depends on u in N(v') and the trial's squeeze tests leave it open
+    bool adj = false;
+    if (second ? (u != c.vp && (rvs ? J.need_member != 0
+                                    : !csplit && UB < __fmul_rn(J.whi1, hk) && UB >= __fmul_rn(J.wlo1, hk)))
+               : (pr2 && (rvs || (!split && UB < __fmul_rn(c.w1, hk) && UB >= __fmul_rn(c.w2, hk))))) {
+      uint32_t pb = 0;
+      adj = prev_contains(g, J, c, u, pb);
+      probes += pb;
+    }
+    if (rvs) {
+      float wt;
+      if (second) wt = __fmul_rn(u == c.vp ? J.inv_p : (adj || !J.need_member ? 1.0f : J.inv_q), hk);
+      else if (FW_ALGO(J) == ALGO_METAPATH) wt = grp || (uint8_t)b.z == want ? hk : 0.0f;
+      else wt = pr2 ? __fmul_rn(adj ? c.w1 : c.w2, hk) : hk;
+      if (COUNT) lc.rvs_items++;
+      if (t == 0) {
+        beta2 = -CUDART_INF_F;
+        beta = 0.0f;  // no positive weight so far: the first positive item crosses
+        pos_ret = -1;
+      }
+      const bool jump = !(J.flags & FW_FLAG_RVS_NOJUMP);
+      if (wt > 0.0f) {
+        const bool cross = jump && t > 0 && (beta -= wt) <= 0.0f;
+        if (cross || !jump || t == 0) {
+          // key; after the first position of a jumping scan conditioned on beating the best one
+          const float K = cross ? log1pf(expm1f(beta2 * wt) * u01_open(x.y)) / wt : logf(u01_open(x.x)) / wt;
+          if (COUNT) lc.rvs_keys++;
+          if (cross || K >= beta2) {
+            beta2 = K;
+            pos_ret = t;
+          }
+          if (jump) beta = (beta2 < 0.0f) ? logf(u01_open(t == 0 ? x.w : x.z)) / beta2 : CUDART_INF_F;
+        }
+      }
+      const int32_t len = (FW_ALGO(J) == ALGO_METAPATH) && grp ? c.pe - c.ps : c.d;
+      if (t + 1 >= len) {
+        if (beta2 == -CUDART_INF_F) pos_ret = -1;
+        found = true;
+        break;
+      }
+      continue;
+    }
     bool accept;
     if (second) {
       if (u == c.vp) {
@@ -704,31 +763,13 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
         accept = UB < __fmul_rn(J.inv_p, hk);
       } else if (csplit) {
         accept = UB < hk;                       // component 1: (1/q) h against (1/q) h_MAX
-      } else if (UB >= __fmul_rn(J.whi1, hk)) {
-        accept = false;                         // squeeze: above the largest possible weight
-      } else if (UB < __fmul_rn(J.wlo1, hk)) {
-        accept = true;                          // squeeze: below the smallest possible weight
-      } else {
-        uint32_t pb = 0;
-        const bool adj = prev_contains(g, J, c, u, pb);
-        probes += pb;
+      } else {                                  // adj is false above the largest and below the smallest weight
         accept = UB < __fmul_rn(adj ? 1.0f : J.inv_q, hk);
       }
     } else if (FW_ALGO(J) == ALGO_METAPATH) {
       accept = ((uint8_t)b.z == want) && (UB < hk);
-    } else if (FW_ALGO(J) == ALGO_PAGERANK2 && c.vp >= 0 && split) {
-      accept = UB < __fmul_rn(c.w2, hk);        // the w2 part; C is proposed by the split
-    } else if (FW_ALGO(J) == ALGO_PAGERANK2 && c.vp >= 0) {
-      if (UB >= __fmul_rn(c.w1, hk)) {
-        accept = false;                         // squeeze: above the larger weight
-      } else if (UB < __fmul_rn(c.w2, hk)) {
-        accept = true;                          // squeeze: below the smaller weight
-      } else {
-        uint32_t pb = 0;
-        const bool adj = prev_contains(g, J, c, u, pb);
-        probes += pb;
-        accept = UB < __fmul_rn(adj ? c.w1 : c.w2, hk);
-      }
+    } else if (pr2) {
+      accept = UB < __fmul_rn(adj ? c.w1 : c.w2, hk);
     } else {
       accept = UB < hk;
     }

@@ -420,6 +420,16 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
   static_assert(ALG >= 0 && ALG < kAlgos, "the walk loop is compiled for one algorithm");
+  // Short eRVS rows in step with the trials (see rjs_trials): node2vec only.
+  // There a row's positions each wait for a membership test, and a warp paid
+  // for them whenever one of its lanes had such a step: GB300, one walker per
+  // node x 80 hops, whole rows at once -> one position per trial: s20 p = 4,
+  // q = 1/4 7.60 -> 6.71 ms, s22 p = 1/4, q = 4 49.5 -> 44.9 ms.  First-order
+  // rows are one or two sectors of h that stay in L1 (weighted s22 7.46 ms at
+  // once, 7.64 in step; metapath 1.32 and 1.40 ms); so are launches with few
+  // lanes per warp (5,003 walkers 379 and 538 us); second-order PageRank
+  // seldom has such rows and loses the registers (8.46 and 8.80 ms).
+  constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC;
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -683,20 +693,26 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         }
       }
     }
-    // ------------------------------------------------------------ eRJS trials
+    // ------------------------------------------------------------ eRJS trials and lane eRVS positions
     int32_t ent = -2;  // position drawn by eRVS / exact in the row (grouped metapath: label segment); -1: dead end
-    if (widx >= 0 && pick == -2 && plan == PLAN_RJS) {
+    if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || (kLaneRvs && plan == PLAN_RVS_T))) {
+      const bool rvs = plan == PLAN_RVS_T;
       Accept acc;
-      if (rjs_trials<COUNT, ALG>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
-                                 grp)) {
-        pick = acc.k;
-        node = acc.node;
-        h_in = acc.h;
-        nxt = acc.rec;
-        nxt_n0 = acc.rec_n0;
-        nxt_n1 = acc.rec_n1;
-        nxt_ok = acc.rec_ok;
-        if (COUNT) lc.rjs_steps++;
+      if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
+                                 grp, rvs)) {
+        if (rvs) {
+          ent = pos_ret;
+          if (COUNT) lc.rvs_steps++;
+        } else {
+          pick = acc.k;
+          node = acc.node;
+          h_in = acc.h;
+          nxt = acc.rec;
+          nxt_n0 = acc.rec_n0;
+          nxt_n1 = acc.rec_n1;
+          nxt_ok = acc.rec_ok;
+          if (COUNT) lc.rjs_steps++;
+        }
       } else {
         trials += J.rjs_batch;
         // trial budget: the cap, or (default) as many trials as the eRVS scan
@@ -705,14 +721,16 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         const int32_t dd = grp ? c.pe - c.ps : c.d;  // entries the eRVS hand-off would scan
         const int32_t cap =
             J.fixed_cap ? J.rjs_cap : max(J.rjs_cap, (int32_t)fminf(ceilf(J.budget * (float)dd / J.ratio), 1.0e9f));
-        if (trials >= cap) {
+        if (!rvs && trials >= cap) {
           plan = (dd <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W;
+          trials = 0;
+          split = csplit = false;
           if (COUNT) lc.handoffs++;
         }
       }
     }
     // ------------------------------------------------------------ single-lane eRVS / exact
-    if (widx >= 0 && pick == -2 && plan == PLAN_RVS_T) {
+    if (!kLaneRvs && widx >= 0 && pick == -2 && plan == PLAN_RVS_T) {
       const bool jump = !(J.flags & FW_FLAG_RVS_NOJUMP);
       if ((FW_ALGO(J) == ALGO_METAPATH) && grp) {
         StepCtx cg = c;

@@ -52,3 +52,25 @@ def test_small_batch_spreads_each_job(walks):
     for j, (w, out, _) in enumerate(outs):
         ref, _ = oracle.walk(g, starts[:w], LEN, "node2vec", 2.0, 0.5, seed=j)
         assert np.array_equal(out.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("p,q", [(2.0, 0.5), (0.25, 4.0), (1.0, 4.0)])
+@pytest.mark.parametrize("mode,flags,shape", [("rvs", 0, {}), ("rvs", 0, {"lane_max_degree": 64, "rjs_batch": 3}),
+                                              ("rvs", fw.FLAG_RVS_NOJUMP, {"lane_max_degree": 33}),
+                                              ("rvs", fw.FLAG_UNWEIGHTED, {"lane_max_degree": 1}),
+                                              ("auto", 0, {"cost_ratio": 8.0}),
+                                              ("rjs", 0, {"rjs_cap": 1, "lane_max_degree": 40})])
+@pytest.mark.parametrize("quantized", [False, True])
+def test_lane_scans_in_step_with_trials_equal_whole_lane_scans(p, q, mode, flags, shape, quantized):
+    """node2vec's short eRVS rows: scanned one position per trial round by the
+    queued kernel (which the counting build is), at once by the spread one."""
+    g = synth.workload_graph("small")
+    G = fw.Graph(g)
+    if quantized:
+        G.quantize_weights()
+    starts = torch.arange(g.n, dtype=torch.int32, device="cuda")
+    a = G.walk(starts, 20, "node2vec", p=p, q=q, mode=mode, seed=3, flags=flags, **shape)
+    b = G.walk(starts, 20, "node2vec", p=p, q=q, mode=mode, seed=3, flags=flags | fw.FLAG_COUNTERS, **shape)
+    assert torch.equal(a, b)
+    assert G.counters()["rvs_steps"] > 0
+    G.close()
