@@ -517,6 +517,12 @@ __device__ __forceinline__ bool lemire_index(uint32_t x0, uint32_t x1, uint32_t 
   return true;
 }
 
+// What a lane of rjs_trials does: eRJS trials, or an eRVS row of its own
+// scanned one position per trial -- with jumps (rvs_pick<1>), or every
+// position keyed (a warp scan of at most 32 positions is its phase 1 only).
+enum : int32_t { kLaneNone = 0, kLaneJump = 1, kLaneKeyed = 2 };
+constexpr int32_t kLaneKeyedMax = 32;
+
 // One eRJS acceptance: the neighbour position, the node, its effective
 // property weight, and the target's node record (rec_ok = 0: unknown).
 struct Accept {
@@ -575,8 +581,9 @@ template <bool COUNT, int ALG = -1, bool LANE_RVS = false>
 __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, const StepCtx& c, float B, bool split,
                                            float& beta, int32_t& pos_ret, float h_ret, int32_t t0, int32_t nt,
                                            Accept& acc, LaneCounters& lc, bool csplit, float& beta2, bool grp,
-                                           bool lane_rvs = false) {
-  const bool rvs = LANE_RVS && lane_rvs;
+                                           int32_t lane_rvs = kLaneNone) {
+  const bool rvs = LANE_RVS && lane_rvs != kLaneNone;
+  const bool keyed = LANE_RVS && lane_rvs == kLaneKeyed;
   const uint32_t d = (uint32_t)c.d;
   const uint8_t want = (FW_ALGO(J) == ALGO_METAPATH) ? J.schema[c.step % J.schema_len] : 0;
   const bool second = (FW_ALGO(J) == ALGO_NODE2VEC) && c.vp >= 0 && J.second_order;
@@ -584,7 +591,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
   uint32_t probes = 0;
   bool found = false;
   for (int32_t t = t0; t < t0 + nt; ++t) {
-    const uint4 x = philox(make_uint4(c.wid, (uint32_t)c.step, rvs ? (t == 0 ? 6u : 2u) : 1u, (uint32_t)t), J.key0, J.key1);
+    const uint4 x = philox(make_uint4(c.wid, (uint32_t)c.step, rvs ? (t == 0 || keyed ? 6u : 2u) : 1u, (uint32_t)t), J.key0, J.key1);
     if (COUNT && !rvs) lc.rjs_trials++;
     const float ucomp = u01(x.w);
     if (!rvs && beta > 0.0f && ucomp < beta) {
@@ -734,7 +741,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
         beta = 0.0f;  // no positive weight so far: the first positive item crosses
         pos_ret = -1;
       }
-      const bool jump = !(J.flags & FW_FLAG_RVS_NOJUMP);
+      const bool jump = !keyed && !(J.flags & FW_FLAG_RVS_NOJUMP);
       if (wt > 0.0f) {
         const bool cross = jump && t > 0 && (beta -= wt) <= 0.0f;
         if (cross || !jump || t == 0) {

@@ -424,7 +424,9 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   // There a row's positions each wait for a membership test, and a warp paid
   // for them whenever one of its lanes had such a step: GB300, one walker per
   // node x 80 hops, whole rows at once -> one position per trial: s20 p = 4,
-  // q = 1/4 7.60 -> 6.71 ms, s22 p = 1/4, q = 4 49.5 -> 44.9 ms.  First-order
+  // q = 1/4 7.60 -> 6.71 ms, s22 p = 1/4, q = 4 49.5 -> 44.9 ms; with warp
+  // rows of up to 32 entries as well, each of which held all 32 lanes, 6.28
+  // and 39.3 ms.  First-order
   // rows are one or two sectors of h that stay in L1 (weighted s22 7.46 ms at
   // once, 7.64 in step; metapath 1.32 and 1.40 ms); so are launches with few
   // lanes per warp (5,003 walkers 379 and 538 us); second-order PageRank
@@ -695,11 +697,14 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     }
     // ------------------------------------------------------------ eRJS trials and lane eRVS positions
     int32_t ent = -2;  // position drawn by eRVS / exact in the row (grouped metapath: label segment); -1: dead end
-    if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || (kLaneRvs && plan == PLAN_RVS_T))) {
-      const bool rvs = plan == PLAN_RVS_T;
+    const int32_t lane_rvs = !kLaneRvs ? kLaneNone
+                             : plan == PLAN_RVS_T ? kLaneJump
+                             : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
+    if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
+      const bool rvs = lane_rvs != kLaneNone;
       Accept acc;
       if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
-                                 grp, rvs)) {
+                                 grp, lane_rvs)) {
         if (rvs) {
           ent = pos_ret;
           if (COUNT) lc.rvs_steps++;
@@ -748,7 +753,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       if (COUNT) lc.exact_steps++;
     }
     // ------------------------------------------------------------ warp hand-off
-    unsigned wm = __ballot_sync(kFull, widx >= 0 && pick == -2 && ent == -2 && (plan == PLAN_RVS_W || plan == PLAN_EXACT_W));
+    unsigned wm = __ballot_sync(kFull, widx >= 0 && pick == -2 && ent == -2 && lane_rvs == kLaneNone && (plan == PLAN_RVS_W || plan == PLAN_EXACT_W));
     while (wm != 0u) {
       const int src = __ffs(wm) - 1;
       wm &= wm - 1u;

@@ -57,6 +57,7 @@ def test_small_batch_spreads_each_job(walks):
 @pytest.mark.parametrize("p,q", [(2.0, 0.5), (0.25, 4.0), (1.0, 4.0)])
 @pytest.mark.parametrize("mode,flags,shape", [("rvs", 0, {}), ("rvs", 0, {"lane_max_degree": 64, "rjs_batch": 3}),
                                               ("rvs", fw.FLAG_RVS_NOJUMP, {"lane_max_degree": 33}),
+                                              ("rvs", 0, {"lane_max_degree": 1}), ("rvs", fw.FLAG_RVS_NOJUMP, {}),
                                               ("rvs", fw.FLAG_UNWEIGHTED, {"lane_max_degree": 1}),
                                               ("auto", 0, {"cost_ratio": 8.0}),
                                               ("rjs", 0, {"rjs_cap": 1, "lane_max_degree": 40})])
