@@ -49,6 +49,41 @@ DevGraph dev_graph(const fw_graph* g) {
   return d;
 }
 
+// Queue counters come from a pool of the graph's own that keeps up to
+// kCounterPoolKeep bytes: the device's default pool gives its memory back at
+// every synchronisation, so that the first walk after one paid about 0.2 ms
+// for mapping it again.
+static constexpr unsigned long long kCounterPoolKeep = 4ull << 20;
+
+static void create_counter_pool(fw_graph* g) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = g->device;
+  if (cudaMemPoolCreate(&g->counter_pool, &props) != cudaSuccess) {
+    g->counter_pool = nullptr;
+    cudaGetLastError();  // not sticky; the default pool serves
+    return;
+  }
+  unsigned long long keep = kCounterPoolKeep;
+  cudaMemPoolSetAttribute(g->counter_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+static cudaError_t alloc_scratch(const fw_graph* g, size_t bytes, unsigned long long** out, cudaStream_t st) {
+  void** p = reinterpret_cast<void**>(out);
+  return g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
+cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t st) {
+  const size_t bytes = sizeof(unsigned long long) * (size_t)count;
+  cudaError_t e = alloc_scratch(g, bytes, out, st);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(*out, 0, bytes, st);
+  if (e != cudaSuccess) cudaFreeAsync(*out, st);
+  return e;
+}
+
 static float recip_f32(float p) { return (float)(1.0 / (double)p); }
 
 fw_status make_job(const fw_graph* g, int32_t algo, const fw_params* params, uint64_t seed, Job* job) {
@@ -124,7 +159,7 @@ fw_status make_job(const fw_graph* g, int32_t algo, const fw_params* params, uin
 // The label-grouped view of the rows (metapath's fast modes sample inside
 // the required label's segment).  Needs the per-label statistics.  If the
 // device has no room for it, metapath walks keep the full-row path.
-static fw_status build_label_groups(fw_graph* g, cudaStream_t st) {
+static fw_status build_label_groups(fw_graph* g, const RowLists& rows, cudaStream_t st) {
   const size_t lrec_bytes = 2 * sizeof(int4) * kLabelStats * ((size_t)g->n + 1);
   const size_t gerec_bytes = 2 * sizeof(int4) * (size_t)g->e, gh_bytes = sizeof(float) * (size_t)g->e;
   if (!g->d_lrec) {
@@ -147,7 +182,7 @@ static fw_status build_label_groups(fw_graph* g, cudaStream_t st) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, st);
-  cudaError_t le = launch_label_group(g->d_off, g->d_col, g->d_h, g->d_lab, g->d_nrec, g->d_lstat, g->n, g->d_lrec,
+  cudaError_t le = launch_label_group(g->d_off, g->d_col, g->d_h, g->d_lab, g->d_nrec, g->d_lstat, g->n, rows, g->d_lrec,
                                       g->d_gerec, g->d_gh, g->num_sms, st);
   cudaEventRecord(e1, st);
   cudaError_t se = cudaStreamSynchronize(st);
@@ -167,6 +202,7 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   int* d_maxdeg = reinterpret_cast<int*>(g->d_err) + 8;
   unsigned* d_asym = g->d_err + 12;
   unsigned* d_lbad = g->d_err + 13;
+  unsigned long long* d_sides = reinterpret_cast<unsigned long long*>(g->d_err) + 1;
   const bool want_labels = g->d_lab != nullptr && !g->lstat_bad;
   const bool build_bloom = g->d_bloom == nullptr;  // depends on the structure only: built once
   if (build_bloom) {
@@ -197,85 +233,64 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
     cudaError_t pe = prime_preprocess_kernels();
     if (pe != cudaSuccess) return cuda_error(pe, "load preprocessing kernels");
   }
+  unsigned long long* scratch = nullptr;  // the row lists
+  {
+    cudaError_t ae = alloc_scratch(g, sizeof(int32_t) * row_list_words(e), &scratch, st);
+    if (ae != cudaSuccess) return cuda_error(ae, "row lists");
+  }
+  const RowLists rows = row_lists(reinterpret_cast<int32_t*>(scratch), e);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  cudaError_t le = cudaMemsetAsync(d_maxdeg, 0, sizeof(int), st);
-  if (le == cudaSuccess) le = cudaMemsetAsync(d_asym, 0, 2 * sizeof(unsigned), st);
+  // one memset over the words these kernels use: sides (2..5), max degree (8), asymmetry (12), bad label (13)
+  cudaError_t le = cudaMemsetAsync(g->d_err + 2, 0, 12 * sizeof(unsigned), st);
+  if (le == cudaSuccess) le = cudaMemsetAsync(rows.counts, 0, 2 * sizeof(int), st);
   cudaEventRecord(e0, st);
   if (le == cudaSuccess)
-    le = launch_node_stats(g->d_off, g->d_h, n, g->d_hmax, g->d_hsum, g->d_nrec, d_maxdeg, g->num_sms, st);
-  if (le == cudaSuccess) le = launch_edge_records(g->d_col, g->d_h, g->d_lab, g->d_nrec, e, g->d_erec, g->num_sms, st);
-  if (le == cudaSuccess && g->d_cerec)
-    le = launch_class_group(g->d_off, g->d_h, g->d_nrec, g->d_erec, n, g->d_cerec, g->num_sms, st);
-  if (le == cudaSuccess) le = launch_symmetry(g->d_off, g->d_col, g->d_h, n, e, d_asym, g->num_sms, st);
+    le = launch_node_stats(g->d_off, g->d_h, n, g->d_hmax, g->d_hsum, g->d_nrec, d_maxdeg, rows, g->num_sms, st);
+  if (le == cudaSuccess && e > 0)
+    le = launch_edge_records(g->d_off, g->d_col, g->d_h, g->d_lab, g->d_nrec, n, rows, g->d_erec, g->d_cerec,
+                             g->num_sms, st);
+  if (le == cudaSuccess && e > 0)
+    le = launch_symmetry(g->d_off, g->d_col, g->d_h, n, rows, d_asym, d_sides, g->num_sms, st);
   if (le == cudaSuccess && build_bloom)
-    le = launch_bloom(g->d_off, g->d_col, n, e, g->d_bloom, g->d_mtab, g->num_sms, st);
+    le = launch_bloom(g->d_off, g->d_col, n, e, rows, g->d_bloom, g->d_mtab, g->num_sms, st);
   if (le == cudaSuccess && want_labels)
-    le = launch_label_stats(g->d_off, g->d_h, g->d_lab, n, g->d_lstat, d_lbad, g->num_sms, st);
+    le = launch_label_stats(g->d_off, g->d_h, g->d_lab, n, rows, g->d_lstat, d_lbad, g->num_sms, st);
   cudaEventRecord(e1, st);
-  int maxdeg = 0;
-  unsigned flags[2] = {1, 0};
-  cudaError_t ce = cudaMemcpyAsync(&maxdeg, d_maxdeg, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (ce == cudaSuccess) ce = cudaMemcpyAsync(flags, d_asym, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+  unsigned words[16] = {};
+  cudaError_t ce = cudaMemcpyAsync(words, g->d_err, sizeof(words), cudaMemcpyDeviceToHost, st);
   cudaError_t se = cudaStreamSynchronize(st);
   float ms = 0.0f;
   cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (le != cudaSuccess) return cuda_error(le, "preprocessing kernels");
-  if (ce != cudaSuccess) return cuda_error(ce, "read preprocessing results");
-  if (se != cudaSuccess) return cuda_error(se, "sync after preprocessing");
+  fw_status fs = FW_OK;
+  if (le != cudaSuccess) fs = cuda_error(le, "preprocessing kernels");
+  else if (ce != cudaSuccess) fs = cuda_error(ce, "read preprocessing results");
+  else if (se != cudaSuccess) fs = cuda_error(se, "sync after preprocessing");
+  if (fs != FW_OK) {
+    cudaFreeAsync(scratch, st);
+    return fs;
+  }
+  const int maxdeg = (int)words[8];
   g->max_degree = maxdeg;
-  g->sym = flags[0] == 0 ? 1 : 0;
+  g->sym = words[12] == 0 && words[2] == words[4] && words[3] == words[5] ? 1 : 0;
   if (g->d_cerec && maxdeg >= (1 << 24)) {  // edge records carry class counts in 24 bits
     cudaFree(g->d_cerec);
     g->d_cerec = nullptr;
     g->bytes -= 2 * sizeof(int4) * (size_t)e;
   }
-  if (want_labels && flags[1] != 0) {  // a label >= kLabelStats: per-label statistics unused
+  if (want_labels && words[13] != 0) {  // a label >= kLabelStats: per-label statistics unused
     cudaFree(g->d_lstat);
     g->d_lstat = nullptr;
     g->bytes -= sizeof(float2) * kLabelStats * ((size_t)n + 1);
     g->lstat_bad = true;
   }
   g->preprocess_ms += ms;
-  if (g->d_lstat && e > 0) {
-    fw_status gs = build_label_groups(g, st);
-    if (gs != FW_OK) return gs;
-  }
-  return FW_OK;
-}
-
-// Queue counters come from a pool of the graph's own that keeps up to
-// kCounterPoolKeep bytes: the device's default pool gives its memory back at
-// every synchronisation, so that the first walk after one paid about 0.2 ms
-// for mapping it again.
-static constexpr unsigned long long kCounterPoolKeep = 4ull << 20;
-
-static void create_counter_pool(fw_graph* g) {
-  cudaMemPoolProps props = {};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.handleTypes = cudaMemHandleTypeNone;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = g->device;
-  if (cudaMemPoolCreate(&g->counter_pool, &props) != cudaSuccess) {
-    g->counter_pool = nullptr;
-    cudaGetLastError();  // not sticky; the default pool serves
-    return;
-  }
-  unsigned long long keep = kCounterPoolKeep;
-  cudaMemPoolSetAttribute(g->counter_pool, cudaMemPoolAttrReleaseThreshold, &keep);
-}
-
-cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t st) {
-  const size_t bytes = sizeof(unsigned long long) * (size_t)count;
-  void** p = reinterpret_cast<void**>(out);
-  cudaError_t e = g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(*out, 0, bytes, st);
-  if (e != cudaSuccess) cudaFreeAsync(*out, st);
-  return e;
+  if (g->d_lstat && e > 0) fs = build_label_groups(g, rows, st);
+  cudaFreeAsync(scratch, st);
+  return fs;
 }
 
 static fw_status with_qctr(const fw_graph* g, const Job* jobs, long long total, bool count, cudaStream_t st) {
@@ -438,7 +453,7 @@ extern "C" fw_status fw_graph_create(const int32_t* offsets, const int32_t* cols
     FW_TRY(cudaMemcpyAsync(&bits, g->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st), "read check");
     FW_TRY(cudaStreamSynchronize(st), "sync");
     if (bits == 0) {
-      FW_TRY(launch_check_rows(g->d_off, g->d_col, g->d_h, n, g->d_err, g->num_sms, st), "check rows");
+      FW_TRY(launch_check_rows(g->d_off, g->d_col, g->d_h, n, e, g->d_err, g->num_sms, st), "check rows");
       FW_TRY(cudaMemcpyAsync(&bits, g->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st), "read check");
       FW_TRY(cudaStreamSynchronize(st), "sync");
     }

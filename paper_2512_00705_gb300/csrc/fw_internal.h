@@ -103,31 +103,44 @@ constexpr int kQueueCounters = fw::kAlgos;  // counters a multi-job launch needs
 cudaError_t prime_walk_occupancy();
 cudaError_t prime_walk_mixed_occupancy();
 
+// Rows by length, for the kernels of fw_preprocess.cu: up to kWarpRow entries
+// a warp each, up to kBlockRow (`mid`) a block of 8 warps, the rest (`big`) a
+// block of 32.  counts: rows in mid and in big.
+constexpr int32_t kWarpRow = 256, kBlockRow = 2048;
+struct RowLists {
+  int32_t *mid, *big;
+  int* counts;
+};
+size_t row_list_words(long long e);                      // int32 words of scratch the lists need
+RowLists row_lists(int32_t* scratch, long long e);       // lay them out (the counts come first)
+
+// Also fills `rows` (counts zeroed before).
 cudaError_t launch_node_stats(const int32_t* off, const float* h, int32_t n, float* hmax, float* hsum, int4* nrec,
-                              int* maxdeg, int num_sms, cudaStream_t stream);
-cudaError_t launch_edge_records(const int32_t* col, const float* h, const uint8_t* lab, const int4* nrec, long long e,
-                                int4* erec, int num_sms, cudaStream_t stream);
-cudaError_t launch_label_stats(const int32_t* off, const float* h, const uint8_t* lab, int32_t n, float2* out,
-                               unsigned* bad, int num_sms, cudaStream_t stream);
-cudaError_t launch_class_group(const int32_t* off, const float* h, const int4* nrec, const int4* erec, int32_t n,
-                               int4* cerec, int num_sms, cudaStream_t stream);
+                              int* maxdeg, const RowLists& rows, int num_sms, cudaStream_t stream);
+cudaError_t launch_edge_records(const int32_t* off, const int32_t* col, const float* h, const uint8_t* lab,
+                                const int4* nrec, int32_t n, const RowLists& rows, int4* erec, int4* cerec,
+                                int num_sms, cudaStream_t stream);  // cerec may be nullptr
+cudaError_t launch_label_stats(const int32_t* off, const float* h, const uint8_t* lab, int32_t n,
+                               const RowLists& rows, float2* out, unsigned* bad, int num_sms, cudaStream_t stream);
 cudaError_t launch_label_group(const int32_t* off, const int32_t* col, const float* h, const uint8_t* lab,
-                               const int4* nrec, const float2* lstat, int32_t n, int4* lrec, int4* gerec, float* gh,
-                               int num_sms, cudaStream_t stream);
-cudaError_t launch_symmetry(const int32_t* off, const int32_t* col, const float* h, int32_t n, long long e,
-                            unsigned* flag, int num_sms, cudaStream_t stream);
+                               const int4* nrec, const float2* lstat, int32_t n, const RowLists& rows, int4* lrec,
+                               int4* gerec, float* gh, int num_sms, cudaStream_t stream);
+// Weight-symmetric: *flag stays 0 and sides[0] == sides[1] (all zeroed before).
+cudaError_t launch_symmetry(const int32_t* off, const int32_t* col, const float* h, int32_t n, const RowLists& rows,
+                            unsigned* flag, unsigned long long* sides, int num_sms, cudaStream_t stream);
 cudaError_t launch_quantize(const int32_t* off, float* h, const float* hmax, int32_t n, uint8_t* codes,
                             float* scales, float* max_scale, unsigned* maxbits, int num_sms, cudaStream_t stream);
 size_t bloom_bytes(int32_t n, long long e);
 size_t table_bytes(int32_t n, long long e);
 cudaError_t prime_preprocess_kernels();
-cudaError_t launch_bloom(const int32_t* off, const int32_t* col, int32_t n, long long e, uint32_t* bloom,
-                         int32_t* mtab, int num_sms, cudaStream_t stream);
+cudaError_t prime_node_stats();
+cudaError_t launch_bloom(const int32_t* off, const int32_t* col, int32_t n, long long e, const RowLists& rows,
+                         uint32_t* bloom, int32_t* mtab, int num_sms, cudaStream_t stream);
 fw_status rebuild_derived(fw_graph* g, cudaStream_t stream);
 cudaError_t launch_check_offsets(const int32_t* off, int32_t n, int64_t e, unsigned* err, int num_sms,
                                  cudaStream_t stream);
-cudaError_t launch_check_rows(const int32_t* off, const int32_t* col, const float* h, int32_t n, unsigned* err,
-                              int num_sms, cudaStream_t stream);
+cudaError_t launch_check_rows(const int32_t* off, const int32_t* col, const float* h, int32_t n, long long e,
+                              unsigned* err, int num_sms, cudaStream_t stream);
 cudaError_t launch_step_plan(const fw_graph* g, const Job& job, const int32_t* v, const int32_t* v_prev,
                              int32_t count, float* bound, float* sum_hat, int32_t* mode, cudaStream_t stream);
 

@@ -1,5 +1,5 @@
-// fw_kernels.cu -- the single-job walk kernel and the preprocessing /
-// validation kernels.
+// fw_kernels.cu -- the single-job walk kernel, the node statistics and the
+// quantization and offset checks (per-row preprocessing: fw_preprocess.cu).
 //
 // A single job is one persistent launch of the walk kernel (fw_walk.cuh)
 // compiled for its algorithm, so the other algorithms' code folds away;
@@ -70,10 +70,14 @@ cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long
 
 // ---------------------------------------------------------------- preprocessing
 // h_MAX[v] and h_SUM[v]: one warp per node, lanes stride over the row
-// (coalesced), then a shuffle-tree max and sum (Sec. 4.2 preprocess()).
+// (coalesced), then a shuffle-tree max and sum (Sec. 4.2 preprocess()).  A
+// lane adds its entries in order, kAhead loads in flight: the kernel lasts as
+// long as the hub row's warp.  Lists the rows too long for one warp in the
+// kernels that follow.
+constexpr int kAhead = 8;
 __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* __restrict__ h, int32_t n,
                                   float* __restrict__ hmax, float* __restrict__ hsum, int4* __restrict__ nrec,
-                                  int* __restrict__ maxdeg) {
+                                  int* __restrict__ maxdeg, RowLists rows) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -82,7 +86,18 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     const int32_t s = off[v], e = off[v + 1];
     float m = 0.0f, sum = 0.0f;
     if (h) {
-      for (int32_t i = s + lane; i < e; i += 32) {
+      int32_t i = s + lane;
+      for (; i + 32 * (kAhead - 1) < e; i += 32 * kAhead) {
+        float x[kAhead];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) x[q] = h[i + 32 * q];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+          m = fmaxf(m, x[q]);
+          sum += x[q];
+        }
+      }
+      for (; i < e; i += 32) {
         const float x = h[i];
         m = fmaxf(m, x);
         sum += x;
@@ -102,6 +117,7 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     if (h) {
       const float half = 0.5f * m, quarter = 0.25f * m;
       n0 = 0;
+#pragma unroll 8
       for (int32_t i = s + lane; i < e; i += 32) {
         const float x = h[i];
         n0 += (x > half) ? 1 : 0;
@@ -118,6 +134,8 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
       hsum[v] = sum;
       nrec[2 * v] = make_int4(s, e - s, __float_as_int(m), __float_as_int(sum));
       nrec[2 * v + 1] = make_int4(n0, n1, 0, 0);
+      if (e - s > kBlockRow) rows.big[atomicAdd(rows.counts + 1, 1)] = (int32_t)v;
+      else if (e - s > kWarpRow) rows.mid[atomicAdd(rows.counts, 1)] = (int32_t)v;
     }
     localmax = max(localmax, e - s);
   }
@@ -125,354 +143,20 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
 }
 
 cudaError_t launch_node_stats(const int32_t* off, const float* h, int32_t n, float* hmax, float* hsum, int4* nrec,
-                              int* maxdeg, int num_sms, cudaStream_t stream) {
+                              int* maxdeg, const RowLists& rows, int num_sms, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   const long long want = ((long long)n * 32 + 255) / 256;
   const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
-  node_stats_kernel<<<grid, 256, 0, stream>>>(off, h, n, hmax, hsum, nrec, maxdeg);
+  node_stats_kernel<<<grid, 256, 0, stream>>>(off, h, n, hmax, hsum, nrec, maxdeg, rows);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }
 
-// Per-label node statistics: {max h, sum h} over the edges of each label
-// l < kLabelStats (h = 1 without weights); one warp per node.  Sets *bad if
-// a label >= kLabelStats occurs (the statistics are then not used).
-__global__ void label_stats_kernel(const int32_t* __restrict__ off, const float* __restrict__ h,
-                                   const uint8_t* __restrict__ lab, int32_t n, float2* __restrict__ out,
-                                   unsigned* __restrict__ bad) {
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long v = warp; v < n; v += nwarps) {
-    float mx[kLabelStats], sm[kLabelStats];
-#pragma unroll
-    for (int l = 0; l < kLabelStats; ++l) mx[l] = sm[l] = 0.0f;
-    bool over = false;
-    for (int32_t i = off[v] + lane; i < off[v + 1]; i += 32) {
-      const int l = lab[i];
-      const float x = h ? h[i] : 1.0f;
-      over |= l >= kLabelStats;
-#pragma unroll
-      for (int k = 0; k < kLabelStats; ++k)
-        if (k == l) {
-          mx[k] = fmaxf(mx[k], x);
-          sm[k] += x;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < kLabelStats; ++k) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mx[k] = fmaxf(mx[k], __shfl_xor_sync(kFull, mx[k], o));
-        sm[k] += __shfl_xor_sync(kFull, sm[k], o);
-      }
-    }
-    if (lane < kLabelStats) {
-      float a = 0.0f, b = 0.0f;
-#pragma unroll
-      for (int k = 0; k < kLabelStats; ++k)
-        if (k == lane) {
-          a = mx[k];
-          b = sm[k];
-        }
-      out[v * kLabelStats + lane] = make_float2(a, b);
-    }
-    if (__any_sync(kFull, over) && lane == 0) atomicOr(bad, 1u);
-  }
-}
-
-// Label-grouped view (metapath): one warp per node reorders its row stably
-// by (label, weight class) -- labels < kLabelStats; within a label, class c
-// < kWClasses - 1 holds h in (M / 2^(c+1), M / 2^c] and the last class h <=
-// M / 2^(kWClasses-1), M the label's max h -- by a counting pass over the
-// kLabelStats * kWClasses buckets, an exclusive prefix over them and a
-// ballot-ranked scatter.  It writes grouped edge records (the second half's
-// third word is the entry's position in the row, the fourth the target's
-// n_A), the grouped h, and per label a 32-byte record {max h, sum h (from
-// the label statistics), segment start, segment length}, {counts of classes
-// 0 .. kWClasses-2}.
-__global__ void label_group_kernel(const int32_t* __restrict__ off, const int32_t* __restrict__ col,
-                                   const float* __restrict__ h, const uint8_t* __restrict__ lab,
-                                   const int4* __restrict__ nrec, const float2* __restrict__ lstat, int32_t n,
-                                   int4* __restrict__ lrec, int4* __restrict__ gerec, float* __restrict__ gh) {
-  constexpr int kB = kLabelStats * kWClasses;  // buckets; bucket k lives in lane k % 32 of (k < 32 ? lo : hi)
-  static_assert(kB <= 64, "two registers of bucket counters per lane");
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long v = warp; v < n; v += nwarps) {
-    const int32_t s = off[v], d = off[v + 1] - s;
-    const float2 ls = lane < kLabelStats ? lstat[v * kLabelStats + lane] : make_float2(0.0f, 0.0f);
-    // bucket of entry i of the row (kB for lanes past the row end)
-    auto bucket = [&](int32_t i, bool valid) -> int {
-      const int l = valid ? (int)lab[s + i] : 0;
-      const float m = __shfl_sync(kFull, ls.x, l);
-      if (!valid) return kB;
-      const float x = h ? h[s + i] : 1.0f;
-      int c = 0;
-      float t = 0.5f * m;
-      while (c < kWClasses - 1 && !(x > t)) {
-        ++c;
-        t *= 0.5f;
-      }
-      return l * kWClasses + c;
-    };
-    int lo = 0, hi = 0;  // bucket counts
-    for (int32_t b = 0; b < d; b += 32) {
-      const int k = bucket(b + lane, b + lane < d);
-#pragma unroll 8
-      for (int q = 0; q < kB; ++q) {
-        const int cnt = __popc(__ballot_sync(kFull, k == q));
-        if (lane == (q & 31)) {
-          if (q < 32) lo += cnt;
-          else hi += cnt;
-        }
-      }
-    }
-    // exclusive prefix over the buckets: lo holds buckets 0..31, hi buckets 32..kB-1
-    int ilo = lo, ihi = hi;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, ilo, o), z = __shfl_up_sync(kFull, ihi, o);
-      if (lane >= o) {
-        ilo += y;
-        ihi += z;
-      }
-    }
-    const int total_lo = __shfl_sync(kFull, ilo, 31);
-    int run_lo = ilo - lo, run_hi = total_lo + ihi - hi;  // start of bucket lane / 32 + lane
-    // per-label record: lane l < kLabelStats gathers its kWClasses buckets
-    {
-      int cnt[kWClasses], start0 = 0;
-#pragma unroll
-      for (int c = 0; c < kWClasses; ++c) {
-        const int q = (lane < kLabelStats ? lane : 0) * kWClasses + c;
-        const int a = __shfl_sync(kFull, lo, q & 31), bb = __shfl_sync(kFull, hi, q & 31);
-        const int sa = __shfl_sync(kFull, run_lo, q & 31), sb = __shfl_sync(kFull, run_hi, q & 31);
-        cnt[c] = q < 32 ? a : bb;
-        if (c == 0) start0 = q < 32 ? sa : sb;
-      }
-      int len = 0;
-#pragma unroll
-      for (int c = 0; c < kWClasses; ++c) len += cnt[c];
-      if (lane < kLabelStats) {
-        lrec[2 * (v * kLabelStats + lane)] = make_int4(__float_as_int(ls.x), __float_as_int(ls.y), start0, len);
-        lrec[2 * (v * kLabelStats + lane) + 1] = make_int4(cnt[0], cnt[1], cnt[2], cnt[3]);
-      }
-    }
-    for (int32_t b = 0; b < d; b += 32) {
-      const bool valid = b + lane < d;
-      const int k = bucket(b + lane, valid);
-      int dst = 0;
-#pragma unroll 8
-      for (int q = 0; q < kB; ++q) {
-        const unsigned m = __ballot_sync(kFull, k == q);
-        const int base = q < 32 ? __shfl_sync(kFull, run_lo, q & 31) : __shfl_sync(kFull, run_hi, q & 31);
-        if (k == q) dst = base + __popc(m & lt);
-        if (lane == (q & 31)) {
-          if (q < 32) run_lo += __popc(m);
-          else run_hi += __popc(m);
-        }
-      }
-      if (valid) {
-        const long long i = (long long)s + b + lane;
-        const int32_t u = col[i];
-        const int4 nr = nrec[2 * u];
-        const float hv = h ? h[i] : 1.0f;
-        const long long o = (long long)s + dst;
-        gerec[2 * o] = make_int4(u, __float_as_int(hv), nr.x, nr.y);
-        gerec[2 * o + 1] = make_int4(nr.z, nr.w, b + lane, 0);
-        gh[o] = hv;
-      }
-    }
-  }
-}
-
-cudaError_t launch_label_group(const int32_t* off, const int32_t* col, const float* h, const uint8_t* lab,
-                               const int4* nrec, const float2* lstat, int32_t n, int4* lrec, int4* gerec, float* gh,
-                               int num_sms, cudaStream_t stream) {
-  label_group_kernel<<<num_sms * 8, 256, 0, stream>>>(off, col, h, lab, nrec, lstat, n, lrec, gerec, gh);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_label_stats(const int32_t* off, const float* h, const uint8_t* lab, int32_t n, float2* out,
-                               unsigned* bad, int num_sms, cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  const long long want = ((long long)n * 32 + 255) / 256;
-  const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
-  label_stats_kernel<<<grid, 256, 0, stream>>>(off, h, lab, n, out, bad);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-// Edge records (32 bytes per CSR entry): everything one eRJS trial needs and
-// everything the next step's plan needs if the trial is accepted.
-__global__ void edge_rec_kernel(const int32_t* __restrict__ col, const float* __restrict__ h,
-                                const uint8_t* __restrict__ lab, const int4* __restrict__ nrec, long long e,
-                                int4* __restrict__ erec) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (long long)gridDim.x * blockDim.x) {
-    const int32_t u = col[i];
-    const int4 nr = nrec[2 * u];
-    const int4 nc = nrec[2 * u + 1];
-    const int hb = h ? __float_as_int(h[i]) : __float_as_int(1.0f);
-    const int lb = lab ? (int)lab[i] : 0;
-    erec[2 * i] = make_int4(u, hb, nr.x, nr.y);
-    // label in the low byte, the target's class-0 count above it (degrees < 2^24)
-    erec[2 * i + 1] = make_int4(nr.z, nr.w, lb | (int)((unsigned)nc.x << 8), nc.y);
-  }
-}
-
-// Class-ordered copy of the edge records: each row stably partitioned into
-// its weight classes 0 (h > h_MAX / 2), 1 (h_MAX / 4 < h <= h_MAX / 2) and
-// 2 (the rest), one warp per row, ballot-ranked scatter.
-__global__ void class_group_kernel(const int32_t* __restrict__ off, const float* __restrict__ h,
-                                   const int4* __restrict__ nrec, const int4* __restrict__ erec, int32_t n,
-                                   int4* __restrict__ cerec) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long v = warp; v < n; v += nwarps) {
-    const int32_t s = off[v], d = off[v + 1] - s;
-    const float m = __int_as_float(nrec[2 * v].z);
-    const float half = 0.5f * m, quarter = 0.25f * m;
-    const int4 nc = nrec[2 * v + 1];
-    int run0 = 0, run1 = nc.x, run2 = nc.x + nc.y;
-    for (int32_t b = 0; b < d; b += 32) {
-      const bool valid = b + lane < d;
-      const long long i = (long long)s + b + lane;
-      const float x = valid ? h[i] : 0.0f;
-      const int cls = (x > half) ? 0 : ((x > quarter) ? 1 : 2);
-      const unsigned m0 = __ballot_sync(kFull, valid && cls == 0), m1 = __ballot_sync(kFull, valid && cls == 1),
-                     m2 = __ballot_sync(kFull, valid && cls == 2);
-      if (valid) {
-        const int r = cls == 0 ? run0 + __popc(m0 & lt) : (cls == 1 ? run1 + __popc(m1 & lt) : run2 + __popc(m2 & lt));
-        const long long o = (long long)s + r;
-        cerec[2 * o] = erec[2 * i];
-        cerec[2 * o + 1] = erec[2 * i + 1];
-      }
-      run0 += __popc(m0);
-      run1 += __popc(m1);
-      run2 += __popc(m2);
-    }
-  }
-}
-
-cudaError_t launch_class_group(const int32_t* off, const float* h, const int4* nrec, const int4* erec, int32_t n,
-                               int4* cerec, int num_sms, cudaStream_t stream) {
-  class_group_kernel<<<num_sms * 8, 256, 0, stream>>>(off, h, nrec, erec, n, cerec);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_edge_records(const int32_t* col, const float* h, const uint8_t* lab, const int4* nrec, long long e,
-                                int4* erec, int num_sms, cudaStream_t stream) {
-  if (e == 0) return cudaSuccess;
-  const long long want = (e + 255) / 256;
-  const int grid = (int)(want < (long long)num_sms * 16 ? want : (long long)num_sms * 16);
-  edge_rec_kernel<<<grid, 256, 0, stream>>>(col, h, lab, nrec, e, erec);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-// Sets *flag if some edge (v, u) has no mirror (u, v) with the same weight.
-// Weight symmetry: does every entry (v, u) have a mirror (u, v) of the same
-// weight?  One thread per entry (a node-per-warp split leaves the hub rows'
-// warps running long after the rest); the entry's row v comes from a binary
-// search of the offsets (L2-resident), its mirror from a search of row u.
-__global__ void symmetry_kernel(const int32_t* __restrict__ off, const int32_t* __restrict__ col,
-                                const float* __restrict__ h, int32_t n, long long e, unsigned* __restrict__ flag) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (long long)gridDim.x * blockDim.x) {
-    int32_t lo = 0, hi = n;  // last v with off[v] <= i
-    while (hi - lo > 1) {
-      const int32_t mid = (lo + hi) >> 1;
-      if (__ldg(off + mid) <= i) lo = mid;
-      else hi = mid;
-    }
-    const int32_t u = col[i];
-    uint32_t pb = 0;
-    const int32_t j = row_find(col, off[u], off[u + 1], lo, n, pb);
-    if (j < 0 || (h && h[j] != h[i])) atomicOr(flag, 1u);
-  }
-}
-
-cudaError_t launch_symmetry(const int32_t* off, const int32_t* col, const float* h, int32_t n, long long e,
-                            unsigned* flag, int num_sms, cudaStream_t stream) {
-  if (n == 0 || e == 0) return cudaSuccess;
-  const long long want = (e + 255) / 256;
-  const int grid = (int)(want < (long long)num_sms * 16 ? want : (long long)num_sms * 16);
-  symmetry_kernel<<<grid, 256, 0, stream>>>(off, col, h, n, e, flag);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-// Blocked Bloom filters and membership tables of the rows with at least
-// kBloomMinDeg entries (layouts and hashing are those of row_member; the
-// table may be nullptr); one warp per row.  A table entry goes to the first
-// slot at or after its home bucket that an atomicCAS finds free (-1); slots
-// are tried in order, so filled slots stay a prefix of every bucket.
-__global__ void bloom_kernel(const int32_t* __restrict__ off, const int32_t* __restrict__ col, int32_t n,
-                             uint32_t* __restrict__ bloom, int32_t* __restrict__ mtab) {
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long x = warp; x < n; x += nwarps) {
-    const int32_t s = off[x], e = off[x + 1];
-    if (e - s < kBloomMinDeg) continue;
-    const long long tb0 = table_bucket0((int32_t)x, s);
-    const uint32_t tnb = table_buckets(s, e);
-    for (int32_t i = s + lane; i < e; i += 32) {
-      const int32_t u = col[i];
-      const unsigned long long hk = bloom_mix((uint32_t)u);
-      uint32_t* blk = bloom + bloom_word((int32_t)x, s, e, hk);
-#pragma unroll
-      for (int j = 0; j < kBloomBits; ++j) {
-        const uint32_t bit = (uint32_t)(hk >> (8 * j)) & 255u;
-        atomicOr(blk + (bit >> 5), 1u << (bit & 31u));
-      }
-      if (mtab) {
-        // at most e - s < 8 * tnb ids share the row's buckets, so a free slot exists
-        uint32_t b = __umulhi((uint32_t)(hk >> 32), tnb);
-        bool placed = false;
-        for (uint32_t k = 0; k < tnb && !placed; ++k) {
-          int32_t* bucket = mtab + 8ll * (tb0 + b);
-          for (int q = 0; q < 8 && !placed; ++q) placed = atomicCAS(bucket + q, -1, u) == -1;
-          b = (b + 1 == tnb) ? 0u : b + 1;
-        }
-      }
-    }
-  }
-}
-
-size_t bloom_bytes(int32_t n, long long e) { return 32ull * (size_t)((e >> 5) + (long long)n + 1); }
-size_t table_bytes(int32_t n, long long e) { return 32ull * (size_t)((e >> 2) + (long long)n + 1); }
-
-cudaError_t launch_bloom(const int32_t* off, const int32_t* col, int32_t n, long long e, uint32_t* bloom,
-                         int32_t* mtab, int num_sms, cudaStream_t stream) {
-  cudaError_t err = cudaMemsetAsync(bloom, 0, bloom_bytes(n, e), stream);
-  if (err == cudaSuccess && mtab) err = cudaMemsetAsync(mtab, 0xff, table_bytes(n, e), stream);
-  if (err != cudaSuccess || n == 0) return err;
-  const long long want = ((long long)n * 32 + 255) / 256;
-  const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
-  bloom_kernel<<<grid, 256, 0, stream>>>(off, col, n, bloom, mtab);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-// Loads the preprocessing kernels (lazy module loading would otherwise do it
-// inside the first timed launch) so that preprocess_ms is kernel time.
-cudaError_t prime_preprocess_kernels() {
+// Loads the statistics kernel (lazy module loading would otherwise do it
+// inside the first timed launch).
+cudaError_t prime_node_stats() {
   cudaFuncAttributes a;
-  cudaError_t e = cudaFuncGetAttributes(&a, node_stats_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, edge_rec_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, symmetry_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, bloom_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, label_stats_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, label_group_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, class_group_kernel);
-  return e;
+  return cudaFuncGetAttributes(&a, node_stats_kernel);
 }
 
 // 8-bit weights with one scale per node: s_v = h_MAX[v] / 255 (FP32
@@ -518,8 +202,8 @@ cudaError_t launch_quantize(const int32_t* off, float* h, const float* hmax, int
   return cudaSuccess;
 }
 
-// CSR validation of device-resident input: bit 1 = offsets, bit 2 = column
-// range, bit 4 = row order, bit 8 = weights.
+// CSR validation of device-resident input: bit 1 = offsets (the rows: see
+// check_rows_kernel).
 __global__ void check_offsets_kernel(const int32_t* __restrict__ off, int32_t n, int64_t e, unsigned* err) {
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += (long long)gridDim.x * blockDim.x) {
     const int32_t o = off[v];
@@ -528,42 +212,11 @@ __global__ void check_offsets_kernel(const int32_t* __restrict__ off, int32_t n,
   }
 }
 
-__global__ void check_rows_kernel(const int32_t* __restrict__ off, const int32_t* __restrict__ col,
-                                  const float* __restrict__ h, int32_t n, unsigned* err) {
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long v = warp; v < n; v += nwarps) {
-    const int32_t s = off[v], e = off[v + 1];
-    unsigned bits = 0;
-    for (int32_t i = s + lane; i < e; i += 32) {
-      const int32_t c = col[i];
-      if (c < 0 || c >= n) bits |= 2u;
-      if (i + 1 < e && col[i + 1] <= c) bits |= 4u;
-      if (h) {
-        const float x = h[i];
-        if (!(x > 0.0f) || !isfinite(x)) bits |= 8u;
-      }
-    }
-    if (bits) atomicOr(err, bits);
-  }
-}
-
 cudaError_t launch_check_offsets(const int32_t* off, int32_t n, int64_t e, unsigned* err, int num_sms,
                                  cudaStream_t stream) {
   const long long want = ((long long)n + 1 + 255) / 256;
   const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
   check_offsets_kernel<<<grid > 0 ? grid : 1, 256, 0, stream>>>(off, n, e, err);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_check_rows(const int32_t* off, const int32_t* col, const float* h, int32_t n, unsigned* err,
-                              int num_sms, cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  const long long want = ((long long)n * 32 + 255) / 256;
-  const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
-  check_rows_kernel<<<grid, 256, 0, stream>>>(off, col, h, n, err);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }
