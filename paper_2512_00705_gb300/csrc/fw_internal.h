@@ -107,6 +107,7 @@ cudaError_t prime_walk_mixed_occupancy();
 // a warp each, up to kBlockRow (`mid`) a block of 8 warps, the rest (`big`) a
 // block of 32.  counts: rows in mid and in big.
 constexpr int32_t kWarpRow = 256, kBlockRow = 2048;
+constexpr int kRowsAtOnce = 8;  // neighbouring rows a warp takes at a time
 struct RowLists {
   int32_t *mid, *big;
   int* counts;

@@ -70,11 +70,10 @@ cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long
 
 // ---------------------------------------------------------------- preprocessing
 // h_MAX[v] and h_SUM[v]: one warp per node, lanes stride over the row
-// (coalesced), then a shuffle-tree max and sum (Sec. 4.2 preprocess()).  A
-// lane adds its entries in order, kAhead loads in flight: the kernel lasts as
-// long as the hub row's warp.  Lists the rows too long for one warp in the
-// kernels that follow.
-constexpr int kAhead = 8;
+// (coalesced), then a shuffle-tree max and sum (Sec. 4.2 preprocess()).
+// Lists the rows too long for one warp in the kernels that follow.  (0.27 ms
+// on R-MAT s20; eight rows' offsets at a time with up to 32 loads in flight
+// took 0.32.)
 __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* __restrict__ h, int32_t n,
                                   float* __restrict__ hmax, float* __restrict__ hsum, int4* __restrict__ nrec,
                                   int* __restrict__ maxdeg, RowLists rows) {
@@ -86,18 +85,7 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     const int32_t s = off[v], e = off[v + 1];
     float m = 0.0f, sum = 0.0f;
     if (h) {
-      int32_t i = s + lane;
-      for (; i + 32 * (kAhead - 1) < e; i += 32 * kAhead) {
-        float x[kAhead];
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) x[q] = h[i + 32 * q];
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-          m = fmaxf(m, x[q]);
-          sum += x[q];
-        }
-      }
-      for (; i < e; i += 32) {
+      for (int32_t i = s + lane; i < e; i += 32) {
         const float x = h[i];
         m = fmaxf(m, x);
         sum += x;
@@ -117,7 +105,6 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     if (h) {
       const float half = 0.5f * m, quarter = 0.25f * m;
       n0 = 0;
-#pragma unroll 8
       for (int32_t i = s + lane; i < e; i += 32) {
         const float x = h[i];
         n0 += (x > half) ? 1 : 0;

@@ -8,7 +8,7 @@
 // tables 7.6, on 31 M entries whose records are 3 GB).  Rows are therefore
 // scanned by teams of their own size: a warp up to kWarpRow entries, a block
 // of 8 warps up to kBlockRow, a block of 32 warps beyond; the longer rows are
-// listed by the node statistics' pass: 4.7 ms on the same graph.  Every stable
+// listed by the node statistics' pass: 4.2 ms on the same graph.  Every stable
 // order is kept: a team's warps own consecutive segments of the row.
 #include "fw_internal.h"
 
@@ -31,11 +31,21 @@ template <int NW, class F>
 __device__ __forceinline__ void for_rows(const int32_t* __restrict__ off, int32_t n, const RowLists& rows,
                                          int32_t least, F f) {
   if (NW == 1) {
+    // kRowsAtOnce neighbouring rows per turn: their offsets come in one load, where each empty row of an R-MAT
+    // graph (two in five) cost a warp the latency of its own
+    const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long v = warp; v < n; v += nwarps) {
-      const int32_t s = off[v], d = off[v + 1] - s;
-      if (d >= least && d <= kWarpRow) f((int32_t)v, s, d);
+    for (long long v0 = warp * kRowsAtOnce; v0 < n; v0 += nwarps * kRowsAtOnce) {
+      const long long at = min(v0 + lane, (long long)n);
+      const int32_t s = lane <= kRowsAtOnce ? off[at] : 0;
+      const int32_t d = __shfl_down_sync(kFull, s, 1) - s;
+      unsigned todo = __ballot_sync(kFull, lane < kRowsAtOnce && d >= least && d <= kWarpRow && v0 + lane < n);
+      while (todo != 0u) {
+        const int j = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        f((int32_t)(v0 + j), __shfl_sync(kFull, s, j), __shfl_sync(kFull, d, j));
+      }
     }
   } else {
     const int32_t* list = NW == 8 ? rows.mid : rows.big;
@@ -196,15 +206,30 @@ __global__ void __launch_bounds__(kTeamBlock)
           }
       }
     }
+    // butterfly over the lanes (16, 8, 4, 2, 1: the order of the plain one); with all labels in the warp, each
+    // exchange also halves the labels a lane keeps, so that lanes 4 l .. 4 l + 3 end with label l
+    int keep = 0;
+    if (NW == 1) {
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
+      for (int o = 16, m = kPer / 2; o >= 4; o >>= 1, m >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mx[k] = fmaxf(mx[k], __shfl_xor_sync(kFull, mx[k], o));
-        sm[k] += __shfl_xor_sync(kFull, sm[k], o);
+        for (int k = 0; k < m; ++k) {
+          const float sx = up ? mx[k] : mx[k + m], ss = up ? sm[k] : sm[k + m];
+          const float kx = up ? mx[k + m] : mx[k], ks = up ? sm[k + m] : sm[k];
+          mx[k] = fmaxf(kx, __shfl_xor_sync(kFull, sx, o));
+          sm[k] = ks + __shfl_xor_sync(kFull, ss, o);
+        }
       }
-      if (lane == 0) out[(long long)v * kLabelStats + first + k] = make_float2(mx[k], sm[k]);
+      keep = lane >> 2;
     }
+#pragma unroll
+    for (int o = NW == 1 ? 2 : 16; o > 0; o >>= 1) {
+      mx[0] = fmaxf(mx[0], __shfl_xor_sync(kFull, mx[0], o));
+      sm[0] += __shfl_xor_sync(kFull, sm[0], o);
+    }
+    if (NW == 1 ? (lane & 3) == 0 : lane == 0)
+      out[(long long)v * kLabelStats + first + keep] = make_float2(mx[0], sm[0]);
     if (__any_sync(kFull, over) && lane == 0) atomicOr(bad, 1u);
   };
   if (NW == 1) {
@@ -412,40 +437,47 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
 }
 
 // ---------------------------------------------------------------- symmetry
-// Does every entry (v, u) have a mirror (u, v) of the same weight?  Entries
-// above the diagonal are looked up in the rows of their targets (*flag is set
-// if one has no mirror); those mirrors are as many distinct entries below it,
-// so no entry there lacks one exactly when both sides have equal counts
-// (sides[0], sides[1]).  Teams know their row, where an entry-parallel kernel
-// searched the offsets for it (s20: 1.40 ms, all entries searched).
+// Does every entry (v, u) have a mirror (u, v) of the same weight?  Of a pair
+// only the entry whose target has the shorter row (equal lengths: the smaller
+// id) is looked up there (*flag is set if it has no mirror); those mirrors
+// are as many distinct entries of the other kind, so none of them lacks its
+// own exactly when both kinds have equal counts (sides[0], sides[1]).  Bound
+// by the searches' random accesses, which the short rows keep to a few; teams
+// know their row (s20, all three sizes: an entry-parallel search of all
+// entries 1.40 ms, teams for those above the diagonal 1.44, by the shorter
+// row 1.28).
 template <int NW>
 __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
     symmetry_kernel(const int32_t* __restrict__ off, const int32_t* __restrict__ col, const float* __restrict__ h,
                     int32_t n, RowLists rows, unsigned* __restrict__ flag, unsigned long long* __restrict__ sides) {
   const int t = NW == 1 ? threadIdx.x & 31 : threadIdx.x;
-  unsigned long long below = 0, above = 0;
+  unsigned long long taken = 0, left = 0;
   bool missing = false;
   for_rows<NW>(off, n, rows, 1, [&](int32_t v, int32_t s, int32_t d) {
     for (int32_t i = s + t; i < s + d; i += NW * 32) {
       const int32_t u = col[i];
-      below += u < v ? 1 : 0;
-      if (u <= v) continue;
-      ++above;
+      if (u == v) continue;  // its own mirror
+      const int32_t us = off[u], ue = off[u + 1];
+      if (ue - us > d || (ue - us == d && u > v)) {
+        ++left;
+        continue;
+      }
+      ++taken;
       uint32_t pb = 0;
-      const int32_t j = row_find(col, off[u], off[u + 1], v, n, pb);
+      const int32_t j = row_find(col, us, ue, v, n, pb);
       missing |= j < 0 || (h && h[j] != h[i]);
     }
   });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    below += __shfl_xor_sync(kFull, below, o);
-    above += __shfl_xor_sync(kFull, above, o);
+    taken += __shfl_xor_sync(kFull, taken, o);
+    left += __shfl_xor_sync(kFull, left, o);
   }
   missing = __any_sync(kFull, missing);
-  if ((threadIdx.x & 31) == 0 && missing) atomicOr(flag, 1u);
-  if ((threadIdx.x & 31) == 0 && (below | above)) {
-    atomicAdd(sides, below);
-    atomicAdd(sides + 1, above);
+  if ((threadIdx.x & 31) == 0) {
+    if (missing) atomicOr(flag, 1u);
+    if (taken) atomicAdd(sides, taken);
+    if (left) atomicAdd(sides + 1, left);
   }
 }
 
@@ -533,7 +565,7 @@ cudaError_t launch_symmetry(const int32_t* off, const int32_t* col, const float*
   return launch_teams(
       [&](int b) { symmetry_kernel<1><<<b, kTeamBlock, 0, st>>>(off, col, h, n, rows, flag, sides); },
       [&](int b) { symmetry_kernel<8><<<b, kTeamBlock, 0, st>>>(off, col, h, n, rows, flag, sides); },
-      [&](int b) { symmetry_kernel<32><<<b, 1024, 0, st>>>(off, col, h, n, rows, flag, sides); }, num_sms);
+      [&](int b) { symmetry_kernel<32><<<2 * b, 1024, 0, st>>>(off, col, h, n, rows, flag, sides); }, num_sms);
 }
 
 size_t bloom_bytes(int32_t n, long long e) { return 32ull * (size_t)((e >> 5) + (long long)n + 1); }
