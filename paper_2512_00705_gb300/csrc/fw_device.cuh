@@ -44,7 +44,8 @@ constexpr int kAlgos = 4;  // a multi-job launch keeps one walker queue per algo
 enum : int32_t { MODE_AUTO = 0, MODE_RJS = 1, MODE_RVS = 2, MODE_EXACT = 3, MODE_RANDOM = 4, MODE_DEGREE = 5 };
 constexpr int32_t kDegreeRuleThreshold = 1000;  // Sec. 5.4 degree-based selection
 enum : int32_t { JOB_WALK = 0, JOB_HIST = 1 };
-enum : int32_t { PLAN_NONE = 0, PLAN_RJS = 1, PLAN_RVS_T = 2, PLAN_RVS_W = 3, PLAN_EXACT_T = 4, PLAN_EXACT_W = 5 };
+enum : int32_t { PLAN_NONE = 0, PLAN_RJS = 1, PLAN_RVS_T = 2, PLAN_RVS_W = 3, PLAN_EXACT_T = 4, PLAN_EXACT_W = 5,
+                PLAN_READY = 6 };  // NONE, READY: no plan yet; READY: the node's record is at hand
 enum : uint32_t { DEVERR_START = 1u, DEVERR_HUB = 2u };
 
 struct DevGraph {

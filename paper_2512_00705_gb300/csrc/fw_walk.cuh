@@ -40,11 +40,6 @@ constexpr int kThreadExactMaxDeg = 16; // exact steps with d <= this run on one 
 // Slot s of lane t lives at obuf[s * kBlock + t] (no bank conflicts).
 constexpr int kStageSlots = 8;  // 32-byte groups
 static_assert(kStageSlots % 4 == 0 && (kStageSlots & (kStageSlots - 1)) == 0, "whole int4s, power of two");
-struct RowStage {
-  int32_t* row;   // current row (nullptr: none)
-  int32_t first;  // first valid slot of the staged group
-};
-
 __device__ __forceinline__ int32_t stage_slot(const int32_t* a) {
   return (int32_t)((reinterpret_cast<uintptr_t>(a) >> 2) & (uintptr_t)(kStageSlots - 1));
 }
@@ -62,30 +57,28 @@ __device__ __forceinline__ void stage_flush(const int32_t* obuf, int tid, int32_
   }
 }
 
-// stage row[p] = val; `final` marks the last entry the lane will write in this row
-__device__ __forceinline__ void stage_put(int32_t* obuf, int tid, RowStage& rs, int32_t p, int32_t val, bool final) {
-  int32_t* a = rs.row + p;
+// stage row[p] = val; `final` marks the last entry the lane will write in this row.  The row's first group may begin
+// before the row.
+__device__ __forceinline__ void stage_put(int32_t* obuf, int tid, int32_t* row, int32_t p, int32_t val, bool final) {
+  int32_t* a = row + p;
   const int32_t slot = stage_slot(a);
   obuf[slot * kBlock + tid] = val;
-  if (slot == kStageSlots - 1 || final) {
-    stage_flush(obuf, tid, a, rs.first, slot);
-    rs.first = 0;
-  }
+  if (slot == kStageSlots - 1 || final) stage_flush(obuf, tid, a, max(slot - p, 0), slot);
 }
 
 // row[from, to) = -1 after a dead end: finish the staged group, then whole groups, then the tail
-__device__ __forceinline__ void stage_fill_minus_one(int32_t* obuf, int tid, RowStage& rs, int32_t from, int32_t to) {
+__device__ __forceinline__ void stage_fill_minus_one(int32_t* obuf, int tid, int32_t* row, int32_t from, int32_t to) {
   int32_t p = from;
-  while (p < to && (p == from || stage_slot(rs.row + p) != 0)) {
-    stage_put(obuf, tid, rs, p, -1, p + 1 == to);
+  while (p < to && (p == from || stage_slot(row + p) != 0)) {
+    stage_put(obuf, tid, row, p, -1, p + 1 == to);
     ++p;
   }
   for (; p + kStageSlots <= to; p += kStageSlots) {
-    int4* q = reinterpret_cast<int4*>(rs.row + p);
+    int4* q = reinterpret_cast<int4*>(row + p);
 #pragma unroll
     for (int k = 0; k < kStageSlots / 4; ++k) q[k] = make_int4(-1, -1, -1, -1);
   }
-  for (; p < to; ++p) rs.row[p] = -1;
+  for (; p < to; ++p) row[p] = -1;
 }
 
 template <int NJ>
@@ -410,12 +403,12 @@ __device__ __forceinline__ int32_t hub_step(const DevGraph& g, const Job* sj, co
 
 // The walk loop of one warp over one queue: take walkers, plan, sample and
 // write rows until the queue is exhausted and the warp holds no walker.
-// `sj` (shared memory) is the queue's job table: its jobs' walkers form the
+// `sj` (shared memory; a single job: kernel parameters) is the queue's job table: its jobs' walkers form the
 // index space [0, total), job j owning [sj[j].gbase, sj[j].gbase + W_j).
 // ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
 // has a lane for every walker, `wpw` walkers per warp, and no queue; SHARE:
 // hub steps may be shared with the block's idle warps (see hub steps).
-template <bool COUNT, int ALG, bool SPREAD, bool SHARE>
+template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE>
 __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
@@ -434,13 +427,18 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC;
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  RowStage rs;
-  rs.row = nullptr;
-  rs.first = 0;
 
-  // walker state: c.v current node, c.vp previous node (-1: none), c.step hop,
-  // c.s / c.d row of c.v, c.ps / c.pe row of c.vp
+  // Walker state that lives across iterations; every word of it is a register
+  // the trials lack (64 per thread with 4 blocks per SM; what does not fit is
+  // spilled in the loop), so values that are never needed together share one
+  // (with the job in constant operands: spill loads of the node2vec kernel
+  // 236 -> 112 bytes; GB300, s22 p = 1/4, q = 4 39.3 -> 33.9 ms, s20 p = 4, q =
+  // 1/4 6.27 -> 5.33 ms, of which the job 5 %):
+  // between a hop and its plan the next node's record sits in c.s, c.d, c.n0,
+  // c.n1, B (h_MAX) and beta (h_SUM).  c.v current node, c.vp previous node
+  // (-1: none), c.step hop, c.s / c.d row of c.v, c.ps / c.pe row of c.vp
+  // (metapath in the label-grouped view: the required label's segment of the
+  // grouped arrays; metapath has no use for the row of v').
   StepCtx c;
   c.v = c.vp = c.s = c.d = c.ps = c.pe = c.step = 0;
   c.wid = 0;
@@ -449,24 +447,17 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   c.n1 = 0;
   c.hsc = 0.0f;
   int32_t job = 0, widx = -1;
-  int32_t plan = PLAN_NONE, trials = 0, pick = -2, node = -1;
+  int32_t plan = PLAN_NONE, trials = 0;
   float B = 0.0f;
   // eRJS with the return edge split off: probability of the return component,
-  // position of v' in N(v) (-1: unknown) and h(v, v')
+  // position of v' in N(v) (-1: unknown) and h(v, v'); before the plan h_ret is h of the edge taken (-1: unknown)
   bool split = false;
-  float beta = 0.0f, h_ret = 0.0f;
+  float beta = 0.0f, h_ret = -1.0f;
   // node2vec with 1/q < 1 and d(v') < d(v): two envelopes; beta2 = (E3 + E2) / E
   bool csplit = false;
   float beta2 = 0.0f;
-  // metapath in the label-grouped view: c.ps / c.pe then hold the required
-  // label's segment of the grouped arrays (metapath has no use for the row of v')
-  bool grp = false;
+  bool grp = false;  // metapath in the label-grouped view
   int32_t pos_ret = -1;
-  // from the accepted trial: the next node's record, and h of the edge taken (-1: unknown)
-  int4 nxt = make_int4(0, 0, 0, 0);
-  int32_t nxt_n0 = 0, nxt_n1 = 0;
-  bool nxt_ok = false;
-  float h_in = -1.0f;
   bool exhausted = false;  // warp-uniform
 
   while (true) {
@@ -488,23 +479,23 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         exhausted = true;
       }
       if (need) {
-        const long long gi = (long long)base + __popc(nm & lt_mask);
+        const long long gi = (long long)base + __popc(nm & ((1u << lane) - 1u));
         if (gi < end) {
-          int j = 0;
-          while (j + 1 < njobs && sj[j + 1].gbase <= gi) ++j;
-          const Job& J = sj[j];
-          job = j;
+          if (NJ > 1) {
+            job = 0;
+            while (job + 1 < njobs && sj[job + 1].gbase <= gi) ++job;
+          }
+          const Job& J = sj[job];
           widx = (int32_t)(gi - J.gbase);
           if (J.kind == JOB_WALK) {
             const int32_t st = __ldg(J.starts + widx);
-            rs.row = J.out + (long long)widx * (J.len + 1);
-            rs.first = stage_slot(rs.row);
+            int32_t* row = J.out + (long long)widx * (J.len + 1);
             if (st < 0 || st >= g.n) {
               atomicOr(err, DEVERR_START);
-              stage_fill_minus_one(obuf, tid, rs, 0, J.len + 1);
+              stage_fill_minus_one(obuf, tid, row, 0, J.len + 1);
               widx = -1;
             } else {
-              stage_put(obuf, tid, rs, 0, st, J.len == 0);
+              stage_put(obuf, tid, row, 0, st, J.len == 0);
               c.v = st;
               c.vp = -1;
               c.step = 0;
@@ -516,14 +507,13 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
             c.step = J.hstep;
             if (c.vp >= 0) {  // during walks the row of v' is carried along; here it is loaded
               const int4 pr = __ldg(g.nrec + 2ll * c.vp);
-              c.s = pr.x;
-              c.d = pr.y;
+              c.ps = pr.x;
+              c.pe = pr.x + pr.y;
             }
           }
+          c.wid = J.wids && widx >= 0 ? __ldg(J.wids + widx) : J.walker_base + (uint32_t)widx;
           plan = PLAN_NONE;
-          pick = -2;
-          nxt_ok = false;
-          h_in = -1.0f;
+          h_ret = -1.0f;
         }
       }
     }
@@ -533,38 +523,30 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     }
 
     const Job& J = sj[job];
+    int32_t pick = -2, node = -1;  // this iteration's outcome: position drawn (-1: dead end, -2: none yet), its node
     // ------------------------------------------------------------ plan
-    if (widx >= 0 && plan == PLAN_NONE) {
-      c.ps = c.s;  // the row of v' is the previous step's row
-      c.pe = c.s + c.d;
-      c.wid = J.wids ? __ldg(J.wids + widx) : J.walker_base + (uint32_t)widx;
-      // row start, degree, h_MAX, h_SUM and class counts of v: from the accepted trial's edge
-      // record, or one load
-      int4 nr;
-      int32_t n0, n1;
-      if (nxt_ok) {
-        nr = nxt;
-        n0 = nxt_n0;
-        n1 = nxt_n1;
-      } else {
-        int4 nr2;
+    if (widx >= 0 && (plan == PLAN_NONE || plan == PLAN_READY)) {
+      // row start, degree, h_MAX, h_SUM and class counts of v: from the hop's edge record, or one load
+      if (plan == PLAN_NONE) {
+        int4 nr, nr2;
         ld_record(g.nrec + 2ll * c.v, nr, nr2);
-        n0 = nr2.x;
-        n1 = nr2.y;
+        c.s = nr.x;
+        c.d = nr.y;
+        c.n0 = nr2.x;
+        c.n1 = nr2.y;
+        B = __int_as_float(nr.z);
+        beta = __int_as_float(nr.w);
         if (COUNT) lc.bytes += 32;
       }
-      nxt_ok = false;
-      c.s = nr.x;
-      c.d = nr.y;
+      const float node_hm = B, node_hs = beta, h_in = h_ret;
+      const int32_t n0 = c.n0, n1 = c.n1;
       if (g.h8) c.hsc = __ldg(g.h8scale + c.v);  // scale of the codes of v's row
       // weight classes in eRJS wherever the bound is a multiple of h_MAX[v]
       const bool cls = J.classes && !(FW_ALGO(J) == ALGO_METAPATH && J.label_stats);
-      c.n0 = cls ? n0 : -1;
-      c.n1 = n1;
+      if (!cls) c.n0 = -1;
       // eRJS envelope mass in units of the class-0 bound: (4 n0 + 2 n1 + n2) / 4
       const float dsl = cls ? __fmul_rn(0.25f, (float)(c.d + 3 * n0 + n1)) : (float)c.d;
       trials = 0;
-      pick = -2;
       split = false;
       csplit = false;
       grp = false;
@@ -580,8 +562,8 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         } else {
           float hm, hs, S;
           if (J.weighted) {
-            hm = __int_as_float(nr.z);
-            hs = __int_as_float(nr.w);
+            hm = node_hm;
+            hs = node_hs;
           } else {
             hm = 1.0f;
             hs = (float)c.d;
@@ -700,9 +682,11 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     const int32_t lane_rvs = !kLaneRvs ? kLaneNone
                              : plan == PLAN_RVS_T ? kLaneJump
                              : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
+    Accept acc;
+    acc.rec_ok = false;
+    acc.h = -1.0f;
     if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
       const bool rvs = lane_rvs != kLaneNone;
-      Accept acc;
       if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
                                  grp, lane_rvs)) {
         if (rvs) {
@@ -711,11 +695,6 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         } else {
           pick = acc.k;
           node = acc.node;
-          h_in = acc.h;
-          nxt = acc.rec;
-          nxt_n0 = acc.rec_n0;
-          nxt_n1 = acc.rec_n1;
-          nxt_ok = acc.rec_ok;
           if (COUNT) lc.rjs_steps++;
         }
       } else {
@@ -816,11 +795,11 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       if (COUNT) lc.bytes += 32;
       pick = in_group ? b.z : ent;
       node = a.x;
-      nxt = make_int4(a.z, a.w, b.x, b.y);
-      nxt_n0 = in_group ? 0 : (int32_t)((uint32_t)b.z >> 8);  // grouped metapath plans without weight classes
-      nxt_n1 = in_group ? 0 : b.w;
-      nxt_ok = true;
-      h_in = J.weighted ? __int_as_float(a.y) : 1.0f;
+      acc.rec = make_int4(a.z, a.w, b.x, b.y);
+      acc.rec_n0 = in_group ? 0 : (int32_t)((uint32_t)b.z >> 8);  // grouped metapath plans without weight classes
+      acc.rec_n1 = in_group ? 0 : b.w;
+      acc.rec_ok = true;
+      acc.h = J.weighted ? __int_as_float(a.y) : 1.0f;
     } else if (ent == -1) {
       pick = -1;
     }
@@ -828,18 +807,32 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     if (widx >= 0 && pick != -2) {
       const int32_t end = (J.kind == JOB_WALK) ? J.len : J.hstep + 1;
       if (J.kind == JOB_WALK) {
+        int32_t* row = J.out + (long long)widx * (J.len + 1);
         if (pick >= 0) {
-          stage_put(obuf, tid, rs, c.step + 1, node, c.step + 1 == end);
+          stage_put(obuf, tid, row, c.step + 1, node, c.step + 1 == end);
         } else {
-          stage_fill_minus_one(obuf, tid, rs, c.step + 1, J.len + 1);
+          stage_fill_minus_one(obuf, tid, row, c.step + 1, J.len + 1);
         }
       } else if (pick >= 0) {
         atomicAdd(J.hist + pick, 1ull);
       }
+      plan = PLAN_NONE;
       if (pick >= 0) {
         c.vp = c.v;
         c.v = node;
+        c.ps = c.s;
+        c.pe = c.s + c.d;
         ++c.step;
+        h_ret = acc.h;
+        if (acc.rec_ok) {
+          c.s = acc.rec.x;
+          c.d = acc.rec.y;
+          c.n0 = acc.rec_n0;
+          c.n1 = acc.rec_n1;
+          B = __int_as_float(acc.rec.z);
+          beta = __int_as_float(acc.rec.w);
+          plan = PLAN_READY;
+        }
         if (COUNT) {
           lc.hops++;
           lc.bytes += 4;
@@ -849,8 +842,6 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         if (COUNT) lc.dead_ends++;
         widx = -1;
       }
-      plan = PLAN_NONE;
-      pick = -2;
     }
   }
 }
@@ -893,17 +884,20 @@ __device__ __forceinline__ void load_jobs(const Job* src_jobs, int njobs, Job* s
   for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
 }
 
-// Single-job (or one-algorithm) launch: the job table in shared memory, one
-// walk loop per warp over the launch's queue.  SHARE: idle warps linger to
+// Single-job (or one-algorithm) launch: one walk loop per warp over the
+// launch's queue.  SHARE: idle warps linger to
 // help the block's hub steps.
 template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(DevGraph g, JobTableN<NJ> tab, int njobs, long long total,
+__global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(const __grid_constant__ DevGraph g,
+                                                      const __grid_constant__ JobTableN<NJ> tab, int njobs, long long total,
                                                       int wpw, unsigned long long* __restrict__ qctr,
                                                       unsigned* __restrict__ err, DevCounters* __restrict__ cnt) {
-  __shared__ Job sj[NJ];
+  __shared__ Job table[NJ > 1 ? NJ : 1];
   __shared__ int32_t obuf[kStageSlots * kBlock];
   __shared__ HubBlock hb;
-  load_jobs(tab.jobs, njobs, sj);
+  // a single job is read where it lies, in the kernel's parameters: constant operands instead of shared-memory loads
+  const Job* sj = NJ > 1 ? table : tab.jobs;
+  if (NJ > 1) load_jobs(tab.jobs, njobs, table);
   if (SHARE && threadIdx.x < kHubTasks) hb.task[threadIdx.x].word = 0u;
   if (SHARE && threadIdx.x == 0) {
     hb.open = 0;
@@ -912,7 +906,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(DevGraph g, Jo
   __syncthreads();
   LaneCounters lc;
   lc.zero();
-  walk_loop<COUNT, ALG, SPREAD, SHARE>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
+  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
   if (SHARE) hub_linger<COUNT, ALG>(g, sj, &hb, lc);
   if (COUNT) flush_counters(lc, cnt);
 }
