@@ -45,7 +45,8 @@ enum : int32_t { MODE_AUTO = 0, MODE_RJS = 1, MODE_RVS = 2, MODE_EXACT = 3, MODE
 constexpr int32_t kDegreeRuleThreshold = 1000;  // Sec. 5.4 degree-based selection
 enum : int32_t { JOB_WALK = 0, JOB_HIST = 1 };
 enum : int32_t { PLAN_NONE = 0, PLAN_RJS = 1, PLAN_RVS_T = 2, PLAN_RVS_W = 3, PLAN_EXACT_T = 4, PLAN_EXACT_W = 5,
-                PLAN_READY = 6 };  // NONE, READY: no plan yet; READY: the node's record is at hand
+                PLAN_READY = 6,    // NONE, READY: no plan yet; READY: the node's record is at hand
+                PLAN_COMMON = 7 }; // second-order PageRank: a common neighbour was drawn and is to be found
 enum : uint32_t { DEVERR_START = 1u, DEVERR_HUB = 2u };
 
 struct DevGraph {
@@ -417,40 +418,6 @@ __device__ __forceinline__ float load_h(const DevGraph& g, const Job& J, int32_t
   return g.h8 ? __fmul_rn((float)__ldg(g.h8 + i), sc) : __ldg(g.h + i);
 }
 
-// Second-order PageRank with a short row of v' (Eq. 2ndpr): the common
-// neighbours C = N(v) and N(v') carry w1 > w2, all others w2.  Enumerating
-// N(v') finds C and S_C = sum of h(v, x) over x in C (FP32, in N(v') order).
-// With t in [0, S_C), common_pick returns the x in C where that running sum
-// first exceeds t (the last one if rounding leaves none), its position in
-// N(v) relative to the row start, and h(v, x).
-static __device__ __noinline__ float common_h_sum(const DevGraph& g, const Job& J, const StepCtx& c, uint32_t& probes) {
-  float sc = 0.0f;
-  for (int32_t j = c.ps; j < c.pe; ++j) {
-    const int32_t pos = row_lookup(g, J, c.v, c.s, c.s + c.d, __ldg(g.col + j), probes);
-    if (pos >= 0) sc = __fadd_rn(sc, load_h(g, J, pos, c.hsc));
-  }
-  return sc;
-}
-
-static __device__ __noinline__ int32_t common_pick(const DevGraph& g, const Job& J, const StepCtx& c, float t,
-                                               int32_t& k, float& hx, uint32_t& probes) {
-  float run = 0.0f;
-  int32_t node = -1;
-  for (int32_t j = c.ps; j < c.pe; ++j) {
-    const int32_t x = __ldg(g.col + j);
-    const int32_t pos = row_lookup(g, J, c.v, c.s, c.s + c.d, x, probes);
-    if (pos < 0) continue;
-    const float h = load_h(g, J, pos, c.hsc);
-    run = __fadd_rn(run, h);
-    node = x;
-    k = pos - c.s;
-    hx = h;
-    if (t < run) break;
-  }
-  return node;
-}
-
-// Transition weight of the neighbour at CSR index i (= s + k) of step c.
 // Transition weight w~ = w * hk of neighbour u (label lb) of step c.
 template <int ALG = -1>
 __device__ __forceinline__ float weight_of(const DevGraph& g, const Job& J, const StepCtx& c, float hk, int32_t u,
@@ -524,6 +491,10 @@ __device__ __forceinline__ bool lemire_index(uint32_t x0, uint32_t x1, uint32_t 
 enum : int32_t { kLaneNone = 0, kLaneJump = 1, kLaneKeyed = 2 };
 constexpr int32_t kLaneKeyedMax = 32;
 
+// Accept::k of a trial that drew the common-neighbour part: h is then t in
+// [0, S_C), and the neighbour is still to be found.
+constexpr int32_t kPickCommon = -3;
+
 // One eRJS acceptance: the neighbour position, the node, its effective
 // property weight, and the target's node record (rec_ok = 0: unknown).
 struct Accept {
@@ -596,10 +567,9 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
     if (COUNT && !rvs) lc.rjs_trials++;
     const float ucomp = u01(x.w);
     if (!rvs && beta > 0.0f && ucomp < beta) {
-      if (FW_ALGO(J) == ALGO_PAGERANK2) {
-        uint32_t pb = 0;
-        acc.node = common_pick(g, J, c, __fmul_rn(u01(x.z), h_ret), acc.k, acc.h, pb);
-        probes += pb;
+      if (FW_ALGO(J) == ALGO_PAGERANK2) {  // a common neighbour, drawn by the warp (see the walk loop)
+        acc.k = kPickCommon;
+        acc.h = __fmul_rn(u01(x.z), h_ret);
       } else {
         acc.k = pos_ret >= 0 ? pos_ret : 0;
         acc.node = c.vp;
