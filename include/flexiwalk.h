@@ -146,7 +146,10 @@ typedef struct {
                               the walker's own lane, longer ones on the whole
                               warp; 1..64 (default 8)                          */
   int32_t rjs_batch;       /* eRJS trials a lane runs between two warp ballots
-                              for hand-offs; 1..16 (default 2)                 */
+                              for hand-offs, 1..16; the trial budget is a
+                              multiple of it.  Default: budgets are multiples
+                              of 2, trials per round follow from the job and
+                              the launch                                       */
   float trial_budget;      /* b of the default rjs_cap, > 0 (default 1)        */
 } fw_params;
 

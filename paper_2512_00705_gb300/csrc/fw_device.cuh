@@ -35,7 +35,7 @@ namespace fw {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxJobs = 64;
 constexpr int kLaneMaxDegree = 8;    // default: eRVS steps with d <= this run on one lane
-constexpr int kRjsBatchDefault = 2;  // default: eRJS trials per round before the warp ballot
+constexpr int kRjsBatchDefault = 2;  // default: trial budgets are a multiple of this, trials per round: round_trials
 constexpr int kLabelStats = 8;       // per-label node statistics for labels 0..7
 constexpr int kWClasses = 5;         // weight classes inside a metapath label segment
 
@@ -101,7 +101,8 @@ struct Job {
   int32_t need_member;     // node2vec with 1/q != 1: membership test needed
   int32_t fixed_cap;       // 1: rjs_cap is a fixed trial cap; 0: cap = max(rjs_cap, ceil(budget * d / ratio))
   int32_t lane_max;        // eRVS steps over at most this many entries run on the walker's lane
-  int32_t rjs_batch;       // eRJS trials per round before the warp's hand-off ballot
+  int32_t rjs_batch;       // the trial budget is a multiple of this
+  int32_t round;           // eRJS trials per round before the warp's hand-off ballot (0: chosen at launch)
   float budget;            // trial budget scale of the default cap
   int32_t split_return;    // node2vec with 1/p > max(1, 1/q): eRJS proposes the return edge separately
   int32_t split_common;    // node2vec with 1/q < 1: eRJS may use the two-envelope proposal (d(v') < d(v))

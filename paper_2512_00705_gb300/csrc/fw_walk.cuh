@@ -757,8 +757,19 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
                              : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
     if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
       const bool rvs = lane_rvs != kLaneNone;
-      if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, J.rjs_batch, acc, lc, csplit, beta2,
-                                 grp, lane_rvs)) {
+      int32_t nt = J.round, budget = 0x7fffffff;
+      if (!rvs && trials + nt >= J.rjs_cap) {
+        // trial budget: the cap, or (default) as many trials as the eRVS scan
+        // they stand in for would cost under the cost model, d / r, times the
+        // budget scale; whole batches of trials
+        const int32_t dd = grp ? c.pe - c.ps : c.d;  // entries the eRVS hand-off would scan
+        const int32_t cap =
+            J.fixed_cap ? J.rjs_cap : max(J.rjs_cap, (int32_t)fminf(ceilf(J.budget * (float)dd / J.ratio), 1.0e9f));
+        budget = (cap + J.rjs_batch - 1) / J.rjs_batch * J.rjs_batch;
+        nt = min(nt, budget - trials);
+      }
+      if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, nt, acc, lc, csplit, beta2,
+                                           grp, lane_rvs)) {
         if (rvs) {
           ent = pos_ret;
           if (COUNT) lc.rvs_steps++;
@@ -771,15 +782,9 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
           if (COUNT) lc.rjs_steps++;
         }
       } else {
-        trials += J.rjs_batch;
-        // trial budget: the cap, or (default) as many trials as the eRVS scan
-        // they stand in for would cost under the cost model, d / r, times the
-        // budget scale
-        const int32_t dd = grp ? c.pe - c.ps : c.d;  // entries the eRVS hand-off would scan
-        const int32_t cap =
-            J.fixed_cap ? J.rjs_cap : max(J.rjs_cap, (int32_t)fminf(ceilf(J.budget * (float)dd / J.ratio), 1.0e9f));
-        if (!rvs && trials >= cap) {
-          plan = (dd <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W;
+        trials += nt;
+        if (trials >= budget) {
+          plan = ((grp ? c.pe - c.ps : c.d) <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W;
           trials = 0;
           split = csplit = false;
           if (COUNT) lc.handoffs++;
@@ -1058,6 +1063,24 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   return cudaSuccess;
 }
 
+// eRJS trials a lane runs per round (0 in the job: this rule; a caller's or
+// a tuned rjs_batch as it is).  After a round the lanes that accepted move on
+// while the others wait, so a second trial pays where most lanes fail the
+// first: measured with 1 / 2 / 3 trials per round on GB300 (s20, ms), U(0,1]
+// weights q = 1/4 2.30 / 2.40 / 2.61 and q = 4 5.05 / 4.88 / 5.05, h = 1 q =
+// 1/4 1.80 / 1.95 / 1.99 and q = 4 3.74 / 3.81 / 4.10, metapath 1.52 / 1.43 /
+// 1.47; second-order PageRank 6.09 / 5.24 / 4.97 and 4.82 with 4; spread
+// launches, bound by latency, 0.369 / 0.331 / 0.326 and 0.318 with 4 (5,003
+// walkers), 57 / 48 / 46 and 45 with 4 (Pareto weights).  Queues of several
+// jobs mix lanes of q < 1 and q > 1 in a warp and keep 2 (64 mixed jobs: 8.54
+// ms, with 1 for q < 1 8.96).
+inline int32_t round_trials(const Job& J, bool spread, int njobs) {
+  if (J.round > 0) return J.round;
+  if (spread || J.algo == ALGO_PAGERANK2) return 4;
+  if (njobs == 1 && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
+  return kRjsBatchDefault;
+}
+
 template <int NJ, bool COUNT, int ALG>
 inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total,
                                  unsigned long long* qctr, cudaStream_t stream) {
@@ -1066,7 +1089,10 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
   if (e != cudaSuccess) return e;
   if (!s.spread && !qctr) return cudaErrorInvalidValue;
   JobTableN<NJ> tab;
-  for (int i = 0; i < njobs; ++i) tab.jobs[i] = jobs[i];
+  for (int i = 0; i < njobs; ++i) {
+    tab.jobs[i] = jobs[i];
+    tab.jobs[i].round = round_trials(jobs[i], s.spread, njobs);
+  }
   if (s.share)
     walk_kernel<NJ, false, ALG, true, true><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw,
                                                                            nullptr, g->d_err, g->d_cnt);
