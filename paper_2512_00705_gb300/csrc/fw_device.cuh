@@ -68,7 +68,7 @@ struct DevGraph {
                                    // classes 0, 1, 2 (class 2: h <= h_MAX / 4); nullptr: no classes
   const float2* __restrict__ lstat; // per node and label l < kLabelStats: {max h, sum h} over the
                                    // edges with that label (nullptr: labels absent or >= kLabelStats)
-  const uint32_t* __restrict__ bloom; // blocked Bloom filters of the rows (nullptr: none)
+  const uint32_t* __restrict__ bloom; // Bloom filters of the rows (nullptr: none)
   const int32_t* __restrict__ mtab;   // per-row membership tables of the node ids (nullptr: none)
   // label-grouped view of the rows (metapath; nullptr: not built): each row
   // reordered stably by (label, weight class).  lrec per node and label
@@ -261,43 +261,51 @@ __device__ __forceinline__ int32_t row_find(const int32_t* __restrict__ col, int
 }
 
 // ---------------------------------------------------------------- membership
-// Blocked Bloom filters over the rows: a pre-check in front of row_find that
-// never changes an answer, it only skips searches whose answer is "absent"
-// (most node2vec candidates with q > 1 lie at distance 2 from v').  Node x
-// owns the 256-bit blocks [bb(x), bb(x+1)) with bb(x) = floor(off[x]/32) + x,
-// one block per 32 row entries plus one; entry u of the row sets kBloomBits
-// bits of one of them, so a filter holds at least 8 bits per entry (false
-// positive rate about 3 %).  Block and bits come from a 64-bit mix of u (the
-// 64-bit finalizer of MurmurHash3, A. Appleby).  Rows shorter than
-// kBloomMinDeg span one or two sectors and are searched directly.
+// Bloom filters over the rows: a pre-check in front of row_find that never
+// changes an answer, it only skips searches whose answer is "absent" (most
+// node2vec candidates with q > 1 lie at distance 2 from v').  Node x owns the
+// 32-bit words [8 bb(x), 8 bb(x+1)) with bb(x) = floor(off[x]/32) + x, eight
+// per 32 row entries plus eight; entry u of the row sets kBloomBits bits of
+// one of them, so a filter holds at least 8 bits per entry (false positive
+// rate about 4 %) and a test is one 4-byte load.  Word and bits come from one
+// 32-bit mix of u (C. Wellons' "lowbias32"): its high part picks the word,
+// its low 5 kBloomBits bits the bits.  (Four bits spread over a 32-byte block
+// by a 64-bit mix took four loads and about 85 instructions, this takes 20:
+// the eRVS scans, bound by instruction issue, test every neighbour.)
+// Rows shorter than kBloomMinDeg span one or two sectors and are searched
+// directly.
 constexpr int32_t kBloomMinDeg = 16;
-constexpr int kBloomBits = 4;
+constexpr int kBloomBits = 3;
 constexpr int32_t kPr2SplitMaxPrev = 64;  // second-order PageRank: longest N(v') enumerated for the split
 
-__device__ __forceinline__ unsigned long long bloom_mix(uint32_t u) {
-  unsigned long long k = (unsigned long long)u + 0x9E3779B97F4A7C15ull;
-  k ^= k >> 33;
-  k *= 0xff51afd7ed558ccdull;
-  k ^= k >> 33;
-  k *= 0xc4ceb9fe1a85ec53ull;
-  k ^= k >> 33;
-  return k;
+__device__ __forceinline__ uint32_t id_hash(uint32_t u) {
+  u ^= u >> 16;
+  u *= 0x7feb352du;
+  u ^= u >> 15;
+  u *= 0x846ca68bu;
+  u ^= u >> 16;
+  return u;
 }
 
-// First word of the block of row x = [rs, re) that entry hash hk maps to.
-__device__ __forceinline__ long long bloom_word(int32_t x, int32_t rs, int32_t re, unsigned long long hk) {
-  const long long b0 = (long long)(rs >> 5) + x;
-  const uint32_t nb = (uint32_t)((re >> 5) - (rs >> 5) + 1);
-  return 8ll * (b0 + (long long)__umulhi((uint32_t)(hk >> 32), nb));
+// Filter of row x = [rs, re): its first word and the number of words.
+__device__ __forceinline__ long long bloom_word0(int32_t x, int32_t rs) { return 8ll * ((long long)(rs >> 5) + x); }
+__device__ __forceinline__ uint32_t bloom_words(int32_t rs, int32_t re) {
+  return 8u * (uint32_t)((re >> 5) - (rs >> 5) + 1);
+}
+
+// Word of hash h among `words`, and its bits there.
+__device__ __forceinline__ uint32_t bloom_word(uint32_t h, uint32_t words) { return __umulhi(h, words); }
+__device__ __forceinline__ uint32_t bloom_bits(uint32_t h) {
+  static_assert(kBloomBits == 3, "three bits from the low 15 of the hash");
+  return (1u << (h & 31u)) | (1u << ((h >> 5) & 31u)) | (1u << ((h >> 10) & 31u));
 }
 
 // Membership tables: an exact set of each row's node ids for rows of at least
 // kBloomMinDeg entries.  Node x owns the 32-byte buckets [tb(x), tb(x+1)),
 // tb(x) = floor(off[x]/4) + x -- more than d/4 buckets of 8 slots, so at most
 // half the slots hold an id and the rest are -1.  Id u lives in the first
-// free slot at or after its home bucket umulhi(hash(u), buckets) (linear
-// probing by bucket, wrapping within the row; hash = the high word of the
-// Bloom mix).  Slots fill in order and are never cleared, so every bucket
+// free slot at or after its home bucket umulhi(id_hash(u), buckets) (linear
+// probing by bucket, wrapping within the row).  Slots fill in order and are never cleared, so every bucket
 // from u's home to the one holding u is full: a lookup reads one bucket,
 // answers "present" on a match and "absent" on a free slot, and moves on
 // only from a full bucket without u (about 5 % of lookups at load 1/2).
@@ -334,10 +342,10 @@ static __device__ __noinline__ bool table_contains_more(const int32_t* __restric
 }
 
 __device__ __forceinline__ bool table_contains(const int32_t* __restrict__ tab, int32_t x, int32_t rs, int32_t re,
-                                               uint32_t hhi, int32_t u, uint32_t& probes) {
+                                               uint32_t h, int32_t u, uint32_t& probes) {
   const long long b0 = table_bucket0(x, rs);
   const uint32_t nb = table_buckets(rs, re);
-  const uint32_t b = __umulhi(hhi, nb);
+  const uint32_t b = __umulhi(h, nb);
   int4 a, c;  // the home bucket
   ld_bucket(tab + 8ll * (b0 + b), a, c);
   ++probes;
@@ -346,19 +354,13 @@ __device__ __forceinline__ bool table_contains(const int32_t* __restrict__ tab, 
   return table_contains_more(tab, b0, nb, b, u, probes);
 }
 
-// Bloom test of u against row x (one probe): false means u is certainly
-// not in the row.
-__device__ __forceinline__ bool bloom_maybe(const DevGraph& g, int32_t x, int32_t rs, int32_t re,
-                                            unsigned long long hk, uint32_t& probes) {
-  const uint32_t* blk = g.bloom + bloom_word(x, rs, re, hk);
+// Bloom test of the id with hash h against row x (one probe): false means it
+// is certainly not in the row.
+__device__ __forceinline__ bool bloom_maybe(const DevGraph& g, int32_t x, int32_t rs, int32_t re, uint32_t h,
+                                            uint32_t& probes) {
   ++probes;
-  uint32_t hit = 1u;
-#pragma unroll
-  for (int j = 0; j < kBloomBits; ++j) {
-    const uint32_t bit = (uint32_t)(hk >> (8 * j)) & 255u;
-    hit &= __ldg(blk + (bit >> 5)) >> (bit & 31u);
-  }
-  return (hit & 1u) != 0u;
+  const uint32_t bits = bloom_bits(h);
+  return (__ldg(g.bloom + bloom_word0(x, rs) + bloom_word(h, bloom_words(rs, re))) & bits) == bits;
 }
 
 // Is u in the row [rs, re) of node x?  Rows of at least kBloomMinDeg
@@ -368,22 +370,22 @@ __device__ __forceinline__ bool bloom_maybe(const DevGraph& g, int32_t x, int32_
 __device__ __forceinline__ bool row_member(const DevGraph& g, const Job& J, int32_t x, int32_t rs, int32_t re,
                                            int32_t u, uint32_t& probes) {
   if (re - rs >= kBloomMinDeg) {
-    if (J.table) return table_contains(g.mtab, x, rs, re, (uint32_t)(bloom_mix((uint32_t)u) >> 32), u, probes);
-    if (J.bloom && !bloom_maybe(g, x, rs, re, bloom_mix((uint32_t)u), probes)) return false;
+    if (J.table) return table_contains(g.mtab, x, rs, re, id_hash((uint32_t)u), u, probes);
+    if (J.bloom && !bloom_maybe(g, x, rs, re, id_hash((uint32_t)u), probes)) return false;
   }
   return row_find(g.col, rs, re, u, g.n, probes) >= 0;
 }
 
 // Membership for the scans of eRVS and exact mode, which test every
 // neighbour of v against the same row of v': the Bloom filter first (its
-// 32-byte blocks, 8 bits per entry, stay cached through the scan), then the
+// words, 8 bits per entry, stay cached through the scan), then the
 // table where the filter passes (or, without tables, the search).  Exact.
 __device__ __forceinline__ bool row_member_scan(const DevGraph& g, const Job& J, int32_t x, int32_t rs, int32_t re,
                                                 int32_t u, uint32_t& probes) {
   if (re - rs >= kBloomMinDeg) {
-    const unsigned long long hk = bloom_mix((uint32_t)u);
-    if (J.bloom && !bloom_maybe(g, x, rs, re, hk, probes)) return false;
-    if (J.table) return table_contains(g.mtab, x, rs, re, (uint32_t)(hk >> 32), u, probes);
+    const uint32_t h = id_hash((uint32_t)u);
+    if (J.bloom && !bloom_maybe(g, x, rs, re, h, probes)) return false;
+    if (J.table) return table_contains(g.mtab, x, rs, re, h, u, probes);
   }
   return row_find(g.col, rs, re, u, g.n, probes) >= 0;
 }
@@ -395,8 +397,8 @@ __device__ __forceinline__ int32_t row_lookup(const DevGraph& g, const Job& J, i
                                               int32_t u, uint32_t& probes) {
   if (re - rs >= kBloomMinDeg) {
     if (J.table) {
-      if (!table_contains(g.mtab, x, rs, re, (uint32_t)(bloom_mix((uint32_t)u) >> 32), u, probes)) return -1;
-    } else if (J.bloom && !bloom_maybe(g, x, rs, re, bloom_mix((uint32_t)u), probes)) {
+      if (!table_contains(g.mtab, x, rs, re, id_hash((uint32_t)u), u, probes)) return -1;
+    } else if (J.bloom && !bloom_maybe(g, x, rs, re, id_hash((uint32_t)u), probes)) {
       return -1;
     }
   }

@@ -32,7 +32,7 @@ struct fw_graph {
   int4* d_cerec = nullptr;     // edge records, rows partitioned by weight class (weighted graphs)
   float2* d_lstat = nullptr;  // per-label node statistics (nullptr: not available)
   bool lstat_bad = false;     // a label >= kLabelStats occurs
-  uint32_t* d_bloom = nullptr; // blocked Bloom filters of the rows (membership pre-check)
+  uint32_t* d_bloom = nullptr; // Bloom filters of the rows (membership pre-check)
   int32_t* d_mtab = nullptr;   // membership tables of the rows (exact; nullptr: not built)
   int4* d_lrec = nullptr;      // label-grouped view for metapath (nullptr: not built)
   int4* d_gerec = nullptr;

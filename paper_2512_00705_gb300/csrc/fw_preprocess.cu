@@ -370,14 +370,13 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
 }
 
 // ---------------------------------------------------------------- filters and tables
-// Blocked Bloom filters and membership tables of the rows with at least
+// Bloom filters and membership tables of the rows with at least
 // kBloomMinDeg entries (layouts and hashing are those of row_member; the
 // table may be nullptr).  An id takes the next slot of its home bucket, or of
 // the first bucket after it that is not full; slots fill in order.  The
 // team's shared memory holds the buckets' slot counts and the row's filter
-// (one shared-memory atomic per bit and per id, where four atomics on the
-// filter and on average 2.5 compare-and-swaps on the table went to L2
-// before); what does not fit, above 100,000 entries the filter and above
+// (one shared-memory atomic each per id, where four atomics on the filter
+// and on average 2.5 compare-and-swaps on the table went to L2 before); what does not fit, above 100,000 entries the filter and above
 // 200,000 the counts too, runs on global memory.
 // kTableWords: shared words a team has.
 // filter: blocks of 8 words, one per 32 entries and up to 2 more; counts: one per bucket, one per 4 entries and up to 2 more
@@ -395,9 +394,9 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
   uint32_t* counts = words + (NW == 1 ? (threadIdx.x >> 5) * kTableWords<NW> : 0);
   for_rows<NW>(off, n, rows, kBloomMinDeg, [&](int32_t v, int32_t s, int32_t d) {
     const int32_t e = s + d;
-    const uint32_t fw = 8u * (uint32_t)((e >> 5) - (s >> 5) + 1);
+    const uint32_t fw = bloom_words(s, e);
     const uint32_t tnb = table_buckets(s, e);
-    uint32_t* gfilter = bloom + 8ll * ((long long)(s >> 5) + v);
+    uint32_t* gfilter = bloom + bloom_word0(v, s);
     int32_t* table = mtab ? mtab + 8ll * table_bucket0(v, s) : nullptr;
     const bool count_here = tnb <= (uint32_t)kTableWords<NW>;  // always, for warps and short blocks
     const bool filter_here = fw + tnb <= (uint32_t)kTableWords<NW>;
@@ -406,16 +405,11 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
     team_sync<NW>();
     for (int32_t i = s + t; i < e; i += NW * 32) {
       const int32_t u = col[i];
-      const unsigned long long hk = bloom_mix((uint32_t)u);
-      uint32_t* blk = bits + (bloom_word(v, s, e, hk) - 8ll * ((long long)(s >> 5) + v));
-#pragma unroll
-      for (int j = 0; j < kBloomBits; ++j) {
-        const uint32_t bit = (uint32_t)(hk >> (8 * j)) & 255u;
-        atomicOr(blk + (bit >> 5), 1u << (bit & 31u));
-      }
+      const uint32_t hk = id_hash((uint32_t)u);
+      atomicOr(bits + bloom_word(hk, fw), bloom_bits(hk));
       if (!table) continue;
       // d < 8 * tnb ids share the row's buckets, so a free slot exists
-      uint32_t b = __umulhi((uint32_t)(hk >> 32), tnb);
+      uint32_t b = __umulhi(hk, tnb);
       bool placed = false;
       for (uint32_t k = 0; k < tnb && !placed; ++k) {
         if (count_here) {
