@@ -51,7 +51,8 @@ def _inputs_digest() -> str:
 
 # The files that define the walk kernel and the device data it reads (records,
 # filters, label-grouped view): profiles of the kernel are keyed to their digest.
-WALK_KERNEL_FILES = ["fw_device.cuh", "fw_walk.cuh", "fw_kernels.cu", "fw_walk_mixed.cu", "fw_internal.h", "fw_api.cu"]
+WALK_KERNEL_FILES = ["fw_device.cuh", "fw_walk.cuh", "fw_kernels.cu", "fw_walk_mixed.cu", "fw_preprocess.cu", "fw_internal.h",
+                     "fw_api.cu"]
 
 
 def _code_only(text: str) -> str:
@@ -99,7 +100,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(r.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=max(1, min(8, os.cpu_count() or 1))) as ex:
+    with ThreadPoolExecutor(max_workers=max(1, min(16, os.cpu_count() or 1))) as ex:
         objs = list(ex.map(compile_one, _sources()))
     tmp = LIB + f".{os.getpid()}.tmp"
     r = subprocess.run([nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-cudart", "static"], capture_output=True, text=True)

@@ -200,9 +200,10 @@ static fw_status build_label_groups(fw_graph* g, const RowLists& rows, cudaStrea
 fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   const int32_t n = g->n;
   const int64_t e = g->e;
-  int* d_maxdeg = reinterpret_cast<int*>(g->d_err) + 8;
-  unsigned* d_asym = g->d_err + 12;
+  int* d_maxdeg = reinterpret_cast<int*>(g->d_err) + 6;
+  unsigned* d_asym = g->d_err + 7;
   unsigned* d_lbad = g->d_err + 13;
+  double* d_mass = reinterpret_cast<double*>(g->d_err) + 4;
   unsigned long long* d_sides = reinterpret_cast<unsigned long long*>(g->d_err) + 1;
   const bool want_labels = g->d_lab != nullptr && !g->lstat_bad;
   const bool build_bloom = g->d_bloom == nullptr;  // depends on the structure only: built once
@@ -243,12 +244,14 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // one memset over the words these kernels use: sides (2..5), max degree (8), asymmetry (12), bad label (13)
+  // one memset over the words these kernels use: sides (2..5), max degree (6), asymmetry (7), envelope mass and
+  // weight (8..11), bad label (13)
   cudaError_t le = cudaMemsetAsync(g->d_err + 2, 0, 12 * sizeof(unsigned), st);
   if (le == cudaSuccess) le = cudaMemsetAsync(rows.counts, 0, 2 * sizeof(int), st);
   cudaEventRecord(e0, st);
   if (le == cudaSuccess)
-    le = launch_node_stats(g->d_off, g->d_h, n, g->d_hmax, g->d_hsum, g->d_nrec, d_maxdeg, rows, g->num_sms, st);
+    le = launch_node_stats(g->d_off, g->d_h, n, g->d_hmax, g->d_hsum, g->d_nrec, d_maxdeg, rows, d_mass, g->num_sms,
+                           st);
   if (le == cudaSuccess && e > 0)
     le = launch_edge_records(g->d_off, g->d_col, g->d_h, g->d_lab, g->d_nrec, n, rows, g->d_erec, g->d_cerec,
                              g->num_sms, st);
@@ -274,9 +277,12 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
     cudaFreeAsync(scratch, st);
     return fs;
   }
-  const int maxdeg = (int)words[8];
+  const int maxdeg = (int)words[6];
+  double mass[2];
+  std::memcpy(mass, words + 8, sizeof(mass));
+  g->envelope = mass[1] > 0.0 ? mass[0] / mass[1] : 1.0;
   g->max_degree = maxdeg;
-  g->sym = words[12] == 0 && words[2] == words[4] && words[3] == words[5] ? 1 : 0;
+  g->sym = words[7] == 0 && words[2] == words[4] && words[3] == words[5] ? 1 : 0;
   if (g->d_cerec && maxdeg >= (1 << 24)) {  // edge records carry class counts in 24 bits
     cudaFree(g->d_cerec);
     g->d_cerec = nullptr;

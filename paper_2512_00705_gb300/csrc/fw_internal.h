@@ -41,6 +41,7 @@ struct fw_graph {
   float* d_h8scale = nullptr; // per node: the scale of its row's codes
   float hscale = 0.0f;        // the largest per-node scale (reported by fw_graph_info)
   int32_t sym = 0;
+  double envelope = 1.0;      // eRJS envelope mass per unit of weight, over all rows (a choice of launch variant only)
   unsigned* d_err = nullptr;
   fw::DevCounters* d_cnt = nullptr;
   float ratio_algo[4] = {4.0f, 4.0f, 4.0f, 4.0f};  // r of Eq. (runtime) per algorithm (fw_algo order)
@@ -115,9 +116,10 @@ struct RowLists {
 size_t row_list_words(long long e);                      // int32 words of scratch the lists need
 RowLists row_lists(int32_t* scratch, long long e);       // lay them out (the counts come first)
 
-// Also fills `rows` (counts zeroed before).
+// Also fills `rows` (counts zeroed before) and adds up the eRJS envelope mass
+// and the weight of all rows in mass[0], mass[1].
 cudaError_t launch_node_stats(const int32_t* off, const float* h, int32_t n, float* hmax, float* hsum, int4* nrec,
-                              int* maxdeg, const RowLists& rows, int num_sms, cudaStream_t stream);
+                              int* maxdeg, const RowLists& rows, double* mass, int num_sms, cudaStream_t stream);
 cudaError_t launch_edge_records(const int32_t* off, const int32_t* col, const float* h, const uint8_t* lab,
                                 const int4* nrec, int32_t n, const RowLists& rows, int4* erec, int4* cerec,
                                 int num_sms, cudaStream_t stream);  // cerec may be nullptr

@@ -1,4 +1,4 @@
-// fw_kernels.cu -- the single-job walk kernel, the node statistics and the
+// fw_kernels.cu -- single-job launches, the node statistics and the
 // quantization and offset checks (per-row preprocessing: fw_preprocess.cu).
 //
 // A single job is one persistent launch of the walk kernel (fw_walk.cuh)
@@ -12,59 +12,34 @@
 namespace fw {
 
 
-template <bool COUNT, bool SPREAD = false, bool SHARE = false>
-static cudaError_t prime_single(int* b) {
-  cudaError_t e = walk_blocks_per_sm<1, COUNT, ALGO_WEIGHTED, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_NODE2VEC, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_METAPATH, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<1, COUNT, ALGO_PAGERANK2, SPREAD, SHARE>(b);
-  return e;
+const WalkLaunches& single_weighted();
+const WalkLaunches& single_node2vec();
+const WalkLaunches& single_metapath();
+const WalkLaunches& single_pagerank2();
+
+const WalkLaunches& single_launches(int algo) {
+  switch (algo) {
+    case ALGO_WEIGHTED: return single_weighted();
+    case ALGO_NODE2VEC: return single_node2vec();
+    case ALGO_METAPATH: return single_metapath();
+    default: return single_pagerank2();
+  }
 }
 
 cudaError_t prime_walk_occupancy() {
-  int b;
-  cudaError_t e = prime_single<false>(&b);
-  if (e == cudaSuccess) e = prime_single<true>(&b);
-  if (e == cudaSuccess) e = prime_single<false, true>(&b);
-  if (e == cudaSuccess) e = prime_single<false, true, true>(&b);
+  cudaError_t e = cudaSuccess;
+  for (int a = 0; a < kAlgos && e == cudaSuccess; ++a) e = single_launches(a).prime();
   if (e == cudaSuccess) e = prime_walk_mixed_occupancy();
   return e;
 }
 
-// One job: the kernel specialised to its algorithm.
-template <bool COUNT>
-static cudaError_t launch_single(const fw_graph* g, const Job* jobs, long long total, unsigned long long* qctr,
-                                 cudaStream_t stream) {
-  switch (jobs[0].algo) {
-    case ALGO_WEIGHTED: return launch_walk_t<1, COUNT, ALGO_WEIGHTED>(g, jobs, 1, total, qctr, stream);
-    case ALGO_NODE2VEC: return launch_walk_t<1, COUNT, ALGO_NODE2VEC>(g, jobs, 1, total, qctr, stream);
-    case ALGO_METAPATH: return launch_walk_t<1, COUNT, ALGO_METAPATH>(g, jobs, 1, total, qctr, stream);
-    default: return launch_walk_t<1, COUNT, ALGO_PAGERANK2>(g, jobs, 1, total, qctr, stream);
-  }
-}
-
-template <bool COUNT>
-static cudaError_t shape_single(const fw_graph* g, const Job* jobs, long long total, LaunchShape* s) {
-  switch (jobs[0].algo) {
-    case ALGO_WEIGHTED: return walk_shape<1, COUNT, ALGO_WEIGHTED>(g, jobs, 1, total, s);
-    case ALGO_NODE2VEC: return walk_shape<1, COUNT, ALGO_NODE2VEC>(g, jobs, 1, total, s);
-    case ALGO_METAPATH: return walk_shape<1, COUNT, ALGO_METAPATH>(g, jobs, 1, total, s);
-    default: return walk_shape<1, COUNT, ALGO_PAGERANK2>(g, jobs, 1, total, s);
-  }
-}
-
 cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, bool* need) {
-  LaunchShape s = {};
-  const cudaError_t e = count ? shape_single<true>(g, &job, total, &s) : shape_single<false>(g, &job, total, &s);
-  *need = !s.spread;
-  return e;
+  return single_launches(job.algo).needs_queue(g, &job, 1, total, count, need);
 }
 
 cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
                         unsigned long long* qctr, cudaStream_t stream) {
-  if (njobs == 1) {
-    return count ? launch_single<true>(g, jobs, total, qctr, stream) : launch_single<false>(g, jobs, total, qctr, stream);
-  }
+  if (njobs == 1) return single_launches(jobs[0].algo).launch(g, jobs, 1, total, count, qctr, stream);
   return launch_walk_mixed(g, jobs, njobs, count, qctr, stream);
 }
 
@@ -76,11 +51,12 @@ cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long
 // took 0.32.)
 __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* __restrict__ h, int32_t n,
                                   float* __restrict__ hmax, float* __restrict__ hsum, int4* __restrict__ nrec,
-                                  int* __restrict__ maxdeg, RowLists rows) {
+                                  int* __restrict__ maxdeg, RowLists rows, double* __restrict__ mass) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   int localmax = 0;
+  double envelope = 0.0, weight = 0.0;  // over the warp's rows: (4 n0 + 2 n1 + n2) / 4 * h_MAX, and h_SUM
   for (long long v = warp; v < n; v += nwarps) {
     const int32_t s = off[v], e = off[v + 1];
     float m = 0.0f, sum = 0.0f;
@@ -125,16 +101,29 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
       else if (e - s > kWarpRow) rows.mid[atomicAdd(rows.counts, 1)] = (int32_t)v;
     }
     localmax = max(localmax, e - s);
+    envelope += 0.25 * (double)(e - s + 3ll * n0 + n1) * (double)m;
+    weight += (double)sum;
   }
   if (lane == 0 && localmax > 0) atomicMax(maxdeg, localmax);
+  __shared__ double part[2][8];
+  if (lane == 0) {
+    part[0][threadIdx.x >> 5] = envelope;
+    part[1][threadIdx.x >> 5] = weight;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double x = 0.0;
+    for (int w = 0; w < 8; ++w) x += part[threadIdx.x][w];
+    atomicAdd(mass + threadIdx.x, x);
+  }
 }
 
 cudaError_t launch_node_stats(const int32_t* off, const float* h, int32_t n, float* hmax, float* hsum, int4* nrec,
-                              int* maxdeg, const RowLists& rows, int num_sms, cudaStream_t stream) {
+                              int* maxdeg, const RowLists& rows, double* mass, int num_sms, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   const long long want = ((long long)n * 32 + 255) / 256;
   const int grid = (int)(want < (long long)num_sms * 8 ? want : (long long)num_sms * 8);
-  node_stats_kernel<<<grid, 256, 0, stream>>>(off, h, n, hmax, hsum, nrec, maxdeg, rows);
+  node_stats_kernel<<<grid, 256, 0, stream>>>(off, h, n, hmax, hsum, nrec, maxdeg, rows, mass);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }

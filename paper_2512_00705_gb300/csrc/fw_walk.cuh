@@ -401,14 +401,36 @@ __device__ __forceinline__ int32_t hub_step(const DevGraph& g, const Job* sj, co
   return (bk == -CUDART_INF_F) ? -1 : bi;
 }
 
+// Trials together: failed trials after which a step's next ones are made by
+// the whole warp.  The code costs the loop registers, so it is a kernel
+// variant, used on graphs whose mean envelope mass per unit of weight, the
+// trials of a first-order hop, is at least kTogetherEnvelope.  Second-order
+// PageRank, whose steps without a split fail most trials, uses it from
+// kTogetherPagerank, and for few walkers always.
+// GB300, R-MAT s18 x 10 hops, 20,000 / 400,000 walkers, a lane's own trials
+// -> together (ms): envelope 1.4 (U(0,1] weights) node2vec p = 2, q = 1/2
+// 0.10 / 0.53 -> 0.13 / 0.78, PageRank 0.46 / 2.19 -> 0.26 / 2.03; 3.6
+// (lognormal) node2vec 0.24 / 0.99 -> 0.26 / 2.09, weighted 0.11 / 0.55 ->
+// 0.11 / 0.62, PageRank 1.93 / 5.22 -> 0.47 / 3.26; 6.5 (Pareto 2) node2vec
+// 1.07 / 4.58 -> 0.35 / 2.77, weighted 0.91 / 2.37 -> 0.13 / 0.80; 246
+// (Pareto 1) node2vec 7.9 / 29.6 -> 2.8 / 19.6, weighted 7.1 / 13.5 -> 0.9 /
+// 5.0, metapath 0.41 / 1.42 -> 0.13 / 0.73.  From 8 / 16 / 32 trials: Pareto
+// 1 node2vec 19.6 / 21.4 / 23.3, PageRank on U(0,1] 2.16 / 2.03 / 1.92 and on
+// Pareto 1 21.3 / 22.6 / 24.7; PageRank on s20, U(0,1], 262,144 walkers x 40
+// hops 4.9 -> 5.3.
+template <int ALG>
+constexpr int32_t kTogetherFrom = ALG == ALGO_PAGERANK2 ? 16 : 8;
+constexpr double kTogetherEnvelope = 5.0, kTogetherPagerank = 2.5;
+
 // The walk loop of one warp over one queue: take walkers, plan, sample and
 // write rows until the queue is exhausted and the warp holds no walker.
 // `sj` (shared memory; a single job: kernel parameters) is the queue's job table: its jobs' walkers form the
 // index space [0, total), job j owning [sj[j].gbase, sj[j].gbase + W_j).
 // ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
-// has a lane for every walker, `wpw` walkers per warp, and no queue; SHARE:
-// hub steps may be shared with the block's idle warps (see hub steps).
-template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE>
+// is given its first walkers by place, `wpw` per warp; SHARE: hub steps may be
+// shared with the block's idle warps (see hub steps); COOP: long eRJS steps
+// try 32 proposals at once (see trials together).
+template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP>
 __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
@@ -459,28 +481,29 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   bool grp = false;  // metapath in the label-grouped view
   int32_t pos_ret = -1;
   bool exhausted = false;  // warp-uniform
+  bool first = SPREAD;     // warp-uniform
 
   while (true) {
     // ------------------------------------------------------------ fetch
-    const bool need = widx < 0;
+    const bool need = widx < 0 && (!SPREAD || lane < wpw);
     const unsigned nm = __ballot_sync(kFull, need);
     if (nm != 0u && !exhausted) {
       const int leader = __ffs(nm) - 1;
       const unsigned cntw = __popc(nm);
       unsigned long long base = 0;
-      long long end = total;
-      if (!SPREAD) {
+      if (SPREAD && first) {  // warp 0 of every block first, then warp 1, ...
+        base = (unsigned)((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (unsigned)wpw;
+        first = false;
+        if (qctr == nullptr) exhausted = true;
+      } else {
         if (lane == leader) base = atomicAdd(qctr, (unsigned long long)cntw);
         base = __shfl_sync(kFull, base, leader);
-        if (base + cntw >= (unsigned long long)total) exhausted = true;
-      } else {  // warp 0 of every block first, then warp 1, ...
-        base = (unsigned)((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (unsigned)wpw;
-        end = min(end, (long long)base + wpw);
-        exhausted = true;
+        if (SPREAD) base += (unsigned)(gridDim.x * (blockDim.x >> 5)) * (unsigned long long)wpw;
       }
+      if (base + cntw >= (unsigned long long)total) exhausted = true;
       if (need) {
         const long long gi = (long long)base + __popc(nm & ((1u << lane) - 1u));
-        if (gi < end) {
+        if (gi < total) {
           if (NJ > 1) {
             job = 0;
             while (job + 1 < njobs && sj[job + 1].gbase <= gi) ++job;
@@ -861,6 +884,92 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         }
       }
     }
+    // ------------------------------------------------------------ trials together
+    // A step that failed that many trials will most likely fail as many
+    // again: the warp makes its next trials 32 at a time (trial t draws from
+    // its own counter, so the first accepted one is the one the lane would
+    // have come to) until one is accepted or the budget ends.
+    if (COOP) {
+      unsigned cm = __ballot_sync(kFull, widx >= 0 && pick == -2 && plan == PLAN_RJS && trials >= kTogetherFrom<ALG>);
+      while (cm != 0u) {
+        const int src = __ffs(cm) - 1;
+        cm &= cm - 1u;
+        StepCtx w;
+        w.v = __shfl_sync(kFull, c.v, src);
+        w.vp = __shfl_sync(kFull, c.vp, src);
+        w.s = __shfl_sync(kFull, c.s, src);
+        w.d = __shfl_sync(kFull, c.d, src);
+        w.ps = __shfl_sync(kFull, c.ps, src);
+        w.pe = __shfl_sync(kFull, c.pe, src);
+        w.step = __shfl_sync(kFull, c.step, src);
+        w.wid = __shfl_sync(kFull, c.wid, src);
+        w.n0 = __shfl_sync(kFull, c.n0, src);
+        w.n1 = __shfl_sync(kFull, c.n1, src);
+        w.hsc = g.h8 ? __shfl_sync(kFull, c.hsc, src) : 0.0f;
+        if (ALG == ALGO_PAGERANK2) {
+          w.w1 = __shfl_sync(kFull, c.w1, src);
+          w.w2 = __shfl_sync(kFull, c.w2, src);
+        }
+        if (ALG == ALGO_METAPATH) {
+          w.gcls.x = __shfl_sync(kFull, c.gcls.x, src);
+          w.gcls.y = __shfl_sync(kFull, c.gcls.y, src);
+          w.gcls.z = __shfl_sync(kFull, c.gcls.z, src);
+          w.gcls.w = __shfl_sync(kFull, c.gcls.w, src);
+        }
+        const Job& JW = sj[NJ > 1 ? __shfl_sync(kFull, job, src) : 0];
+        const float wB = __shfl_sync(kFull, B, src), wh = __shfl_sync(kFull, h_ret, src);
+        float wbeta = __shfl_sync(kFull, beta, src), wbeta2 = __shfl_sync(kFull, beta2, src);
+        int32_t wpos = __shfl_sync(kFull, pos_ret, src);
+        const int fl = __shfl_sync(kFull, (split ? 1 : 0) | (csplit ? 2 : 0) | (grp ? 4 : 0), src);
+        const int32_t dd = (fl & 4) ? w.pe - w.ps : w.d;
+        const int32_t cap =
+            JW.fixed_cap ? JW.rjs_cap : max(JW.rjs_cap, (int32_t)fminf(ceilf(JW.budget * (float)dd / JW.ratio), 1.0e9f));
+        const int32_t budget = (cap + JW.rjs_batch - 1) / JW.rjs_batch * JW.rjs_batch;
+        int32_t t = __shfl_sync(kFull, trials, src);
+        unsigned hit = 0;
+        Accept wa;
+        wa.rec_ok = false;
+        wa.k = -2;
+        wa.node = -1;
+        wa.h = -1.0f;
+        wa.rec = make_int4(0, 0, 0, 0);
+        wa.rec_n0 = wa.rec_n1 = 0;
+        while (hit == 0u && t < budget) {
+          const bool got = t + lane < budget &&
+                           rjs_trials<COUNT, ALG, false>(g, JW, w, wB, (fl & 1) != 0, wbeta, wpos, wh, t + lane, 1, wa, lc,
+                                                         (fl & 2) != 0, wbeta2, (fl & 4) != 0);
+          hit = __ballot_sync(kFull, got);
+          t += 32;
+        }
+        const int win = hit ? __ffs(hit) - 1 : 0;
+        wa.k = __shfl_sync(kFull, wa.k, win);
+        wa.node = __shfl_sync(kFull, wa.node, win);
+        wa.h = __shfl_sync(kFull, wa.h, win);
+        wa.rec.x = __shfl_sync(kFull, wa.rec.x, win);
+        wa.rec.y = __shfl_sync(kFull, wa.rec.y, win);
+        wa.rec.z = __shfl_sync(kFull, wa.rec.z, win);
+        wa.rec.w = __shfl_sync(kFull, wa.rec.w, win);
+        wa.rec_n0 = __shfl_sync(kFull, wa.rec_n0, win);
+        wa.rec_n1 = __shfl_sync(kFull, wa.rec_n1, win);
+        wa.rec_ok = __shfl_sync(kFull, (int)wa.rec_ok, win) != 0;
+        if (lane == src) {
+          if (hit == 0u) {
+            plan = dd <= J.lane_max ? PLAN_RVS_T : PLAN_RVS_W;
+            trials = 0;
+            split = csplit = false;
+            if (COUNT) lc.handoffs++;
+          } else if (ALG == ALGO_PAGERANK2 && wa.k == kPickCommon) {
+            plan = PLAN_COMMON;
+            h_ret = wa.h;
+          } else {
+            acc = wa;
+            pick = wa.k;
+            node = wa.node;
+            if (COUNT) lc.rjs_steps++;
+          }
+        }
+      }
+    }
     // ------------------------------------------------------------ entry drawn -> node and its record
     // One 32-byte edge record gives the node, its node record and h of the
     // edge, as an accepted trial does: the column, the node record and the
@@ -965,7 +1074,7 @@ __device__ __forceinline__ void load_jobs(const Job* src_jobs, int njobs, Job* s
 // Single-job (or one-algorithm) launch: one walk loop per warp over the
 // launch's queue.  SHARE: idle warps linger to
 // help the block's hub steps.
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false>
 __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(const __grid_constant__ DevGraph g,
                                                       const __grid_constant__ JobTableN<NJ> tab, int njobs, long long total,
                                                       int wpw, unsigned long long* __restrict__ qctr,
@@ -984,17 +1093,17 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(const __grid_c
   __syncthreads();
   LaneCounters lc;
   lc.zero();
-  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
+  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE, COOP>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
   if (SHARE) hub_linger<COUNT, ALG>(g, sj, &hb, lc);
   if (COUNT) flush_counters(lc, cnt);
 }
 
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false>
 inline cudaError_t walk_blocks_per_sm(int* out) {
   static std::atomic<int> cached{0};
   int b = cached.load();
   if (b == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE>, kBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP>, kBlock, 0);
     if (e != cudaSuccess) return e;
     b = b > 0 ? b : 1;
     cached.store(b);
@@ -1025,7 +1134,12 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // iteration and scans its lanes' long rows one after another, so walkers are
 // spread over the resident warps before they share one -- wpw is the
 // smallest count with which they fit, and blocks fill before warps do.  No
-// queue counter is needed then.  More walkers than lanes: full warps that
+// queue counter is needed then.  Jobs that only scan rows (forced eRVS,
+// exact mode) keep one walker per warp at every size, the rest in the queue:
+// the warp works for one walker at a time anyway, and a warp's lot of 14
+// walkers with hub rows made some warps run long after the others (65,536
+// walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
+// with 1).  Other launches with more walkers than lanes: full warps that
 // fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
 // full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
@@ -1035,6 +1149,8 @@ struct LaunchShape {
   int grid, wpw;
   bool spread;
   bool share;  // spread, with hub sharing
+  bool coop;   // trials together (see the walk loop)
+  bool queue;  // needs a zeroed queue counter
 };
 
 template <int NJ, bool COUNT, int ALG>
@@ -1045,21 +1161,39 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   if (e != cudaSuccess) return e;
   long long blocks = (long long)g->num_sms * bps;
   s->wpw = 32;
-  s->spread = s->share = false;
+  s->spread = s->share = s->coop = false;
+  bool scans = true, trials = false;
+  for (int i = 0; i < njobs; ++i) {
+    const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
+    scans = scans && scan;
+    trials = trials || (!scan && jobs[i].weighted);
+  }
   if (!COUNT) {
     s->share = hub_share_pays(g, jobs, njobs, total, blocks * kBlock);
-    e = s->share ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps) : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
+    // whether it spreads does not depend on coop: both spread kernels have the same occupancy (their launch bounds)
+    const bool few = total <= blocks * kBlock;
+    s->coop = ALG == ALGO_PAGERANK2 ? !scans && (few || g->envelope >= kTogetherPagerank)
+                                    : trials && g->envelope >= kTogetherEnvelope;
+    e = s->share  ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
+        : s->coop ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
+                  : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
     if (e != cudaSuccess) return e;
     const long long spread_blocks = (long long)g->num_sms * bps;
-    s->spread = total <= spread_blocks * kBlock;
+    s->spread = scans || total <= spread_blocks * kBlock;
     s->share = s->share && s->spread;
     if (s->spread) {
       blocks = spread_blocks;
-      s->wpw = (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
+      s->wpw = scans ? 1 : (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
     }
+  }
+  if (!s->spread && s->coop) {
+    e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&bps);
+    if (e != cudaSuccess) return e;
+    blocks = (long long)g->num_sms * bps;
   }
   const long long per_block = s->spread ? s->wpw : kBlock;  // a spread launch takes a block for every warp while it can
   s->grid = (int)std::min<long long>(blocks, std::max<long long>(1, (total + per_block - 1) / per_block));
+  s->queue = !s->spread || (long long)s->grid * kWarps * s->wpw < total;
   return cudaSuccess;
 }
 
@@ -1087,23 +1221,72 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
   LaunchShape s;
   cudaError_t e = walk_shape<NJ, COUNT, ALG>(g, jobs, njobs, total, &s);
   if (e != cudaSuccess) return e;
-  if (!s.spread && !qctr) return cudaErrorInvalidValue;
+  if (s.queue && !qctr) return cudaErrorInvalidValue;
+  if (!s.queue) qctr = nullptr;
   JobTableN<NJ> tab;
   for (int i = 0; i < njobs; ++i) {
     tab.jobs[i] = jobs[i];
     tab.jobs[i].round = round_trials(jobs[i], s.spread, njobs);
   }
-  if (s.share)
-    walk_kernel<NJ, false, ALG, true, true><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw,
-                                                                           nullptr, g->d_err, g->d_cnt);
-  else if (s.spread)
-    walk_kernel<NJ, false, ALG, true><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, nullptr,
-                                                                     g->d_err, g->d_cnt);
-  else
-    walk_kernel<NJ, COUNT, ALG><<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err,
-                                                               g->d_cnt);
+  auto launch = [&](auto kernel) {
+    kernel<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err, g->d_cnt);
+  };
+  if (s.share) launch(walk_kernel<NJ, false, ALG, true, true>);
+  else if (s.spread && s.coop) launch(walk_kernel<NJ, false, ALG, true, false, true>);
+  else if (s.spread) launch(walk_kernel<NJ, false, ALG, true>);
+  else if (s.coop) launch(walk_kernel<NJ, false, ALG, false, false, true>);
+  else launch(walk_kernel<NJ, COUNT, ALG>);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }
 
+// Cache the occupancy of every variant for one algorithm (outside any capture).
+template <int NJ, int ALG>
+inline cudaError_t prime_walk() {
+  int b;
+  cudaError_t e = walk_blocks_per_sm<NJ, false, ALG>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, true, ALG>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, true>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&b);
+  return e;
+}
+
+// The launches of one algorithm over a table of at most NJ jobs; each is
+// instantiated in a source file of its own (WALK_LAUNCHES), so that they
+// compile side by side.
+struct WalkLaunches {
+  cudaError_t (*launch)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+                        unsigned long long* qctr, cudaStream_t stream);
+  cudaError_t (*needs_queue)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, bool* need);
+  cudaError_t (*prime)();
+};
+const WalkLaunches& single_launches(int algo);  // one job
+const WalkLaunches& table_launches(int algo);   // up to kMaxJobs jobs
+
+template <int NJ, int ALG>
+inline WalkLaunches make_launches() {
+  return {[](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, unsigned long long* qctr,
+             cudaStream_t st) {
+            return count ? launch_walk_t<NJ, true, ALG>(g, jobs, njobs, total, qctr, st)
+                         : launch_walk_t<NJ, false, ALG>(g, jobs, njobs, total, qctr, st);
+          },
+          [](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, bool* need) {
+            LaunchShape s = {};
+            const cudaError_t e = count ? walk_shape<NJ, true, ALG>(g, jobs, njobs, total, &s)
+                                        : walk_shape<NJ, false, ALG>(g, jobs, njobs, total, &s);
+            *need = s.queue;
+            return e;
+          },
+          prime_walk<NJ, ALG>};
+}
+
+#define WALK_LAUNCHES(NAME, NJ, ALG)                             \
+  namespace fw {                                                 \
+  const WalkLaunches& NAME() {                                   \
+    static const WalkLaunches launches = make_launches<NJ, ALG>(); \
+    return launches;                                             \
+  }                                                              \
+  }
 }  // namespace fw

@@ -15,36 +15,23 @@
 #include "fw_walk.cuh"
 
 namespace fw {
-namespace {
+const WalkLaunches& table_weighted();
+const WalkLaunches& table_node2vec();
+const WalkLaunches& table_metapath();
+const WalkLaunches& table_pagerank2();
 
-template <bool COUNT>
-cudaError_t launch_group(int a, const fw_graph* g, const Job* jobs, int njobs, long long total,
-                         unsigned long long* qctr, cudaStream_t st) {
-  switch (a) {
-    case ALGO_WEIGHTED: return launch_walk_t<kMaxJobs, COUNT, ALGO_WEIGHTED>(g, jobs, njobs, total, qctr, st);
-    case ALGO_NODE2VEC: return launch_walk_t<kMaxJobs, COUNT, ALGO_NODE2VEC>(g, jobs, njobs, total, qctr, st);
-    case ALGO_METAPATH: return launch_walk_t<kMaxJobs, COUNT, ALGO_METAPATH>(g, jobs, njobs, total, qctr, st);
-    default: return launch_walk_t<kMaxJobs, COUNT, ALGO_PAGERANK2>(g, jobs, njobs, total, qctr, st);
+const WalkLaunches& table_launches(int algo) {
+  switch (algo) {
+    case ALGO_WEIGHTED: return table_weighted();
+    case ALGO_NODE2VEC: return table_node2vec();
+    case ALGO_METAPATH: return table_metapath();
+    default: return table_pagerank2();
   }
 }
 
-template <bool COUNT, bool SPREAD = false, bool SHARE = false>
-cudaError_t prime_groups(int* b) {
-  cudaError_t e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_WEIGHTED, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_NODE2VEC, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_METAPATH, SPREAD, SHARE>(b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<kMaxJobs, COUNT, ALGO_PAGERANK2, SPREAD, SHARE>(b);
-  return e;
-}
-
-}  // namespace
-
 cudaError_t prime_walk_mixed_occupancy() {
-  int b;
-  cudaError_t e = prime_groups<false>(&b);
-  if (e == cudaSuccess) e = prime_groups<true>(&b);
-  if (e == cudaSuccess) e = prime_groups<false, true>(&b);
-  if (e == cudaSuccess) e = prime_groups<false, true, true>(&b);
+  cudaError_t e = cudaSuccess;
+  for (int a = 0; a < kAlgos && e == cudaSuccess; ++a) e = table_launches(a).prime();
   return e;
 }
 
@@ -79,8 +66,7 @@ cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, boo
   for (int i = 0; i < np && e == cudaSuccess; ++i) {
     const int a = present[i];
     cudaStream_t st = (fork && i > 0) ? side[i - 1] : stream;
-    e = count ? launch_group<true>(a, g, grp + firsts[a], counts[a], totals[a], qctr + a, st)
-              : launch_group<false>(a, g, grp + firsts[a], counts[a], totals[a], qctr + a, st);
+    e = table_launches(a).launch(g, grp + firsts[a], counts[a], totals[a], count, qctr + a, st);
   }
   if (fork) {  // `stream` waits for the helper streams
     for (int i = 1; i < np && e == cudaSuccess; ++i) {

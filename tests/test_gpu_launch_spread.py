@@ -75,3 +75,38 @@ def test_lane_scans_in_step_with_trials_equal_whole_lane_scans(p, q, mode, flags
     assert torch.equal(a, b)
     assert G.counters()["rvs_steps"] > 0
     G.close()
+
+
+@pytest.fixture(scope="module")
+def skewed():
+    g = synth.workload_graph("small")
+    g.h = synth.edge_weights(g, "pareto", 1.0, seed=7)
+    G = fw.Graph(g)
+    yield g, G
+    G.close()
+
+
+@pytest.mark.parametrize("algo,p,q", [("weighted", 1.0, 1.0), ("node2vec", 2.0, 0.5), ("node2vec", 0.25, 4.0),
+                                      ("metapath", 1.0, 1.0), ("pagerank2", 1.0, 1.0)])
+@pytest.mark.parametrize("mode,shape", [("auto", {}), ("rjs", {"rjs_cap": 61}), ("rjs", {"rjs_cap": 9, "rjs_batch": 4}),
+                                        ("rjs", {"rjs_cap": 1 << 30})])
+@pytest.mark.parametrize("walkers,length", [(4099, 12), (155700, 2)])
+def test_trials_together_equal_a_lanes_own(skewed, algo, p, q, mode, shape, walkers, length):
+    """Heavy-tailed weights: steps of many failed trials are tried by the whole
+    warp, except in the counting build."""
+    g, G = skewed
+    starts = torch.from_numpy(synth.random_starts(g.n, walkers, seed=11)).cuda()
+    schema = [0, 1, 2] if algo == "metapath" else None
+    a = G.walk(starts, length, algo, p=p, q=q, schema=schema, mode=mode, seed=3, **shape)
+    b = G.walk(starts, length, algo, p=p, q=q, schema=schema, mode=mode, seed=3, flags=fw.FLAG_COUNTERS, **shape)
+    assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("mode", ["rvs", "exact"])
+def test_scanning_jobs_queue_behind_one_walker_per_warp(walks, mode):
+    g, G, lanes, starts = walks
+    w = lanes // 32 * 3 + 5
+    dev = torch.from_numpy(starts[:w]).cuda()
+    a = G.walk(dev, 6, "node2vec", p=2.0, q=0.5, mode=mode, seed=9)
+    b = G.walk(dev, 6, "node2vec", p=2.0, q=0.5, mode=mode, seed=9, flags=fw.FLAG_COUNTERS)
+    assert torch.equal(a, b)
