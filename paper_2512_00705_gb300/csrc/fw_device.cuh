@@ -392,21 +392,24 @@ __device__ __forceinline__ bool row_member_scan(const DevGraph& g, const Job& J,
 
 // Position of u in the row [rs, re) of node x, or -1: the table or the
 // filter answers "absent" without a search; otherwise the search gives the
-// position.  Exact.
+// position.  FILTER: ask the filter even where there is a table.  Exact.
+template <bool FILTER = false>
 __device__ __forceinline__ int32_t row_lookup(const DevGraph& g, const Job& J, int32_t x, int32_t rs, int32_t re,
                                               int32_t u, uint32_t& probes) {
   if (re - rs >= kBloomMinDeg) {
-    if (J.table) {
+    if (FILTER ? J.bloom : J.bloom && !J.table) {
+      if (!bloom_maybe(g, x, rs, re, id_hash((uint32_t)u), probes)) return -1;
+    } else if (J.table) {
       if (!table_contains(g.mtab, x, rs, re, id_hash((uint32_t)u), u, probes)) return -1;
-    } else if (J.bloom && !bloom_maybe(g, x, rs, re, id_hash((uint32_t)u), probes)) {
-      return -1;
     }
   }
   return row_find(g.col, rs, re, u, g.n, probes);
 }
 
 // Is u in N(v') (the row [c.ps, c.pe) of c.vp)?  SCAN: the test of a scan
-// over N(v) (eRVS, exact mode) rather than of one eRJS trial.
+// over N(v) (eRVS, exact mode) rather than of one eRJS trial.  (Filter first
+// in node2vec's trials too: s22 p = 1/4, q = 4 33.6 -> 35.2 ms, s20 p = 4, q
+// = 1/4 4.92 -> 5.08; in second-order PageRank's trials 4.87 -> 4.65.)
 template <bool SCAN = false>
 __device__ __forceinline__ bool prev_contains(const DevGraph& g, const Job& J, const StepCtx& c, int32_t u,
                                               uint32_t& probes) {
@@ -701,7 +704,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
                                     : !csplit && UB < __fmul_rn(J.whi1, hk) && UB >= __fmul_rn(J.wlo1, hk)))
                : (pr2 && (rvs || (!split && UB < __fmul_rn(c.w1, hk) && UB >= __fmul_rn(c.w2, hk))))) {
       uint32_t pb = 0;
-      adj = prev_contains(g, J, c, u, pb);
+      adj = prev_contains<ALG == ALGO_PAGERANK2>(g, J, c, u, pb);
       probes += pb;
     }
     if (rvs) {

@@ -736,7 +736,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
           if (p < items) {
             uint32_t pb = 0;
             x = __ldg(g.col + ps + k);
-            pos = row_lookup(g, JW, v, s, s + d, x, pb);
+            pos = row_lookup<true>(g, JW, v, s, s + d, x, pb);  // most x are not in N(v): the filter says so from L2
             if (pos >= 0) {
               h = load_h(g, JW, pos, hsc);
               pos -= s;
