@@ -31,7 +31,22 @@
 namespace fw {
 
 constexpr int kBlock = 256;
-constexpr int kMinBlocks = 4;  // 4 x 256 threads per SM (64 registers; 3, 5 and 6 blocks measured slower)
+// Resident blocks of 256 threads per SM, by kernel variant: 64 registers per
+// thread at 4, 80 at 3, 48 at 5, 40 at 6, 32 at 7.  More warps hide the gathers'
+// latency until the spills cost more.  GB300, ms: node2vec s22 p = 1/4, q = 4
+// 40.0 / 33.9 / 37.5 with 3 / 4 / 5, its trials-together variant (Pareto 1,
+// s20) 50.6 / 42.4 / 41.0; weighted s22 8.57 / 7.21 / 7.04 and 7.43 with 6,
+// for few walkers 0.061 with 4, 0.069 with 5; second-order PageRank s20 4.35
+// / 4.49 / 4.8, its trials-together variant on Pareto 1 24.7 / 22.6 with 3 /
+// 4; metapath 1.55 / 1.33 / 1.65; the scanning variant (node2vec s18) 10.5 /
+// 9.5 / 9.1 / 8.42 / 8.40 with 4 / 5 / 6 / 7 / 8.
+template <int ALG, bool SPREAD, bool SHARE, bool COOP, bool SCAN>
+constexpr int kMinBlocks = SCAN                                       ? 7
+                           : SHARE                                    ? 4
+                           : ALG == ALGO_NODE2VEC && COOP             ? 5
+                           : ALG == ALGO_WEIGHTED && !SPREAD && !COOP ? 5
+                           : ALG == ALGO_PAGERANK2 && (SPREAD || !COOP) ? 3
+                                                                      : 4;
 constexpr int kThreadExactMaxDeg = 16; // exact steps with d <= this run on one lane
 
 // Row writes are staged per lane in shared memory, one aligned group of
@@ -429,8 +444,9 @@ constexpr double kTogetherEnvelope = 5.0, kTogetherPagerank = 2.5;
 // ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
 // is given its first walkers by place, `wpw` per warp; SHARE: hub steps may be
 // shared with the block's idle warps (see hub steps); COOP: long eRJS steps
-// try 32 proposals at once (see trials together).
-template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP>
+// try 32 proposals at once (see trials together); SCAN: every job scans rows
+// (forced eRVS, exact mode) and the eRJS code is left out.
+template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP, bool SCAN>
 __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
@@ -647,11 +663,11 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
           } else if (m == MODE_DEGREE) {
             m = (c.d < kDegreeRuleThreshold) ? MODE_RVS : MODE_RJS;
           }
-          plan = (m == MODE_RJS) ? PLAN_RJS : (((grp ? c.pe - c.ps : c.d) <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W);
+          plan = (!SCAN && m == MODE_RJS) ? PLAN_RJS : (((grp ? c.pe - c.ps : c.d) <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W);
           if (ALG == ALGO_PAGERANK2) {
             split = split && plan == PLAN_RJS;
             sum_common = split;
-          } else if (FW_ALGO(J) == ALGO_NODE2VEC && plan == PLAN_RJS && c.vp >= 0 &&
+          } else if (!SCAN && FW_ALGO(J) == ALGO_NODE2VEC && plan == PLAN_RJS && c.vp >= 0 &&
                      (J.split_return || (J.split_common && (float)(c.pe - c.ps) < dsl))) {
             // the return edge alone sets max(w) = 1/p: propose it separately and
             // bound the other neighbours by max(1, 1/q) * h_MAX[v]; with 1/q < 1 and
@@ -706,7 +722,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     Accept acc;
     acc.rec_ok = false;
     acc.h = -1.0f;
-    if (ALG == ALGO_PAGERANK2) {
+    if (!SCAN && ALG == ALGO_PAGERANK2) {
       const bool find = plan == PLAN_COMMON;
       const int32_t len = widx >= 0 && pick == -2 && (find || sum_common) ? c.pe - c.ps : 0;
       if (__any_sync(kFull, len > 0)) {
@@ -778,7 +794,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     const int32_t lane_rvs = !kLaneRvs ? kLaneNone
                              : plan == PLAN_RVS_T ? kLaneJump
                              : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
-    if (widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
+    if (!SCAN && widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
       const bool rvs = lane_rvs != kLaneNone;
       int32_t nt = J.round, budget = 0x7fffffff;
       if (!rvs && trials + nt >= J.rjs_cap) {
@@ -1074,8 +1090,8 @@ __device__ __forceinline__ void load_jobs(const Job* src_jobs, int njobs, Job* s
 // Single-job (or one-algorithm) launch: one walk loop per warp over the
 // launch's queue.  SHARE: idle warps linger to
 // help the block's hub steps.
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(const __grid_constant__ DevGraph g,
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, bool SCAN = false>
+__global__ void __launch_bounds__(kBlock, (kMinBlocks<ALG, SPREAD, SHARE, COOP, SCAN>)) walk_kernel(const __grid_constant__ DevGraph g,
                                                       const __grid_constant__ JobTableN<NJ> tab, int njobs, long long total,
                                                       int wpw, unsigned long long* __restrict__ qctr,
                                                       unsigned* __restrict__ err, DevCounters* __restrict__ cnt) {
@@ -1093,17 +1109,17 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) walk_kernel(const __grid_c
   __syncthreads();
   LaneCounters lc;
   lc.zero();
-  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE, COOP>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
+  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE, COOP, SCAN>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
   if (SHARE) hub_linger<COUNT, ALG>(g, sj, &hb, lc);
   if (COUNT) flush_counters(lc, cnt);
 }
 
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, bool SCAN = false>
 inline cudaError_t walk_blocks_per_sm(int* out) {
   static std::atomic<int> cached{0};
   int b = cached.load();
   if (b == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP>, kBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP, SCAN>, kBlock, 0);
     if (e != cudaSuccess) return e;
     b = b > 0 ? b : 1;
     cached.store(b);
@@ -1139,7 +1155,7 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // the warp works for one walker at a time anyway, and a warp's lot of 14
 // walkers with hub rows made some warps run long after the others (65,536
 // walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
-// with 1).  Other launches with more walkers than lanes: full warps that
+// with 1; without the eRJS code and with its registers 8.4).  Other launches with more walkers than lanes: full warps that
 // fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
 // full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
@@ -1149,6 +1165,7 @@ struct LaunchShape {
   int grid, wpw;
   bool spread;
   bool share;  // spread, with hub sharing
+  bool scan;   // spread, for jobs that only scan rows: no eRJS code
   bool coop;   // trials together (see the walk loop)
   bool queue;  // needs a zeroed queue counter
 };
@@ -1161,7 +1178,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   if (e != cudaSuccess) return e;
   long long blocks = (long long)g->num_sms * bps;
   s->wpw = 32;
-  s->spread = s->share = s->coop = false;
+  s->spread = s->share = s->coop = s->scan = false;
   bool scans = true, trials = false;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
@@ -1170,11 +1187,12 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   }
   if (!COUNT) {
     s->share = hub_share_pays(g, jobs, njobs, total, blocks * kBlock);
-    // whether it spreads does not depend on coop: both spread kernels have the same occupancy (their launch bounds)
     const bool few = total <= blocks * kBlock;
     s->coop = ALG == ALGO_PAGERANK2 ? !scans && (few || g->envelope >= kTogetherPagerank)
                                     : trials && g->envelope >= kTogetherEnvelope;
+    s->scan = scans && !s->share;
     e = s->share  ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
+        : s->scan ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, true>(&bps)
         : s->coop ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
                   : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
     if (e != cudaSuccess) return e;
@@ -1232,6 +1250,7 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
     kernel<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err, g->d_cnt);
   };
   if (s.share) launch(walk_kernel<NJ, false, ALG, true, true>);
+  else if (s.scan) launch(walk_kernel<NJ, false, ALG, true, false, false, true>);
   else if (s.spread && s.coop) launch(walk_kernel<NJ, false, ALG, true, false, true>);
   else if (s.spread) launch(walk_kernel<NJ, false, ALG, true>);
   else if (s.coop) launch(walk_kernel<NJ, false, ALG, false, false, true>);
@@ -1249,6 +1268,7 @@ inline cudaError_t prime_walk() {
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, true>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, true>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&b);
   return e;
 }
