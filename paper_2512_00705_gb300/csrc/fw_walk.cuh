@@ -444,8 +444,8 @@ constexpr double kTogetherEnvelope = 5.0, kTogetherPagerank = 2.5;
 // ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
 // is given its first walkers by place, `wpw` per warp; SHARE: hub steps may be
 // shared with the block's idle warps (see hub steps); COOP: long eRJS steps
-// try 32 proposals at once (see trials together); SCAN: every job scans rows
-// (forced eRVS, exact mode) and the eRJS code is left out.
+// try 32 proposals at once (see trials together); SCAN: every job is forced
+// eRVS and the other samplers' code is left out.
 template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP, bool SCAN>
 __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
@@ -596,7 +596,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         plan = PLAN_RJS;
       } else {
         int32_t m = J.mode;
-        if (m == MODE_EXACT) {
+        if (!SCAN && m == MODE_EXACT) {
           if (FW_ALGO(J) == ALGO_PAGERANK2 && c.vp >= 0) pagerank2_weights(J, c.d, c.pe - c.ps, c.w1, c.w2);
           plan = (c.d <= kThreadExactMaxDeg) ? PLAN_EXACT_T : PLAN_EXACT_W;
         } else {
@@ -843,7 +843,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       }
       if (COUNT) lc.rvs_steps++;
     }
-    if (widx >= 0 && pick == -2 && plan == PLAN_EXACT_T) {
+    if (!SCAN && widx >= 0 && pick == -2 && plan == PLAN_EXACT_T) {
       const float u = u01(philox(make_uint4(c.wid, (uint32_t)c.step, 0u, 0u), J.key0, J.key1).x);
       ent = exact_pick<1, COUNT, ALG>(g, J, c, 0, u, lc);
       if (COUNT) lc.exact_steps++;
@@ -874,7 +874,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       const Job& JW = sj[jb];
       int32_t k;
       const int32_t hd = (ALG == ALGO_METAPATH && wg) ? w.pe - w.ps : w.d;
-      if (pl == PLAN_EXACT_W) {
+      if (!SCAN && pl == PLAN_EXACT_W) {
         const float u = u01(philox(make_uint4(w.wid, (uint32_t)w.step, 0u, 0u), JW.key0, JW.key1).x);
         k = exact_pick<32, COUNT, ALG>(g, JW, w, lane, u, lc);
       } else if (hd >= kHubMinDeg && hub_chunks(hd) <= kHubMaxChunks) {
@@ -1155,7 +1155,8 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // the warp works for one walker at a time anyway, and a warp's lot of 14
 // walkers with hub rows made some warps run long after the others (65,536
 // walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
-// with 1; without the eRJS code and with its registers 8.4).  Other launches with more walkers than lanes: full warps that
+// with 1; by the eRVS-only
+// variant 8.4; exact mode gained nothing from one of its own).  Other launches with more walkers than lanes: full warps that
 // fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
 // full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
@@ -1165,7 +1166,7 @@ struct LaunchShape {
   int grid, wpw;
   bool spread;
   bool share;  // spread, with hub sharing
-  bool scan;   // spread, for jobs that only scan rows: no eRJS code
+  bool scan;   // spread, for forced eRVS: no other sampler's code
   bool coop;   // trials together (see the walk loop)
   bool queue;  // needs a zeroed queue counter
 };
@@ -1179,10 +1180,11 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   long long blocks = (long long)g->num_sms * bps;
   s->wpw = 32;
   s->spread = s->share = s->coop = s->scan = false;
-  bool scans = true, trials = false;
+  bool scans = true, reservoir = true, trials = false;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
     scans = scans && scan;
+    reservoir = reservoir && jobs[i].mode == MODE_RVS;
     trials = trials || (!scan && jobs[i].weighted);
   }
   if (!COUNT) {
@@ -1190,7 +1192,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     const bool few = total <= blocks * kBlock;
     s->coop = ALG == ALGO_PAGERANK2 ? !scans && (few || g->envelope >= kTogetherPagerank)
                                     : trials && g->envelope >= kTogetherEnvelope;
-    s->scan = scans && !s->share;
+    s->scan = reservoir && !s->share;
     e = s->share  ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
         : s->scan ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, true>(&bps)
         : s->coop ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
