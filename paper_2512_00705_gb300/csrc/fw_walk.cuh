@@ -38,10 +38,13 @@ constexpr int kBlock = 256;
 // s20) 50.6 / 42.4 / 41.0; weighted s22 8.57 / 7.21 / 7.04 and 7.43 with 6,
 // for few walkers 0.061 with 4, 0.069 with 5; second-order PageRank s20 4.35
 // / 4.49 / 4.8, its trials-together variant on Pareto 1 24.7 / 22.6 with 3 /
-// 4; metapath 1.55 / 1.33 / 1.65; the scanning variant (node2vec s18) 10.5 /
-// 9.5 / 9.1 / 8.42 / 8.40 with 4 / 5 / 6 / 7 / 8.
-template <int ALG, bool SPREAD, bool SHARE, bool COOP, bool SCAN>
-constexpr int kMinBlocks = SCAN                                       ? 7
+// 4; metapath 1.55 / 1.33 / 1.65; the eRVS-only variant (node2vec s18) 10.5 /
+// 9.5 / 9.1 / 8.42 / 8.40 with 4 / 5 / 6 / 7 / 8, exact-only (weighted s18)
+// 2.92 / 2.87 / 3.14 / 3.80 with 4 / 5 / 6 / 7.
+enum : int { kAny = 0, kOnlyRvs = 1, kOnlyExact = 2 };  // samplers a kernel variant holds
+template <int ALG, bool SPREAD, bool SHARE, bool COOP, int ONLY>
+constexpr int kMinBlocks = ONLY == kOnlyRvs                           ? 7
+                           : ONLY == kOnlyExact                       ? 5
                            : SHARE                                    ? 4
                            : ALG == ALGO_NODE2VEC && COOP             ? 5
                            : ALG == ALGO_WEIGHTED && !SPREAD && !COOP ? 5
@@ -444,9 +447,9 @@ constexpr double kTogetherEnvelope = 5.0, kTogetherPagerank = 2.5;
 // ALG fixes the algorithm of every job at compile time.  SPREAD: the launch
 // is given its first walkers by place, `wpw` per warp; SHARE: hub steps may be
 // shared with the block's idle warps (see hub steps); COOP: long eRJS steps
-// try 32 proposals at once (see trials together); SCAN: every job is forced
-// eRVS and the other samplers' code is left out.
-template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP, bool SCAN>
+// try 32 proposals at once (see trials together); ONLY: every job is forced
+// eRVS, or every job exact, and the other samplers' code is left out.
+template <int NJ, bool COUNT, int ALG, bool SPREAD, bool SHARE, bool COOP, int ONLY>
 __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int njobs, long long total, int wpw,
                                           unsigned long long* __restrict__ qctr, unsigned* __restrict__ err,
                                           int32_t* obuf, HubBlock* hb, LaneCounters& lc) {
@@ -463,6 +466,8 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   // lanes per warp (5,003 walkers 379 and 538 us); second-order PageRank
   // seldom has such rows and loses the registers (8.46 and 8.80 ms).
   constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC;
+  constexpr bool kTrials = ONLY == kAny, kRvs = ONLY != kOnlyExact;
+  constexpr bool kExact = ONLY == kOnlyExact || (ONLY == kAny && (COUNT || NJ > 1));  // single exact jobs: kOnlyExact
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x;
 
@@ -596,7 +601,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         plan = PLAN_RJS;
       } else {
         int32_t m = J.mode;
-        if (!SCAN && m == MODE_EXACT) {
+        if (ONLY == kOnlyExact || (kExact && m == MODE_EXACT)) {
           if (FW_ALGO(J) == ALGO_PAGERANK2 && c.vp >= 0) pagerank2_weights(J, c.d, c.pe - c.ps, c.w1, c.w2);
           plan = (c.d <= kThreadExactMaxDeg) ? PLAN_EXACT_T : PLAN_EXACT_W;
         } else {
@@ -663,11 +668,11 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
           } else if (m == MODE_DEGREE) {
             m = (c.d < kDegreeRuleThreshold) ? MODE_RVS : MODE_RJS;
           }
-          plan = (!SCAN && m == MODE_RJS) ? PLAN_RJS : (((grp ? c.pe - c.ps : c.d) <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W);
+          plan = (kTrials && m == MODE_RJS) ? PLAN_RJS : (((grp ? c.pe - c.ps : c.d) <= J.lane_max) ? PLAN_RVS_T : PLAN_RVS_W);
           if (ALG == ALGO_PAGERANK2) {
             split = split && plan == PLAN_RJS;
             sum_common = split;
-          } else if (!SCAN && FW_ALGO(J) == ALGO_NODE2VEC && plan == PLAN_RJS && c.vp >= 0 &&
+          } else if (kTrials && FW_ALGO(J) == ALGO_NODE2VEC && plan == PLAN_RJS && c.vp >= 0 &&
                      (J.split_return || (J.split_common && (float)(c.pe - c.ps) < dsl))) {
             // the return edge alone sets max(w) = 1/p: propose it separately and
             // bound the other neighbours by max(1, 1/q) * h_MAX[v]; with 1/q < 1 and
@@ -722,7 +727,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     Accept acc;
     acc.rec_ok = false;
     acc.h = -1.0f;
-    if (!SCAN && ALG == ALGO_PAGERANK2) {
+    if (kTrials && ALG == ALGO_PAGERANK2) {
       const bool find = plan == PLAN_COMMON;
       const int32_t len = widx >= 0 && pick == -2 && (find || sum_common) ? c.pe - c.ps : 0;
       if (__any_sync(kFull, len > 0)) {
@@ -794,7 +799,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
     const int32_t lane_rvs = !kLaneRvs ? kLaneNone
                              : plan == PLAN_RVS_T ? kLaneJump
                              : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
-    if (!SCAN && widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
+    if (kTrials && widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
       const bool rvs = lane_rvs != kLaneNone;
       int32_t nt = J.round, budget = 0x7fffffff;
       if (!rvs && trials + nt >= J.rjs_cap) {
@@ -831,7 +836,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       }
     }
     // ------------------------------------------------------------ single-lane eRVS / exact
-    if (!kLaneRvs && widx >= 0 && pick == -2 && plan == PLAN_RVS_T) {
+    if (kRvs && !kLaneRvs && widx >= 0 && pick == -2 && plan == PLAN_RVS_T) {
       const bool jump = !(J.flags & FW_FLAG_RVS_NOJUMP);
       if ((FW_ALGO(J) == ALGO_METAPATH) && grp) {
         StepCtx cg = c;
@@ -843,7 +848,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       }
       if (COUNT) lc.rvs_steps++;
     }
-    if (!SCAN && widx >= 0 && pick == -2 && plan == PLAN_EXACT_T) {
+    if (kExact && widx >= 0 && pick == -2 && plan == PLAN_EXACT_T) {
       const float u = u01(philox(make_uint4(c.wid, (uint32_t)c.step, 0u, 0u), J.key0, J.key1).x);
       ent = exact_pick<1, COUNT, ALG>(g, J, c, 0, u, lc);
       if (COUNT) lc.exact_steps++;
@@ -874,7 +879,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
       const Job& JW = sj[jb];
       int32_t k;
       const int32_t hd = (ALG == ALGO_METAPATH && wg) ? w.pe - w.ps : w.d;
-      if (!SCAN && pl == PLAN_EXACT_W) {
+      if (!kRvs || (kExact && pl == PLAN_EXACT_W)) {
         const float u = u01(philox(make_uint4(w.wid, (uint32_t)w.step, 0u, 0u), JW.key0, JW.key1).x);
         k = exact_pick<32, COUNT, ALG>(g, JW, w, lane, u, lc);
       } else if (hd >= kHubMinDeg && hub_chunks(hd) <= kHubMaxChunks) {
@@ -1090,8 +1095,8 @@ __device__ __forceinline__ void load_jobs(const Job* src_jobs, int njobs, Job* s
 // Single-job (or one-algorithm) launch: one walk loop per warp over the
 // launch's queue.  SHARE: idle warps linger to
 // help the block's hub steps.
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, bool SCAN = false>
-__global__ void __launch_bounds__(kBlock, (kMinBlocks<ALG, SPREAD, SHARE, COOP, SCAN>)) walk_kernel(const __grid_constant__ DevGraph g,
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, int ONLY = kAny>
+__global__ void __launch_bounds__(kBlock, (kMinBlocks<ALG, SPREAD, SHARE, COOP, ONLY>)) walk_kernel(const __grid_constant__ DevGraph g,
                                                       const __grid_constant__ JobTableN<NJ> tab, int njobs, long long total,
                                                       int wpw, unsigned long long* __restrict__ qctr,
                                                       unsigned* __restrict__ err, DevCounters* __restrict__ cnt) {
@@ -1109,17 +1114,17 @@ __global__ void __launch_bounds__(kBlock, (kMinBlocks<ALG, SPREAD, SHARE, COOP, 
   __syncthreads();
   LaneCounters lc;
   lc.zero();
-  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE, COOP, SCAN>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
+  walk_loop<NJ, COUNT, ALG, SPREAD, SHARE, COOP, ONLY>(g, sj, njobs, total, wpw, qctr, err, obuf, &hb, lc);
   if (SHARE) hub_linger<COUNT, ALG>(g, sj, &hb, lc);
   if (COUNT) flush_counters(lc, cnt);
 }
 
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, bool SCAN = false>
+template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, int ONLY = kAny>
 inline cudaError_t walk_blocks_per_sm(int* out) {
   static std::atomic<int> cached{0};
   int b = cached.load();
   if (b == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP, SCAN>, kBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP, ONLY>, kBlock, 0);
     if (e != cudaSuccess) return e;
     b = b > 0 ? b : 1;
     cached.store(b);
@@ -1155,9 +1160,10 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // the warp works for one walker at a time anyway, and a warp's lot of 14
 // walkers with hub rows made some warps run long after the others (65,536
 // walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
-// with 1; by the eRVS-only
-// variant 8.4; exact mode gained nothing from one of its own).  Other launches with more walkers than lanes: full warps that
-// fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
+// with 1, 8.2 in the variant that holds only eRVS; without exact mode's code
+// the others gain too: metapath s21 1.32 -> 1.31 ms, second-order PageRank
+// s20 4.36 -> 4.24, 5,003 walkers 351 -> 338 us).  Other launches with more
+// walkers than lanes: full warps that fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
 // full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
 // kernel variant of its own, because the same choice made inside the queued
@@ -1166,7 +1172,7 @@ struct LaunchShape {
   int grid, wpw;
   bool spread;
   bool share;  // spread, with hub sharing
-  bool scan;   // spread, for forced eRVS: no other sampler's code
+  int only;    // spread, with one sampler's code
   bool coop;   // trials together (see the walk loop)
   bool queue;  // needs a zeroed queue counter
 };
@@ -1179,12 +1185,14 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   if (e != cudaSuccess) return e;
   long long blocks = (long long)g->num_sms * bps;
   s->wpw = 32;
-  s->spread = s->share = s->coop = s->scan = false;
-  bool scans = true, reservoir = true, trials = false;
+  s->spread = s->share = s->coop = false;
+  s->only = kAny;
+  bool scans = true, reservoir = true, exact = true, trials = false;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
     scans = scans && scan;
     reservoir = reservoir && jobs[i].mode == MODE_RVS;
+    exact = exact && jobs[i].mode == MODE_EXACT;
     trials = trials || (!scan && jobs[i].weighted);
   }
   if (!COUNT) {
@@ -1192,11 +1200,12 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     const bool few = total <= blocks * kBlock;
     s->coop = ALG == ALGO_PAGERANK2 ? !scans && (few || g->envelope >= kTogetherPagerank)
                                     : trials && g->envelope >= kTogetherEnvelope;
-    s->scan = reservoir && !s->share;
-    e = s->share  ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
-        : s->scan ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, true>(&bps)
-        : s->coop ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
-                  : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
+    s->only = s->share ? kAny : reservoir ? kOnlyRvs : exact ? kOnlyExact : kAny;
+    e = s->share                ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
+        : s->only == kOnlyRvs   ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyRvs>(&bps)
+        : s->only == kOnlyExact ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyExact>(&bps)
+        : s->coop               ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
+                                : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
     if (e != cudaSuccess) return e;
     const long long spread_blocks = (long long)g->num_sms * bps;
     s->spread = scans || total <= spread_blocks * kBlock;
@@ -1252,7 +1261,8 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
     kernel<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err, g->d_cnt);
   };
   if (s.share) launch(walk_kernel<NJ, false, ALG, true, true>);
-  else if (s.scan) launch(walk_kernel<NJ, false, ALG, true, false, false, true>);
+  else if (s.only == kOnlyRvs) launch(walk_kernel<NJ, false, ALG, true, false, false, kOnlyRvs>);
+  else if (s.only == kOnlyExact) launch(walk_kernel<NJ, false, ALG, true, false, false, kOnlyExact>);
   else if (s.spread && s.coop) launch(walk_kernel<NJ, false, ALG, true, false, true>);
   else if (s.spread) launch(walk_kernel<NJ, false, ALG, true>);
   else if (s.coop) launch(walk_kernel<NJ, false, ALG, false, false, true>);
@@ -1270,7 +1280,8 @@ inline cudaError_t prime_walk() {
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, true>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, true>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyRvs>(&b);
+  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyExact>(&b);
   if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&b);
   return e;
 }
