@@ -70,14 +70,10 @@ static void create_counter_pool(fw_graph* g) {
   cudaMemPoolSetAttribute(g->counter_pool, cudaMemPoolAttrReleaseThreshold, &keep);
 }
 
-static cudaError_t alloc_scratch(const fw_graph* g, size_t bytes, unsigned long long** out, cudaStream_t st) {
-  void** p = reinterpret_cast<void**>(out);
-  return g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
-}
-
 cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t st) {
   const size_t bytes = sizeof(unsigned long long) * (size_t)count;
-  cudaError_t e = alloc_scratch(g, bytes, out, st);
+  void** p = reinterpret_cast<void**>(out);
+  cudaError_t e = g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(*out, 0, bytes, st);
   if (e != cudaSuccess) cudaFreeAsync(*out, st);
@@ -202,7 +198,7 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   const int64_t e = g->e;
   int* d_maxdeg = reinterpret_cast<int*>(g->d_err) + 6;
   unsigned* d_asym = g->d_err + 7;
-  unsigned* d_lbad = g->d_err + 13;
+  unsigned* d_lbad = g->d_err + 1;
   double* d_mass = reinterpret_cast<double*>(g->d_err) + 4;
   unsigned long long* d_sides = reinterpret_cast<unsigned long long*>(g->d_err) + 1;
   const bool want_labels = g->d_lab != nullptr && !g->lstat_bad;
@@ -235,18 +231,21 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
     cudaError_t pe = prime_preprocess_kernels();
     if (pe != cudaSuccess) return cuda_error(pe, "load preprocessing kernels");
   }
-  unsigned long long* scratch = nullptr;  // the row lists
-  {
-    cudaError_t ae = alloc_scratch(g, sizeof(int32_t) * row_list_words(e), &scratch, st);
-    if (ae != cudaSuccess) return cuda_error(ae, "row lists");
+  if (!g->d_rows) {
+    cudaError_t ae = cudaMalloc(&g->d_rows, sizeof(int32_t) * row_list_words(e));
+    if (ae != cudaSuccess) {
+      g->d_rows = nullptr;
+      return cuda_error(ae, "cudaMalloc(row lists)");
+    }
+    g->bytes += sizeof(int32_t) * row_list_words(e);
   }
-  const RowLists rows = row_lists(reinterpret_cast<int32_t*>(scratch), e);
+  const RowLists rows = row_lists(g->d_rows, e);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // one memset over the words these kernels use: sides (2..5), max degree (6), asymmetry (7), envelope mass and
-  // weight (8..11), bad label (13)
-  cudaError_t le = cudaMemsetAsync(g->d_err + 2, 0, 12 * sizeof(unsigned), st);
+  // one memset over the words these kernels use: bad label (1), sides (2..5), max degree (6), asymmetry (7),
+  // envelope mass, weight and squared lengths (8..13)
+  cudaError_t le = cudaMemsetAsync(g->d_err + 1, 0, 13 * sizeof(unsigned), st);
   if (le == cudaSuccess) le = cudaMemsetAsync(rows.counts, 0, 2 * sizeof(int), st);
   cudaEventRecord(e0, st);
   if (le == cudaSuccess)
@@ -273,14 +272,12 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   if (le != cudaSuccess) fs = cuda_error(le, "preprocessing kernels");
   else if (ce != cudaSuccess) fs = cuda_error(ce, "read preprocessing results");
   else if (se != cudaSuccess) fs = cuda_error(se, "sync after preprocessing");
-  if (fs != FW_OK) {
-    cudaFreeAsync(scratch, st);
-    return fs;
-  }
+  if (fs != FW_OK) return fs;
   const int maxdeg = (int)words[6];
-  double mass[2];
+  double mass[3];
   std::memcpy(mass, words + 8, sizeof(mass));
   g->envelope = mass[1] > 0.0 ? mass[0] / mass[1] : 1.0;
+  g->mean_row = e > 0 ? mass[2] / (double)e : 0.0;
   g->max_degree = maxdeg;
   g->sym = words[7] == 0 && words[2] == words[4] && words[3] == words[5] ? 1 : 0;
   if (g->d_cerec && maxdeg >= (1 << 24)) {  // edge records carry class counts in 24 bits
@@ -288,7 +285,7 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
     g->d_cerec = nullptr;
     g->bytes -= 2 * sizeof(int4) * (size_t)e;
   }
-  if (want_labels && words[13] != 0) {  // a label >= kLabelStats: per-label statistics unused
+  if (want_labels && words[1] != 0) {  // a label >= kLabelStats: per-label statistics unused
     cudaFree(g->d_lstat);
     g->d_lstat = nullptr;
     g->bytes -= sizeof(float2) * kLabelStats * ((size_t)n + 1);
@@ -296,7 +293,6 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   }
   g->preprocess_ms += ms;
   if (g->d_lstat && e > 0) fs = build_label_groups(g, rows, st);
-  cudaFreeAsync(scratch, st);
   return fs;
 }
 
@@ -389,6 +385,7 @@ static void free_graph(fw_graph* g) {
   cudaFree(g->d_lrec);
   cudaFree(g->d_gerec);
   cudaFree(g->d_gh);
+  cudaFree(g->d_rows);
   cudaFree(g->d_err);
   cudaFree(g->d_cnt);
   cudaFree(g->d_stage_starts);

@@ -40,7 +40,9 @@ struct fw_graph {
   uint8_t* d_h8 = nullptr;    // 8-bit weight codes after fw_graph_quantize_weights
   float* d_h8scale = nullptr; // per node: the scale of its row's codes
   float hscale = 0.0f;        // the largest per-node scale (reported by fw_graph_info)
+  int32_t* d_rows = nullptr;  // lists of the long rows (RowLists), for the preprocessing kernels
   int32_t sym = 0;
+  double mean_row = 0.0;      // mean length of a row met by following an entry (a choice of launch shape only)
   double envelope = 1.0;      // eRJS envelope mass per unit of weight, over all rows (a choice of launch variant only)
   unsigned* d_err = nullptr;
   fw::DevCounters* d_cnt = nullptr;
@@ -117,7 +119,7 @@ size_t row_list_words(long long e);                      // int32 words of scrat
 RowLists row_lists(int32_t* scratch, long long e);       // lay them out (the counts come first)
 
 // Also fills `rows` (counts zeroed before) and adds up the eRJS envelope mass
-// and the weight of all rows in mass[0], mass[1].
+// and the weight of all rows and the squares of their lengths in mass[0 .. 2].
 cudaError_t launch_node_stats(const int32_t* off, const float* h, int32_t n, float* hmax, float* hsum, int4* nrec,
                               int* maxdeg, const RowLists& rows, double* mass, int num_sms, cudaStream_t stream);
 cudaError_t launch_edge_records(const int32_t* off, const int32_t* col, const float* h, const uint8_t* lab,

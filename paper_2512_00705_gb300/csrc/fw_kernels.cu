@@ -56,7 +56,7 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   int localmax = 0;
-  double envelope = 0.0, weight = 0.0;  // over the warp's rows: (4 n0 + 2 n1 + n2) / 4 * h_MAX, and h_SUM
+  double envelope = 0.0, weight = 0.0, squares = 0.0;  // over the warp's rows: (4 n0 + 2 n1 + n2) / 4 * h_MAX, h_SUM, d^2
   for (long long v = warp; v < n; v += nwarps) {
     const int32_t s = off[v], e = off[v + 1];
     float m = 0.0f, sum = 0.0f;
@@ -103,15 +103,17 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     localmax = max(localmax, e - s);
     envelope += 0.25 * (double)(e - s + 3ll * n0 + n1) * (double)m;
     weight += (double)sum;
+    squares += (double)(e - s) * (double)(e - s);
   }
   if (lane == 0 && localmax > 0) atomicMax(maxdeg, localmax);
-  __shared__ double part[2][8];
+  __shared__ double part[3][8];
   if (lane == 0) {
     part[0][threadIdx.x >> 5] = envelope;
     part[1][threadIdx.x >> 5] = weight;
+    part[2][threadIdx.x >> 5] = squares;
   }
   __syncthreads();
-  if (threadIdx.x < 2) {
+  if (threadIdx.x < 3) {
     double x = 0.0;
     for (int w = 0; w < 8; ++w) x += part[threadIdx.x][w];
     atomicAdd(mass + threadIdx.x, x);

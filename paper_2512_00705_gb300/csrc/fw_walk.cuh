@@ -1156,7 +1156,8 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // spread over the resident warps before they share one -- wpw is the
 // smallest count with which they fit, and blocks fill before warps do.  No
 // queue counter is needed then.  Jobs that only scan rows (forced eRVS,
-// exact mode) keep one walker per warp at every size, the rest in the queue:
+// exact mode) keep one walker per warp at every size (eight where the rows
+// are short, see kShortScan), the rest in the queue:
 // the warp works for one walker at a time anyway, and a warp's lot of 14
 // walkers with hub rows made some warps run long after the others (65,536
 // walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
@@ -1168,6 +1169,14 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
 // kernel variant of its own, because the same choice made inside the queued
 // kernel's fetch cost the whole-graph walks 1 to 3 %.
+// Where eRVS rows are short (mean row of a walk below kShortScan; metapath: of
+// a label's share of it), most of them are their lane's own work and eight
+// walkers go to a warp.  60,000 walkers x 10 hops, 1 / 8 walkers per warp
+// (us): mean row 79 weighted 531 / 366, node2vec 876 / 624, metapath 312 /
+// 143; 142: 601 / 500, 1,018 / 901, 317 / 168; 241: 775 / 697, 1,243 / 1,280,
+// 429 / 255; 430: 995 / 1,009, 1,855 / 2,190, 372 / 225; 1,246: 1,793 /
+// 2,573, 4,051 / 5,364, 557 / 490.
+constexpr double kShortScan = 250.0;
 struct LaunchShape {
   int grid, wpw;
   bool spread;
@@ -1187,6 +1196,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   s->wpw = 32;
   s->spread = s->share = s->coop = false;
   s->only = kAny;
+  const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
   bool scans = true, reservoir = true, exact = true, trials = false;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
@@ -1212,7 +1222,8 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     s->share = s->share && s->spread;
     if (s->spread) {
       blocks = spread_blocks;
-      s->wpw = scans ? 1 : (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
+      s->wpw = (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
+      if (scans) s->wpw = std::min(s->wpw, reservoir && scanned < kShortScan ? 8 : 1);
     }
   }
   if (!s->spread && s->coop) {
