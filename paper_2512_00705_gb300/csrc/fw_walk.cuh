@@ -41,7 +41,8 @@ constexpr int kBlock = 256;
 // 4; metapath 1.55 / 1.33 / 1.65; the eRVS-only variant (node2vec s18) 10.5 /
 // 9.5 / 9.1 / 8.42 / 8.40 with 4 / 5 / 6 / 7 / 8, exact-only (weighted s18)
 // 2.92 / 2.87 / 3.14 / 3.80 with 4 / 5 / 6 / 7.
-enum : int { kAny = 0, kOnlyRvs = 1, kOnlyExact = 2 };  // samplers a kernel variant holds
+// samplers a kernel variant holds (kWhole: all, short eRVS rows scanned at once, see kLaneRvs)
+enum : int { kAny = 0, kOnlyRvs = 1, kOnlyExact = 2, kWhole = 3 };
 template <int ALG, bool SPREAD, bool SHARE, bool COOP, int ONLY>
 constexpr int kMinBlocks = ONLY == kOnlyRvs                           ? 7
                            : ONLY == kOnlyExact                       ? 5
@@ -465,9 +466,9 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   // once, 7.64 in step; metapath 1.32 and 1.40 ms); so are launches with few
   // lanes per warp (5,003 walkers 379 and 538 us); second-order PageRank
   // seldom has such rows and loses the registers (8.46 and 8.80 ms).
-  constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC;
-  constexpr bool kTrials = ONLY == kAny, kRvs = ONLY != kOnlyExact;
-  constexpr bool kExact = ONLY == kOnlyExact || (ONLY == kAny && (COUNT || NJ > 1));  // single exact jobs: kOnlyExact
+  constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC && ONLY != kWhole;
+  constexpr bool kTrials = ONLY == kAny || ONLY == kWhole, kRvs = ONLY != kOnlyExact;
+  constexpr bool kExact = ONLY == kOnlyExact || (kTrials && (COUNT || NJ > 1));  // single exact jobs: kOnlyExact
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x;
 
@@ -1169,6 +1170,12 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
 // kernel variant of its own, because the same choice made inside the queued
 // kernel's fetch cost the whole-graph walks 1 to 3 %.
+// Below this cost ratio, as tuning picks it, eRVS steps are rare and node2vec
+// keeps whole scans, as the code of scans in step costs the trials registers:
+// in step / whole (ms), s22 p = 1/4, q = 4 at r = 1/4 26.6 / 24.1, 1 27.2 /
+// 25.1, 1.5 28.0 / 27.6, 2 28.9 / 30.0, 4 33.7 / 40.8; s20 p = 4, q = 1/4 at
+// r = 1/4 4.80 / 4.20, 1 3.67 / 3.63, 1.5 3.90 / 4.05, 2 4.17 / 4.53.
+constexpr float kRareRatio = 1.5f;
 // Where eRVS rows are short (mean row of a walk below kShortScan; metapath: of
 // a label's share of it), most of them are their lane's own work and eight
 // walkers go to a warp.  60,000 walkers x 10 hops, 1 / 8 walkers per warp
@@ -1197,13 +1204,14 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   s->spread = s->share = s->coop = false;
   s->only = kAny;
   const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
-  bool scans = true, reservoir = true, exact = true, trials = false;
+  bool scans = true, reservoir = true, exact = true, trials = false, rare = true;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
     scans = scans && scan;
     reservoir = reservoir && jobs[i].mode == MODE_RVS;
     exact = exact && jobs[i].mode == MODE_EXACT;
     trials = trials || (!scan && jobs[i].weighted);
+    rare = rare && (jobs[i].mode == MODE_RJS || (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
   }
   if (!COUNT) {
     s->share = hub_share_pays(g, jobs, njobs, total, blocks * kBlock);
@@ -1226,6 +1234,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
       if (scans) s->wpw = std::min(s->wpw, reservoir && scanned < kShortScan ? 8 : 1);
     }
   }
+  if (!COUNT && ALG == ALGO_NODE2VEC && !s->spread && !s->coop && rare) s->only = kWhole;  // the same occupancy as kAny
   if (!s->spread && s->coop) {
     e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&bps);
     if (e != cudaSuccess) return e;
@@ -1247,11 +1256,12 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
 // launches, bound by latency, 0.369 / 0.331 / 0.326 and 0.318 with 4 (5,003
 // walkers), 57 / 48 / 46 and 45 with 4 (Pareto weights).  Queues of several
 // jobs mix lanes of q < 1 and q > 1 in a warp and keep 2 (64 mixed jobs: 8.54
-// ms, with 1 for q < 1 8.96).
-inline int32_t round_trials(const Job& J, bool spread, int njobs) {
+// ms, with 1 for q < 1 8.96); so do launches of whole scans (p = 4, q = 1/4, r
+// = 1/4 4.20, with 1 4.28).
+inline int32_t round_trials(const Job& J, bool spread, int only, int njobs) {
   if (J.round > 0) return J.round;
   if (spread || J.algo == ALGO_PAGERANK2) return 4;
-  if (njobs == 1 && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
+  if (njobs == 1 && only != kWhole && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
   return kRjsBatchDefault;
 }
 
@@ -1266,7 +1276,7 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
   JobTableN<NJ> tab;
   for (int i = 0; i < njobs; ++i) {
     tab.jobs[i] = jobs[i];
-    tab.jobs[i].round = round_trials(jobs[i], s.spread, njobs);
+    tab.jobs[i].round = round_trials(jobs[i], s.spread, s.only, njobs);
   }
   auto launch = [&](auto kernel) {
     kernel<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err, g->d_cnt);
@@ -1277,6 +1287,7 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
   else if (s.spread && s.coop) launch(walk_kernel<NJ, false, ALG, true, false, true>);
   else if (s.spread) launch(walk_kernel<NJ, false, ALG, true>);
   else if (s.coop) launch(walk_kernel<NJ, false, ALG, false, false, true>);
+  else if (ALG == ALGO_NODE2VEC && s.only == kWhole) launch(walk_kernel<NJ, false, ALG, false, false, false, ALG == ALGO_NODE2VEC ? kWhole : kAny>);
   else launch(walk_kernel<NJ, COUNT, ALG>);
   g_launches.fetch_add(1);
   return cudaGetLastError();

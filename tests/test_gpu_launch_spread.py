@@ -110,3 +110,14 @@ def test_scanning_jobs_queue_behind_one_walker_per_warp(walks, mode):
     a = G.walk(dev, 6, "node2vec", p=2.0, q=0.5, mode=mode, seed=9)
     b = G.walk(dev, 6, "node2vec", p=2.0, q=0.5, mode=mode, seed=9, flags=fw.FLAG_COUNTERS)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("mode,shape", [("auto", {"cost_ratio": 0.5}), ("rjs", {"rjs_cap": 3}), ("auto", {"cost_ratio": 1.5})])
+@pytest.mark.parametrize("p,q", [(2.0, 0.5), (0.25, 4.0)])
+def test_whole_scans_of_rare_reservoir_steps(walks, mode, shape, p, q):
+    """node2vec queues with a small cost ratio scan short rows at once, the counting build one position per trial."""
+    g, G, lanes, starts = walks
+    dev = torch.from_numpy(starts).cuda()
+    a = G.walk(dev, 4, "node2vec", p=p, q=q, mode=mode, seed=5, **shape)
+    b = G.walk(dev, 4, "node2vec", p=p, q=q, mode=mode, seed=5, flags=fw.FLAG_COUNTERS, **shape)
+    assert torch.equal(a, b)
