@@ -501,6 +501,20 @@ constexpr int32_t kLaneKeyedMax = 32;
 // [0, S_C), and the neighbour is still to be found.
 constexpr int32_t kPickCommon = -3;
 
+// Trials after which an eRJS step goes to eRVS: the caller's cap, or
+// (default) as many trials as the scan of `entries` they stand in for would
+// cost under the cost model, entries / r, times the budget scale, and at
+// least rjs_cap; whole batches of trials.  A cap may be any positive int32:
+// rounded up in unsigned arithmetic and held at kNoTrialBudget.
+constexpr int32_t kNoTrialBudget = 0x7fffffff;
+
+__device__ __forceinline__ int32_t trial_budget(const Job& J, int32_t entries) {
+  const int32_t cap =
+      J.fixed_cap ? J.rjs_cap : max(J.rjs_cap, (int32_t)fminf(ceilf(J.budget * (float)entries / J.ratio), 1.0e9f));
+  const uint32_t batch = (uint32_t)J.rjs_batch;
+  return (int32_t)min(((uint32_t)cap + batch - 1u) / batch * batch, (uint32_t)kNoTrialBudget);
+}
+
 // One eRJS acceptance: the neighbour position, the node, its effective
 // property weight, and the target's node record (rec_ok = 0: unknown).
 struct Accept {

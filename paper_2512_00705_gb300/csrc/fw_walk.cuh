@@ -802,15 +802,9 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
                              : (plan == PLAN_RVS_W && c.d <= kLaneKeyedMax) ? kLaneKeyed : kLaneNone;
     if (kTrials && widx >= 0 && pick == -2 && (plan == PLAN_RJS || lane_rvs != kLaneNone)) {
       const bool rvs = lane_rvs != kLaneNone;
-      int32_t nt = J.round, budget = 0x7fffffff;
-      if (!rvs && trials + nt >= J.rjs_cap) {
-        // trial budget: the cap, or (default) as many trials as the eRVS scan
-        // they stand in for would cost under the cost model, d / r, times the
-        // budget scale; whole batches of trials
-        const int32_t dd = grp ? c.pe - c.ps : c.d;  // entries the eRVS hand-off would scan
-        const int32_t cap =
-            J.fixed_cap ? J.rjs_cap : max(J.rjs_cap, (int32_t)fminf(ceilf(J.budget * (float)dd / J.ratio), 1.0e9f));
-        budget = (cap + J.rjs_batch - 1) / J.rjs_batch * J.rjs_batch;
+      int32_t nt = J.round, budget = kNoTrialBudget;
+      if (!rvs && nt >= J.rjs_cap - trials) {  // every budget is at least rjs_cap
+        budget = trial_budget(J, grp ? c.pe - c.ps : c.d);
         nt = min(nt, budget - trials);
       }
       if (rjs_trials<COUNT, ALG, kLaneRvs>(g, J, c, B, split, beta, pos_ret, h_ret, trials, nt, acc, lc, csplit, beta2,
@@ -944,9 +938,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         int32_t wpos = __shfl_sync(kFull, pos_ret, src);
         const int fl = __shfl_sync(kFull, (split ? 1 : 0) | (csplit ? 2 : 0) | (grp ? 4 : 0), src);
         const int32_t dd = (fl & 4) ? w.pe - w.ps : w.d;
-        const int32_t cap =
-            JW.fixed_cap ? JW.rjs_cap : max(JW.rjs_cap, (int32_t)fminf(ceilf(JW.budget * (float)dd / JW.ratio), 1.0e9f));
-        const int32_t budget = (cap + JW.rjs_batch - 1) / JW.rjs_batch * JW.rjs_batch;
+        const int32_t budget = trial_budget(JW, dd);
         int32_t t = __shfl_sync(kFull, trials, src);
         unsigned hit = 0;
         Accept wa;
@@ -957,11 +949,11 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
         wa.rec = make_int4(0, 0, 0, 0);
         wa.rec_n0 = wa.rec_n1 = 0;
         while (hit == 0u && t < budget) {
-          const bool got = t + lane < budget &&
+          const bool got = lane < budget - t &&
                            rjs_trials<COUNT, ALG, false>(g, JW, w, wB, (fl & 1) != 0, wbeta, wpos, wh, t + lane, 1, wa, lc,
                                                          (fl & 2) != 0, wbeta2, (fl & 4) != 0);
           hit = __ballot_sync(kFull, got);
-          t += 32;
+          t += min(32, budget - t);
         }
         const int win = hit ? __ffs(hit) - 1 : 0;
         wa.k = __shfl_sync(kFull, wa.k, win);
