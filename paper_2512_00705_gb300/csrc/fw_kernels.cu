@@ -7,6 +7,7 @@
 #include <cstring>
 
 #include "fw_internal.h"
+#include "fw_rows.h"
 #include "fw_walk.cuh"
 
 namespace fw {
@@ -61,11 +62,11 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     const int32_t s = off[v], e = off[v + 1];
     float m = 0.0f, sum = 0.0f;
     if (h) {
-      for (int32_t i = s + lane; i < e; i += 32) {
+      for_entries(s, e - s, lane, 32, [&](int32_t i) {
         const float x = h[i];
         m = fmaxf(m, x);
         sum += x;
-      }
+      });
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
@@ -81,11 +82,11 @@ __global__ void node_stats_kernel(const int32_t* __restrict__ off, const float* 
     if (h) {
       const float half = 0.5f * m, quarter = 0.25f * m;
       n0 = 0;
-      for (int32_t i = s + lane; i < e; i += 32) {
+      for_entries(s, e - s, lane, 32, [&](int32_t i) {
         const float x = h[i];
         n0 += (x > half) ? 1 : 0;
         n1 += (x > quarter && !(x > half)) ? 1 : 0;
-      }
+      });
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         n0 += __shfl_xor_sync(kFull, n0, o);
@@ -153,11 +154,11 @@ __global__ void quantize_rows_kernel(const int32_t* __restrict__ off, float* __r
     const float sv = __fdiv_rn(hmax[v], 255.0f);
     if (lane == 0) scales[v] = sv;
     m = max(m, __float_as_uint(sv));
-    for (int32_t i = off[v] + lane; i < off[v + 1]; i += 32) {
+    for_entries(off[v], off[v + 1] - off[v], lane, 32, [&](int32_t i) {
       const float c = fminf(255.0f, fmaxf(1.0f, rintf(__fdiv_rn(h[i], sv))));
       codes[i] = (uint8_t)c;
       h[i] = __fmul_rn(c, sv);
-    }
+    });
   }
   if (lane == 0 && m) atomicMax(maxbits, m);
 }

@@ -11,6 +11,7 @@
 // listed by the node statistics' pass: 4.2 ms on the same graph.  Every stable
 // order is kept: a team's warps own consecutive segments of the row.
 #include "fw_internal.h"
+#include "fw_rows.h"
 
 namespace fw {
 
@@ -114,11 +115,11 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
       quarter = 0.25f * m;
       if (NW > 1) {
         int c0 = 0, c1 = 0;
-        for (int32_t i = lo + lane; i < hi; i += 32) {
-          const float x = h[s + i];
+        for_entries(s + lo, hi - lo, lane, 32, [&](int32_t i) {
+          const float x = h[i];
           c0 += x > half ? 1 : 0;
           c1 += x > quarter && !(x > half) ? 1 : 0;
-        }
+        });
         c0 = __reduce_add_sync(kFull, c0);
         c1 = __reduce_add_sync(kFull, c1);
         if (lane == 0) {
@@ -134,8 +135,8 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
       run1 += nc.x;
       run2 += nc.x + nc.y;
     }
-    for (int32_t b = lo; b < hi; b += 32) {
-      const bool valid = b + lane < hi;
+    for (uint32_t b = lo; b < (uint32_t)hi; b += 32) {
+      const bool valid = b + lane < (uint32_t)hi;
       const long long i = (long long)s + b + lane;
       float x = 1.0f;
       int4 a = make_int4(0, 0, 0, 0), r = a;
@@ -186,14 +187,15 @@ __global__ void __launch_bounds__(kTeamBlock)
     for (int k = 0; k < kPer; ++k) mx[k] = sm[k] = 0.0f;
     bool over = false;
     constexpr int kAhead = NW == 1 ? 1 : 8;
-    for (int32_t b = lane; b < d; b += 32 * kAhead) {
+    for (uint32_t b = lane; b < (uint32_t)d; b += 32 * kAhead) {
       int l[kAhead];
       float x[kAhead];
 #pragma unroll
       for (int q = 0; q < kAhead; ++q) {
-        const int32_t i = b + 32 * q;
-        l[q] = i < d ? (int)lab[s + i] : -1;
-        x[q] = i < d && h ? h[s + i] : 1.0f;
+        const bool valid = b + 32 * q < (uint32_t)d;
+        const long long i = (long long)s + b + 32 * q;
+        l[q] = valid ? (int)lab[i] : -1;
+        x[q] = valid && h ? h[i] : 1.0f;
       }
 #pragma unroll
       for (int q = 0; q < kAhead; ++q) {
@@ -285,8 +287,8 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
     };
     for (int q = lane; q < kB; q += 32) mine[q] = 0;
     __syncwarp();
-    for (int32_t b = lo; b < hi; b += 32) {
-      const bool valid = b + lane < hi;
+    for (uint32_t b = lo; b < (uint32_t)hi; b += 32) {
+      const bool valid = b + lane < (uint32_t)hi;
       const long long i = (long long)s + b + lane;
       const int k = bucket(valid ? (int)lab[i] : 0, valid && h ? h[i] : 1.0f, valid);
       const unsigned same = __match_any_sync(kFull, k);
@@ -342,8 +344,8 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
       }
     }
     team_sync<NW>();
-    for (int32_t b = lo; b < hi; b += 32) {
-      const bool valid = b + lane < hi;
+    for (uint32_t b = lo; b < (uint32_t)hi; b += 32) {
+      const bool valid = b + lane < (uint32_t)hi;
       const long long i = (long long)s + b + lane;
       const float x = valid && h ? h[i] : 1.0f;
       int4 nr = make_int4(0, 0, 0, 0);
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
       __syncwarp();
       if (valid) {
         const long long o = (long long)s + at;
-        st_record(gerec + 2 * o, make_int4(u, __float_as_int(x), nr.x, nr.y), make_int4(nr.z, nr.w, b + lane, 0));
+        st_record(gerec + 2 * o, make_int4(u, __float_as_int(x), nr.x, nr.y), make_int4(nr.z, nr.w, (int)(b + lane), 0));
         gh[o] = x;
       }
     }
@@ -403,11 +405,11 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
     uint32_t* bits = filter_here ? counts + tnb : gfilter;  // global filters were cleared before
     for (uint32_t i = t; i < (count_here ? tnb + (filter_here ? fw : 0u) : 0u); i += NW * 32) counts[i] = 0u;
     team_sync<NW>();
-    for (int32_t i = s + t; i < e; i += NW * 32) {
+    for_entries(s, d, t, NW * 32, [&](int32_t i) {
       const int32_t u = col[i];
       const uint32_t hk = id_hash((uint32_t)u);
       atomicOr(bits + bloom_word(hk, fw), bloom_bits(hk));
-      if (!table) continue;
+      if (!table) return;
       // d < 8 * tnb ids share the row's buckets, so a free slot exists
       uint32_t b = __umulhi(hk, tnb);
       bool placed = false;
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
         }
         b = (b + 1 == tnb) ? 0u : b + 1;
       }
-    }
+    });
     team_sync<NW>();
     if (filter_here) {
       for (uint32_t i = t; i < fw; i += NW * 32) gfilter[i] = bits[i];
@@ -448,19 +450,19 @@ __global__ void __launch_bounds__(NW == 32 ? 1024 : kTeamBlock)
   unsigned long long taken = 0, left = 0;
   bool missing = false;
   for_rows<NW>(off, n, rows, 1, [&](int32_t v, int32_t s, int32_t d) {
-    for (int32_t i = s + t; i < s + d; i += NW * 32) {
+    for_entries(s, d, t, NW * 32, [&](int32_t i) {
       const int32_t u = col[i];
-      if (u == v) continue;  // its own mirror
+      if (u == v) return;  // its own mirror
       const int32_t us = off[u], ue = off[u + 1];
       if (ue - us > d || (ue - us == d && u > v)) {
         ++left;
-        continue;
+        return;
       }
       ++taken;
       uint32_t pb = 0;
       const int32_t j = row_find(col, us, ue, v, n, pb);
       missing |= j < 0 || (h && h[j] != h[i]);
-    }
+    });
   });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
