@@ -1112,15 +1112,50 @@ __global__ void __launch_bounds__(kBlock, (kMinBlocks<ALG, SPREAD, SHARE, COOP, 
   if (COUNT) flush_counters(lc, cnt);
 }
 
-template <int NJ, bool COUNT, int ALG, bool SPREAD = false, bool SHARE = false, bool COOP = false, int ONLY = kAny>
-inline cudaError_t walk_blocks_per_sm(int* out) {
-  static std::atomic<int> cached{0};
-  int b = cached.load();
+// The kernel variants of one algorithm.  A launch takes its kernel, its
+// occupancy and its priming from this one list, so that none of them can be
+// first loaded inside a stream capture or a served wave.
+enum WalkVariant : int {
+  V_COUNTING = 0,     // queued, with the counters
+  V_QUEUED,           // full warps that fetch from the queue
+  V_QUEUED_TOGETHER,  // the same, with trials together
+  V_QUEUED_WHOLE,     // the same, short eRVS rows scanned at once (node2vec; elsewhere V_QUEUED does that)
+  V_SPREAD,           // walkers given by place
+  V_SPREAD_TOGETHER,  // the same, with trials together
+  V_SPREAD_SHARE,     // the same, with hub sharing
+  V_SPREAD_RVS,       // forced eRVS only
+  V_SPREAD_EXACT,     // exact mode only
+  kWalkVariants
+};
+
+template <int NJ>
+using WalkKernel = void (*)(DevGraph, JobTableN<NJ>, int, long long, int, unsigned long long*, unsigned*, DevCounters*);
+
+template <int NJ, int ALG>
+inline WalkKernel<NJ> walk_variant(int v) {
+  switch (v) {
+    case V_COUNTING: return walk_kernel<NJ, true, ALG>;
+    case V_QUEUED_TOGETHER: return walk_kernel<NJ, false, ALG, false, false, true>;
+    case V_QUEUED_WHOLE: return walk_kernel<NJ, false, ALG, false, false, false, ALG == ALGO_NODE2VEC ? kWhole : kAny>;
+    case V_SPREAD: return walk_kernel<NJ, false, ALG, true>;
+    case V_SPREAD_TOGETHER: return walk_kernel<NJ, false, ALG, true, false, true>;
+    case V_SPREAD_SHARE: return walk_kernel<NJ, false, ALG, true, true>;
+    case V_SPREAD_RVS: return walk_kernel<NJ, false, ALG, true, false, false, kOnlyRvs>;
+    case V_SPREAD_EXACT: return walk_kernel<NJ, false, ALG, true, false, false, kOnlyExact>;
+    default: return walk_kernel<NJ, false, ALG>;
+  }
+}
+
+// Resident blocks per SM of a variant; the first call loads its kernel.
+template <int NJ, int ALG>
+inline cudaError_t walk_blocks_per_sm(int v, int* out) {
+  static std::atomic<int> cached[kWalkVariants];
+  int b = cached[v].load();
   if (b == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_kernel<NJ, COUNT, ALG, SPREAD, SHARE, COOP, ONLY>, kBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, walk_variant<NJ, ALG>(v), kBlock, 0);
     if (e != cudaSuccess) return e;
     b = b > 0 ? b : 1;
-    cached.store(b);
+    cached[v].store(b);
   }
   *out = b;
   return cudaSuccess;
@@ -1177,24 +1212,15 @@ constexpr float kRareRatio = 1.5f;
 // 2,573, 4,051 / 5,364, 557 / 490.
 constexpr double kShortScan = 250.0;
 struct LaunchShape {
+  int variant;  // WalkVariant
   int grid, wpw;
-  bool spread;
-  bool share;  // spread, with hub sharing
-  int only;    // spread, with one sampler's code
-  bool coop;   // trials together (see the walk loop)
   bool queue;  // needs a zeroed queue counter
 };
 
-template <int NJ, bool COUNT, int ALG>
-inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, LaunchShape* s) {
+template <int NJ, int ALG>
+inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+                              LaunchShape* s) {
   constexpr int kWarps = kBlock / 32;
-  int bps = 1;
-  cudaError_t e = walk_blocks_per_sm<NJ, COUNT, ALG>(&bps);
-  if (e != cudaSuccess) return e;
-  long long blocks = (long long)g->num_sms * bps;
-  s->wpw = 32;
-  s->spread = s->share = s->coop = false;
-  s->only = kAny;
   const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
   bool scans = true, reservoir = true, exact = true, trials = false, rare = true;
   for (int i = 0; i < njobs; ++i) {
@@ -1205,36 +1231,37 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     trials = trials || (!scan && jobs[i].weighted);
     rare = rare && (jobs[i].mode == MODE_RJS || (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
   }
-  if (!COUNT) {
-    s->share = hub_share_pays(g, jobs, njobs, total, blocks * kBlock);
-    const bool few = total <= blocks * kBlock;
-    s->coop = ALG == ALGO_PAGERANK2 ? !scans && (few || g->envelope >= kTogetherPagerank)
-                                    : trials && g->envelope >= kTogetherEnvelope;
-    s->only = s->share ? kAny : reservoir ? kOnlyRvs : exact ? kOnlyExact : kAny;
-    e = s->share                ? walk_blocks_per_sm<NJ, false, ALG, true, true>(&bps)
-        : s->only == kOnlyRvs   ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyRvs>(&bps)
-        : s->only == kOnlyExact ? walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyExact>(&bps)
-        : s->coop               ? walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&bps)
-                                : walk_blocks_per_sm<NJ, false, ALG, true>(&bps);
+  int bps = 1;
+  cudaError_t e = walk_blocks_per_sm<NJ, ALG>(count ? V_COUNTING : V_QUEUED, &bps);
+  if (e != cudaSuccess) return e;
+  const long long lanes = (long long)g->num_sms * bps * kBlock;
+  s->variant = V_COUNTING;
+  s->wpw = 32;
+  bool spread = false;
+  if (!count) {
+    const bool together = ALG == ALGO_PAGERANK2 ? !scans && (total <= lanes || g->envelope >= kTogetherPagerank)
+                                                : trials && g->envelope >= kTogetherEnvelope;
+    s->variant = hub_share_pays(g, jobs, njobs, total, lanes) ? V_SPREAD_SHARE
+                 : reservoir                                  ? V_SPREAD_RVS
+                 : exact                                      ? V_SPREAD_EXACT
+                 : together                                   ? V_SPREAD_TOGETHER
+                                                              : V_SPREAD;
+    e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
     if (e != cudaSuccess) return e;
-    const long long spread_blocks = (long long)g->num_sms * bps;
-    s->spread = scans || total <= spread_blocks * kBlock;
-    s->share = s->share && s->spread;
-    if (s->spread) {
-      blocks = spread_blocks;
-      s->wpw = (int)std::max<long long>(1, (total + blocks * kWarps - 1) / (blocks * kWarps));
+    const long long resident = (long long)g->num_sms * bps * kWarps;  // warps
+    spread = scans || total <= resident * 32;
+    if (spread) {
+      s->wpw = (int)std::max<long long>(1, (total + resident - 1) / resident);
       if (scans) s->wpw = std::min(s->wpw, reservoir && scanned < kShortScan ? 8 : 1);
+    } else {
+      s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
+      e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
+      if (e != cudaSuccess) return e;
     }
   }
-  if (!COUNT && ALG == ALGO_NODE2VEC && !s->spread && !s->coop && rare) s->only = kWhole;  // the same occupancy as kAny
-  if (!s->spread && s->coop) {
-    e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&bps);
-    if (e != cudaSuccess) return e;
-    blocks = (long long)g->num_sms * bps;
-  }
-  const long long per_block = s->spread ? s->wpw : kBlock;  // a spread launch takes a block for every warp while it can
-  s->grid = (int)std::min<long long>(blocks, std::max<long long>(1, (total + per_block - 1) / per_block));
-  s->queue = !s->spread || (long long)s->grid * kWarps * s->wpw < total;
+  const long long per_block = spread ? s->wpw : kBlock;  // a spread launch takes a block for every warp while it can
+  s->grid = (int)std::min<long long>((long long)g->num_sms * bps, std::max<long long>(1, (total + per_block - 1) / per_block));
+  s->queue = !spread || (long long)s->grid * kWarps * s->wpw < total;
   return cudaSuccess;
 }
 
@@ -1250,53 +1277,38 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
 // jobs mix lanes of q < 1 and q > 1 in a warp and keep 2 (64 mixed jobs: 8.54
 // ms, with 1 for q < 1 8.96); so do launches of whole scans (p = 4, q = 1/4, r
 // = 1/4 4.20, with 1 4.28).
-inline int32_t round_trials(const Job& J, bool spread, int only, int njobs) {
+inline int32_t round_trials(const Job& J, int variant, int njobs) {
   if (J.round > 0) return J.round;
-  if (spread || J.algo == ALGO_PAGERANK2) return 4;
-  if (njobs == 1 && only != kWhole && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
+  if (variant >= V_SPREAD || J.algo == ALGO_PAGERANK2) return 4;
+  if (njobs == 1 && variant != V_QUEUED_WHOLE && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
   return kRjsBatchDefault;
 }
 
-template <int NJ, bool COUNT, int ALG>
-inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total,
+template <int NJ, int ALG>
+inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
                                  unsigned long long* qctr, cudaStream_t stream) {
   LaunchShape s;
-  cudaError_t e = walk_shape<NJ, COUNT, ALG>(g, jobs, njobs, total, &s);
+  cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, &s);
   if (e != cudaSuccess) return e;
   if (s.queue && !qctr) return cudaErrorInvalidValue;
   if (!s.queue) qctr = nullptr;
   JobTableN<NJ> tab;
   for (int i = 0; i < njobs; ++i) {
     tab.jobs[i] = jobs[i];
-    tab.jobs[i].round = round_trials(jobs[i], s.spread, s.only, njobs);
+    tab.jobs[i].round = round_trials(jobs[i], s.variant, njobs);
   }
-  auto launch = [&](auto kernel) {
-    kernel<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err, g->d_cnt);
-  };
-  if (s.share) launch(walk_kernel<NJ, false, ALG, true, true>);
-  else if (s.only == kOnlyRvs) launch(walk_kernel<NJ, false, ALG, true, false, false, kOnlyRvs>);
-  else if (s.only == kOnlyExact) launch(walk_kernel<NJ, false, ALG, true, false, false, kOnlyExact>);
-  else if (s.spread && s.coop) launch(walk_kernel<NJ, false, ALG, true, false, true>);
-  else if (s.spread) launch(walk_kernel<NJ, false, ALG, true>);
-  else if (s.coop) launch(walk_kernel<NJ, false, ALG, false, false, true>);
-  else if (ALG == ALGO_NODE2VEC && s.only == kWhole) launch(walk_kernel<NJ, false, ALG, false, false, false, ALG == ALGO_NODE2VEC ? kWhole : kAny>);
-  else launch(walk_kernel<NJ, COUNT, ALG>);
+  walk_variant<NJ, ALG>(s.variant)<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err,
+                                                                 g->d_cnt);
   g_launches.fetch_add(1);
   return cudaGetLastError();
 }
 
-// Cache the occupancy of every variant for one algorithm (outside any capture).
+// Load every variant of one algorithm and cache its occupancy (outside any capture).
 template <int NJ, int ALG>
 inline cudaError_t prime_walk() {
+  cudaError_t e = cudaSuccess;
   int b;
-  cudaError_t e = walk_blocks_per_sm<NJ, false, ALG>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, true, ALG>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, true>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, true>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyRvs>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, true, false, false, kOnlyExact>(&b);
-  if (e == cudaSuccess) e = walk_blocks_per_sm<NJ, false, ALG, false, false, true>(&b);
+  for (int v = 0; v < kWalkVariants && e == cudaSuccess; ++v) e = walk_blocks_per_sm<NJ, ALG>(v, &b);
   return e;
 }
 
@@ -1316,13 +1328,11 @@ template <int NJ, int ALG>
 inline WalkLaunches make_launches() {
   return {[](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, unsigned long long* qctr,
              cudaStream_t st) {
-            return count ? launch_walk_t<NJ, true, ALG>(g, jobs, njobs, total, qctr, st)
-                         : launch_walk_t<NJ, false, ALG>(g, jobs, njobs, total, qctr, st);
+            return launch_walk_t<NJ, ALG>(g, jobs, njobs, total, count, qctr, st);
           },
           [](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, bool* need) {
             LaunchShape s = {};
-            const cudaError_t e = count ? walk_shape<NJ, true, ALG>(g, jobs, njobs, total, &s)
-                                        : walk_shape<NJ, false, ALG>(g, jobs, njobs, total, &s);
+            const cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, &s);
             *need = s.queue;
             return e;
           },
