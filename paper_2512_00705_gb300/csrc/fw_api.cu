@@ -4,7 +4,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "fw_internal.h"
@@ -296,16 +298,22 @@ fw_status rebuild_derived(fw_graph* g, cudaStream_t st) {
   return fs;
 }
 
-static fw_status with_qctr(const fw_graph* g, const Job* jobs, long long total, bool count, cudaStream_t st) {
+int streams_at_work(const fw_graph* g, cudaStream_t stream) {
+  uintptr_t id = reinterpret_cast<uintptr_t>(stream);
+  if (stream == cudaStreamPerThread) id = (uintptr_t)std::hash<std::thread::id>{}(std::this_thread::get_id());
+  return g->streams.note(id);
+}
+
+static fw_status with_qctr(const fw_graph* g, const Job* jobs, long long total, bool count, int beside, cudaStream_t st) {
   bool need = true;
-  cudaError_t e = single_needs_queue(g, jobs[0], total, count, &need);
+  cudaError_t e = single_needs_queue(g, jobs[0], total, count, beside, &need);
   if (e != cudaSuccess) return cuda_error(e, "walk launch");
   unsigned long long* q = nullptr;
   if (need) {
     e = alloc_counters(g, 1, &q, st);
     if (e != cudaSuccess) return cuda_error(e, "queue counter");
   }
-  e = launch_walk(g, jobs, 1, total, count, q, st);
+  e = launch_walk(g, jobs, 1, total, count, beside, q, st);
   cudaError_t e2 = q ? cudaFreeAsync(q, st) : cudaSuccess;
   if (e != cudaSuccess) return cuda_error(e, "walk launch");
   if (e2 != cudaSuccess) return cuda_error(e2, "cudaFreeAsync(queue counter)");
@@ -599,7 +607,8 @@ extern "C" fw_status fw_walk(const fw_graph* g, const int32_t* starts, int32_t n
   J.len = len;
   J.gbase = 0;
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
-  return with_qctr(g, &J, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
+  const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  return with_qctr(g, &J, num_walkers, count, streams_at_work(g, st), st);
 }
 
 extern "C" fw_status fw_walk_ids(const fw_graph* g, const int32_t* starts, const uint32_t* walker_ids,
@@ -620,7 +629,8 @@ extern "C" fw_status fw_walk_ids(const fw_graph* g, const int32_t* starts, const
   J.len = len;
   J.gbase = 0;
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
-  return with_qctr(g, &J, num_walkers, count, reinterpret_cast<cudaStream_t>(stream));
+  const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  return with_qctr(g, &J, num_walkers, count, streams_at_work(g, st), st);
 }
 
 // Rows of at least this many bytes are walked in chunks so that the copy of
@@ -675,6 +685,7 @@ extern "C" fw_status fw_walk_host(fw_graph* g, const int32_t* starts, int32_t nu
   const size_t bytes_out = nout * sizeof(int32_t);
   const int K = (int)std::min<size_t>((size_t)kHostChunksMax, std::max<size_t>(1, bytes_out / kHostChunkBytes));
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
+  const int beside = std::max(streams_at_work(g, st), std::min(K, kHostWalkStreams));  // chunks in flight
   cudaEvent_t* ev = g->host_ev;
   cudaError_t e = cudaMemcpyAsync(g->d_stage_starts, starts, nin * sizeof(int32_t), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaEventRecord(ev[kHostChunksMax], st);
@@ -695,7 +706,7 @@ extern "C" fw_status fw_walk_host(fw_graph* g, const int32_t* starts, int32_t nu
     Jc.len = len;
     Jc.gbase = 0;
     Jc.walker_base = J.walker_base + (uint32_t)lo;
-    s = with_qctr(g, &Jc, (long long)(hi - lo), count, ws);
+    s = with_qctr(g, &Jc, (long long)(hi - lo), count, beside, ws);
     if (s != FW_OK) break;
     e = cudaEventRecord(ev[c], ws);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(g->host_copy, ev[c], 0);
@@ -736,12 +747,14 @@ extern "C" fw_status fw_sample_hist(const fw_graph* g, int32_t v, int32_t v_prev
   J.hstep = step;
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
   const uint32_t base0 = J.walker_base;
+  const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const int beside = streams_at_work(g, st);
   for (int64_t done = 0; done < ndraws;) {
     const int64_t chunk = (ndraws - done) < (1LL << 30) ? (ndraws - done) : (1LL << 30);
     J.walker_base = base0 + (uint32_t)done;
     J.num_walkers = (int32_t)chunk;
     J.len = 1;
-    s = with_qctr(g, &J, chunk, count, reinterpret_cast<cudaStream_t>(stream));
+    s = with_qctr(g, &J, chunk, count, beside, st);
     if (s != FW_OK) return s;
     done += chunk;
   }

@@ -59,7 +59,7 @@ extern "C" fw_status fw_walk_batch(const fw_graph* g, const fw_job* jobs, int32_
     unsigned long long* q = nullptr;  // one walker queue per algorithm
     cudaError_t e = alloc_counters(g, kQueueCounters, &q, st);
     if (e != cudaSuccess) return cuda_error(e, "queue counter");
-    e = launch_walk(g, tab.data(), (int)tab.size(), total, count, q, st);
+    e = launch_walk(g, tab.data(), (int)tab.size(), total, count, streams_at_work(g, st), q, st);
     cudaError_t e2 = cudaFreeAsync(q, st);
     if (e != cudaSuccess) return cuda_error(e, "batch launch");
     if (e2 != cudaSuccess) return cuda_error(e2, "cudaFreeAsync(queue counter)");
@@ -126,8 +126,8 @@ extern "C" fw_status fw_batch_plan_create(const fw_graph* g, const fw_job* jobs,
     e = cudaMemsetAsync(q, 0, sizeof(unsigned long long) * kQueueCounters, cap);
     const unsigned long long before = g_launches.load();
     if (e == cudaSuccess) {
-      e = tabs[c].size() == 1 ? launch_walk(g, tabs[c].data(), 1, totals[c], counts[c], q, cap)
-                              : launch_walk_mixed(g, tabs[c].data(), (int)tabs[c].size(), counts[c], q, cap, side, ev);
+      e = tabs[c].size() == 1 ? launch_walk(g, tabs[c].data(), 1, totals[c], counts[c], 1, q, cap)
+                              : launch_walk_mixed(g, tabs[c].data(), (int)tabs[c].size(), counts[c], 1, q, cap, side, ev);
     }
     const unsigned long long launched = g_launches.load() - before;
     p->kernels += (int)launched;

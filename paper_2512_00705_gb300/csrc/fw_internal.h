@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "fw_device.cuh"
+#include "fw_streams.h"
 #include "../../include/flexiwalk.h"
 
 // fw_walk_host splits large requests into at most this many chunks
@@ -55,6 +56,7 @@ struct fw_graph {
   unsigned long long fingerprint = 0;
   double preprocess_ms = 0.0;
   size_t bytes = 0;
+  mutable fw::RecentStreams streams;     // streams of recent launches (a choice of launch shape only)
   cudaMemPool_t counter_pool = nullptr;  // queue counters of launches (nullptr: the device's default pool)
   // staging of fw_walk_host
   std::mutex stage_mu;
@@ -85,12 +87,14 @@ fw_status make_job(const fw_graph* g, int32_t algo, const fw_params* params, uin
 // Launch the walk over `njobs` jobs (total walkers `total`; njobs <= kMaxJobs).
 // `qctr` points to zeroed device counters the launch uses as walker queues:
 // one for a single job (see single_needs_queue), kAlgos (one per algorithm) for several.  Several
-// jobs give one kernel launch per algorithm present.
-cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+// jobs give one kernel launch per algorithm present.  `beside`: calls, this
+// one included, whose launches are meant to run at the same time (1: it has
+// the GPU to itself); the rows do not depend on it.
+cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                         unsigned long long* qctr, cudaStream_t stream);
 // Does a single-job launch need a queue counter?  Without one (every walker
 // has a lane of its own) launch_walk may be given qctr = nullptr.
-cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, bool* need);
+cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, int beside, bool* need);
 // `count` zeroed queue counters for one launch on `stream`, from the graph's
 // pool; release with cudaFreeAsync on the same stream after the launch.
 cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t stream);
@@ -98,8 +102,12 @@ cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** ou
 // `stream` one after another, or (side: kAlgos - 1 helper streams, ev:
 // kAlgos events) side by side, joined back into `stream`.  qctr: kAlgos
 // zeroed counters.
-cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, bool count, unsigned long long* qctr,
-                              cudaStream_t stream, const cudaStream_t* side = nullptr, cudaEvent_t* ev = nullptr);
+cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, bool count, int beside,
+                              unsigned long long* qctr, cudaStream_t stream, const cudaStream_t* side = nullptr,
+                              cudaEvent_t* ev = nullptr);
+// Streams this graph's walks were launched on a moment ago, `stream` included
+// (noted as one of them): `beside` of calls that do not know.
+int streams_at_work(const fw_graph* g, cudaStream_t stream);
 constexpr int kQueueCounters = fw::kAlgos;  // counters a multi-job launch needs
 
 // Cache the walk kernels' occupancy (call outside any stream capture).

@@ -34,14 +34,14 @@ cudaError_t prime_walk_occupancy() {
   return e;
 }
 
-cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, bool* need) {
-  return single_launches(job.algo).needs_queue(g, &job, 1, total, count, need);
+cudaError_t single_needs_queue(const fw_graph* g, const Job& job, long long total, bool count, int beside, bool* need) {
+  return single_launches(job.algo).needs_queue(g, &job, 1, total, count, beside, need);
 }
 
-cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+cudaError_t launch_walk(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                         unsigned long long* qctr, cudaStream_t stream) {
-  if (njobs == 1) return single_launches(jobs[0].algo).launch(g, jobs, 1, total, count, qctr, stream);
-  return launch_walk_mixed(g, jobs, njobs, count, qctr, stream);
+  if (njobs == 1) return single_launches(jobs[0].algo).launch(g, jobs, 1, total, count, beside, qctr, stream);
+  return launch_walk_mixed(g, jobs, njobs, count, beside, qctr, stream);
 }
 
 // ---------------------------------------------------------------- preprocessing

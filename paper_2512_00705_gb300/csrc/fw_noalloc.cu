@@ -96,7 +96,7 @@ extern "C" fw_status fw_walk_host_noalloc(const fw_graph* g, const int32_t* star
   const bool count = params && (params->flags & FW_FLAG_COUNTERS);
   e = cudaMemsetAsync(qctr, 0, sizeof(unsigned long long), st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_starts, starts, in_bytes, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_walk(g, &J, 1, num_walkers, count, qctr, st);
+  if (e == cudaSuccess) e = launch_walk(g, &J, 1, num_walkers, count, streams_at_work(g, st), qctr, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, out_bytes, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {

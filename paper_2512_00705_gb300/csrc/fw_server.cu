@@ -207,8 +207,9 @@ struct CopyRun {
 // algorithm present), copy the rows out, record the wave's event.  Called
 // WITHOUT the server lock, so submit / poll are not held up by the CUDA
 // calls: it only reads the requests' immutable fields and uses the wave,
-// which the worker reserved.  Returns the first failing CUDA call's error.
-cudaError_t enqueue_wave(fw_server* s, Wave& w, const std::vector<Request*>& batch) {
+// which the worker reserved.  `beside`: waves in flight, this one included.
+// Returns the first failing CUDA call's error.
+cudaError_t enqueue_wave(fw_server* s, Wave& w, const std::vector<Request*>& batch, int beside) {
   using namespace fw;
   *w.hops_host = 0;
   CopyRun up(cudaMemcpyHostToDevice, w.stream), down(cudaMemcpyDeviceToHost, w.stream);
@@ -239,8 +240,9 @@ cudaError_t enqueue_wave(fw_server* s, Wave& w, const std::vector<Request*>& bat
   if (e == cudaSuccess) e = up.flush();
   if (e == cudaSuccess) e = cudaMemsetAsync(w.qctr, 0, sizeof(unsigned long long) * (kHopSlot + 1), w.stream);
   if (e == cudaSuccess && total > 0)
-    e = tab.size() == 1 ? launch_walk(s->g, tab.data(), 1, total, false, w.qctr, w.stream)
-                        : launch_walk_mixed(s->g, tab.data(), (int)tab.size(), false, w.qctr, w.stream, w.side, w.fork);
+    e = tab.size() == 1 ? launch_walk(s->g, tab.data(), 1, total, false, beside, w.qctr, w.stream)
+                        : launch_walk_mixed(s->g, tab.data(), (int)tab.size(), false, beside, w.qctr, w.stream, w.side,
+                                            w.fork);
   if (e == cudaSuccess && total > 0) {
     HopRows hr;
     hr.n = (int)tab.size();
@@ -284,6 +286,8 @@ void launch_wave(fw_server* s, Wave& w, int cls, std::unique_lock<std::mutex>& l
     r->t_launch = now;
   }
   w.busy = true;  // reserved: no other launch takes this wave meanwhile
+  int beside = 0;
+  for (const Wave& x : s->waves) beside += x.busy ? 1 : 0;
   bool need_mirror = false;
   for (Request* r : batch) need_mirror = need_mirror || !r->pinned_in || !r->pinned_out;
   lk.unlock();
@@ -297,7 +301,7 @@ void launch_wave(fw_server* s, Wave& w, int cls, std::unique_lock<std::mutex>& l
     }
   }
   const auto t0 = Clock::now();
-  const cudaError_t e = enqueue_wave(s, w, batch);
+  const cudaError_t e = enqueue_wave(s, w, batch, beside);
   const double host_ms = std::chrono::duration<double, std::milli>(Clock::now() - t0).count();
   lk.lock();
   s->enqueue_ms += host_ms;

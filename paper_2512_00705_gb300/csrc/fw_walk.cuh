@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "fw_internal.h"
+#include "fw_shape.h"
 
 namespace fw {
 
@@ -1218,9 +1219,9 @@ struct LaunchShape {
 };
 
 template <int NJ, int ALG>
-inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                               LaunchShape* s) {
-  constexpr int kWarps = kBlock / 32;
+  static_assert(kBlock == 32 * kShapeWarps, "place_walkers knows the block size");
   const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
   bool scans = true, reservoir = true, exact = true, trials = false, rare = true;
   for (int i = 0; i < njobs; ++i) {
@@ -1235,9 +1236,8 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   cudaError_t e = walk_blocks_per_sm<NJ, ALG>(count ? V_COUNTING : V_QUEUED, &bps);
   if (e != cudaSuccess) return e;
   const long long lanes = (long long)g->num_sms * bps * kBlock;
+  WalkerPlacement place = {false, 32, 0};
   s->variant = V_COUNTING;
-  s->wpw = 32;
-  bool spread = false;
   if (!count) {
     const bool together = ALG == ALGO_PAGERANK2 ? !scans && (total <= lanes || g->envelope >= kTogetherPagerank)
                                                 : trials && g->envelope >= kTogetherEnvelope;
@@ -1248,20 +1248,18 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
                                                               : V_SPREAD;
     e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
     if (e != cudaSuccess) return e;
-    const long long resident = (long long)g->num_sms * bps * kWarps;  // warps
-    spread = scans || total <= resident * 32;
-    if (spread) {
-      s->wpw = (int)std::max<long long>(1, (total + resident - 1) / resident);
-      if (scans) s->wpw = std::min(s->wpw, reservoir && scanned < kShortScan ? 8 : 1);
-    } else {
+    place = place_walkers(total, g->num_sms * bps, scans, reservoir && scanned < kShortScan ? 8 : 1, NJ > 1, beside);
+    if (!place.by_place) {
       s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
       if (e != cudaSuccess) return e;
     }
   }
-  const long long per_block = spread ? s->wpw : kBlock;  // a spread launch takes a block for every warp while it can
-  s->grid = (int)std::min<long long>((long long)g->num_sms * bps, std::max<long long>(1, (total + per_block - 1) / per_block));
-  s->queue = !spread || (long long)s->grid * kWarps * s->wpw < total;
+  if (!place.by_place)  // full warps, at most the resident blocks
+    place.grid = (int)std::min<long long>((long long)g->num_sms * bps, std::max<long long>(1, (total + kBlock - 1) / kBlock));
+  s->wpw = place.wpw;
+  s->grid = place.grid;
+  s->queue = !place.by_place || (long long)place.grid * kShapeWarps * place.wpw < total;
   return cudaSuccess;
 }
 
@@ -1285,10 +1283,10 @@ inline int32_t round_trials(const Job& J, int variant, int njobs) {
 }
 
 template <int NJ, int ALG>
-inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                                  unsigned long long* qctr, cudaStream_t stream) {
   LaunchShape s;
-  cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, &s);
+  cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, beside, &s);
   if (e != cudaSuccess) return e;
   if (s.queue && !qctr) return cudaErrorInvalidValue;
   if (!s.queue) qctr = nullptr;
@@ -1316,9 +1314,10 @@ inline cudaError_t prime_walk() {
 // instantiated in a source file of its own (WALK_LAUNCHES), so that they
 // compile side by side.
 struct WalkLaunches {
-  cudaError_t (*launch)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count,
+  cudaError_t (*launch)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                         unsigned long long* qctr, cudaStream_t stream);
-  cudaError_t (*needs_queue)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, bool* need);
+  cudaError_t (*needs_queue)(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
+                             bool* need);
   cudaError_t (*prime)();
 };
 const WalkLaunches& single_launches(int algo);  // one job
@@ -1326,13 +1325,10 @@ const WalkLaunches& table_launches(int algo);   // up to kMaxJobs jobs
 
 template <int NJ, int ALG>
 inline WalkLaunches make_launches() {
-  return {[](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, unsigned long long* qctr,
-             cudaStream_t st) {
-            return launch_walk_t<NJ, ALG>(g, jobs, njobs, total, count, qctr, st);
-          },
-          [](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, bool* need) {
+  return {launch_walk_t<NJ, ALG>,
+          [](const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside, bool* need) {
             LaunchShape s = {};
-            const cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, &s);
+            const cudaError_t e = walk_shape<NJ, ALG>(g, jobs, njobs, total, count, beside, &s);
             *need = s.queue;
             return e;
           },

@@ -35,8 +35,8 @@ cudaError_t prime_walk_mixed_occupancy() {
   return e;
 }
 
-cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, bool count, unsigned long long* qctr,
-                              cudaStream_t stream, const cudaStream_t* side, cudaEvent_t* ev) {
+cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, bool count, int beside,
+                              unsigned long long* qctr, cudaStream_t stream, const cudaStream_t* side, cudaEvent_t* ev) {
   if (njobs < 1 || njobs > kMaxJobs) return cudaErrorInvalidValue;
   Job grp[kMaxJobs];
   int present[kAlgos], np = 0;
@@ -66,7 +66,7 @@ cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, boo
   for (int i = 0; i < np && e == cudaSuccess; ++i) {
     const int a = present[i];
     cudaStream_t st = (fork && i > 0) ? side[i - 1] : stream;
-    e = table_launches(a).launch(g, grp + firsts[a], counts[a], totals[a], count, qctr + a, st);
+    e = table_launches(a).launch(g, grp + firsts[a], counts[a], totals[a], count, fork ? beside * np : beside, qctr + a, st);
   }
   if (fork) {  // `stream` waits for the helper streams
     for (int i = 1; i < np && e == cudaSuccess; ++i) {
