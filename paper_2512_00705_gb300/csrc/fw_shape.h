@@ -24,8 +24,21 @@ struct WalkerPlacement {
   int grid;       // blocks
 };
 
-// `total` walkers on a GPU that holds `blocks` resident blocks of the kernel
-// that gives walkers by place; `scans`: jobs that only scan rows, at most
+// Blocks per SM whose warps a launch fills before its walkers share warps
+// further: launches of more than two walkers for each resident warp.
+// First-order walks (weighted, metapath) are bound by instruction issue before
+// their warps fill every slot.  GB300, R-MAT s12 /
+// s16 / s20, U(0,1] and no weights, x 30 hops, mean speed against full warps
+// with all resident blocks / 3 / 2 / 1: weighted 5,000 walkers 1.60 / 1.60 /
+// 1.59 / 1.56, 20,000 1.23 / 1.28 / 1.34 / 1.31, 60,000 1.00 / 1.12 / 1.18 /
+// 1.17, 120,000 1.13 / 1.16 / 1.16 / 1.16 (with every block slower than full
+// warps from 40,000 to 60,000, down to 0.91); metapath 20,000 1.28 / 1.32 /
+// 1.39 / 1.33, 60,000 1.05 / 1.14 / 1.19 / 1.13.  node2vec 20,000 1.79 with
+// all, 1.69 with 2.
+constexpr int kFirstOrderFill = 2, kFillAll = 64;
+
+// `total` walkers on `sms` SMs with `bps` resident blocks each of the kernel
+// that gives walkers by place, of which it fills `fill` per SM first; `scans`: jobs that only scan rows, at most
 // `scan_wpw` walkers per warp, the rest in the queue.  `table`: several jobs.
 // `beside`: launches, this one included, that are meant to run at the same
 // time.
@@ -39,9 +52,12 @@ struct WalkerPlacement {
 // -> its share of it (us per launch): node2vec 3,000 walkers 60 -> 32, 20,000
 // 184 -> 68, 60,000 313 -> 127 (full warps always: 59 / 75 / 169); batches of
 // 64 served queries 583 -> 463 ms.
-inline WalkerPlacement place_walkers(long long total, int blocks, bool scans, int scan_wpw, bool table, int beside) {
+inline WalkerPlacement place_walkers(long long total, int sms, int bps, int fill, bool scans, int scan_wpw, bool table,
+                                     int beside) {
   WalkerPlacement p;
-  const long long share = std::max(1, blocks / std::max(1, beside));
+  const int blocks = sms * bps;
+  if (total <= 2ll * blocks * kShapeWarps) fill = kFillAll;
+  const long long share = std::max(1, std::min(sms * fill, blocks / std::max(1, beside)));
   const long long warps = share * kShapeWarps;
   p.wpw = (int)std::min<long long>(32, std::max<long long>(1, (total + warps - 1) / warps));
   if (scans) p.wpw = std::min(p.wpw, scan_wpw);

@@ -1248,7 +1248,8 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
                                                               : V_SPREAD;
     e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
     if (e != cudaSuccess) return e;
-    place = place_walkers(total, g->num_sms * bps, scans, reservoir && scanned < kShortScan ? 8 : 1, NJ > 1, beside);
+    const int fill = !scans && (ALG == ALGO_WEIGHTED || ALG == ALGO_METAPATH) ? kFirstOrderFill : kFillAll;
+    place = place_walkers(total, g->num_sms, bps, fill, scans, reservoir && scanned < kShortScan ? 8 : 1, NJ > 1, beside);
     if (!place.by_place) {
       s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);

@@ -15,21 +15,26 @@ SHAPE = r"""
 #include "fw_shape.h"
 #define CHECK(c) do { if (!(c)) { std::printf("FAIL line %d: %s (total %lld blocks %d beside %d)\n", __LINE__, #c, total, blocks, beside); return 1; } } while (0)
 
+#define CHECK3(c) do { if (!(c)) { std::printf("FAIL line %d: %s\n", __LINE__, #c); return 1; } } while (0)
+
 int main() {
-  for (int blocks : {1, 2, 152, 456, 608, 1064})
+  for (int sms : {1, 2, 152})
+  for (int bps : {1, 3, 4, 7})
     for (int beside : {1, 2, 3, 4, 8, 24, 192})
       for (long long total : {1ll, 2ll, 31ll, 37ll, 300ll, 3000ll, 5003ll, 20000ll, 60000ll, 77824ll, 77825ll, 155647ll, 155648ll, 155649ll, 272384ll, 2000000ll, 1ll << 30})
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < 16; ++k) {
+          const int blocks = sms * bps, fill = k >= 8 ? fw::kFirstOrderFill : fw::kFillAll;
           const int scan = (k & 3) == 0 ? 0 : (k & 3) == 1 ? 1 : (k & 3) == 2 ? 8 : 32;
-          const bool table = k >= 4;
-          const fw::WalkerPlacement p = fw::place_walkers(total, blocks, scan > 0, scan, table, beside);
+          const bool table = (k & 4) != 0;
+          const fw::WalkerPlacement p = fw::place_walkers(total, sms, bps, fill, scan > 0, scan, table, beside);
           const long long lanes = 256ll * blocks, placed = (long long)p.grid * fw::kShapeWarps * p.wpw;
           CHECK(p.wpw >= 1 && p.wpw <= 32 && p.grid >= 1 && p.grid <= blocks);
           CHECK(p.by_place || p.wpw == 32);
           CHECK(!scan || (p.by_place && p.wpw <= scan));
           if (p.by_place && !scan) CHECK(placed >= total);                          // no queue
           if (!scan && beside == 1) CHECK(p.by_place == (total <= lanes));
-          if (!scan && beside == 1 && total <= lanes / 32) CHECK(p.wpw == 1 && p.grid == (total < blocks ? total : blocks));
+          const long long filled = 8ll * blocks;
+          if (!scan && beside == 1 && total <= filled) CHECK(p.wpw == 1 && p.grid == (total < blocks ? total : blocks));
           if (!scan && beside > 1 && p.by_place) {                                  // its share, filled
             CHECK(p.wpw <= (table ? fw::kSharedWalkersTable : fw::kSharedWalkersJob));
             CHECK((long long)p.grid * beside <= blocks || p.grid == 1);
@@ -37,8 +42,10 @@ int main() {
           }
           if (!scan && beside > 1 && !p.by_place) CHECK(p.grid == (total + 255) / 256 || p.grid == blocks);
         }
+  // first-order: 60,000 walkers alone, 25 to a warp
+  CHECK3(fw::place_walkers(60000, 152, 4, fw::kFirstOrderFill, false, 32, false, 1).wpw == 25);
   // 20,000 walkers on 152 SMs x 4 blocks: alone on every block, beside seven others in 79 blocks of full warps
-  const fw::WalkerPlacement a = fw::place_walkers(20000, 608, false, 32, false, 1), b = fw::place_walkers(20000, 608, false, 32, false, 8);
+  const fw::WalkerPlacement a = fw::place_walkers(20000, 152, 4, fw::kFillAll, false, 32, false, 1), b = fw::place_walkers(20000, 152, 4, fw::kFillAll, false, 32, false, 8);
   long long total = 20000;
   int blocks = 608, beside = 8;
   CHECK(a.by_place && a.wpw == 5 && a.grid == 608);
