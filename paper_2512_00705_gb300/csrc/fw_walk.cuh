@@ -36,20 +36,21 @@ constexpr int kBlock = 256;
 // thread at 4, 80 at 3, 48 at 5, 40 at 6, 32 at 7.  More warps hide the gathers'
 // latency until the spills cost more.  GB300, ms: node2vec s22 p = 1/4, q = 4
 // 40.0 / 33.9 / 37.5 with 3 / 4 / 5, its trials-together variant (Pareto 1,
-// s20) 50.6 / 42.4 / 41.0; weighted s22 8.57 / 7.21 / 7.04 and 7.43 with 6,
-// for few walkers 0.061 with 4, 0.069 with 5; second-order PageRank s20 4.35
+// s20) 50.6 / 42.4 / 41.0; weighted s22 8.57 / 7.21 / 7.04 and 7.43 with 6
+// (5: the dense variant, see kDenseRecords), for few walkers 0.061 with 4,
+// 0.069 with 5; second-order PageRank s20 4.35
 // / 4.49 / 4.8, its trials-together variant on Pareto 1 24.7 / 22.6 with 3 /
 // 4; metapath 1.55 / 1.33 / 1.65; the eRVS-only variant (node2vec s18) 10.5 /
 // 9.5 / 9.1 / 8.42 / 8.40 with 4 / 5 / 6 / 7 / 8, exact-only (weighted s18)
 // 2.92 / 2.87 / 3.14 / 3.80 with 4 / 5 / 6 / 7.
-// samplers a kernel variant holds (kWhole: all, short eRVS rows scanned at once, see kLaneRvs)
-enum : int { kAny = 0, kOnlyRvs = 1, kOnlyExact = 2, kWhole = 3 };
+// samplers a kernel variant holds (kWhole: all, short eRVS rows scanned at once, see kLaneRvs; kDense: all)
+enum : int { kAny = 0, kOnlyRvs = 1, kOnlyExact = 2, kWhole = 3, kDense = 4 };
 template <int ALG, bool SPREAD, bool SHARE, bool COOP, int ONLY>
 constexpr int kMinBlocks = ONLY == kOnlyRvs                           ? 7
                            : ONLY == kOnlyExact                       ? 5
                            : SHARE                                    ? 4
                            : ALG == ALGO_NODE2VEC && COOP             ? 5
-                           : ALG == ALGO_WEIGHTED && !SPREAD && !COOP ? 5
+                           : ONLY == kDense                           ? 5
                            : ALG == ALGO_PAGERANK2 && (SPREAD || !COOP) ? 3
                                                                       : 4;
 constexpr int kThreadExactMaxDeg = 16; // exact steps with d <= this run on one lane
@@ -468,7 +469,7 @@ __device__ __forceinline__ void walk_loop(const DevGraph& g, const Job* sj, int 
   // lanes per warp (5,003 walkers 379 and 538 us); second-order PageRank
   // seldom has such rows and loses the registers (8.46 and 8.80 ms).
   constexpr bool kLaneRvs = !SPREAD && ALG == ALGO_NODE2VEC && ONLY != kWhole;
-  constexpr bool kTrials = ONLY == kAny || ONLY == kWhole, kRvs = ONLY != kOnlyExact;
+  constexpr bool kTrials = ONLY != kOnlyRvs && ONLY != kOnlyExact, kRvs = ONLY != kOnlyExact;
   constexpr bool kExact = ONLY == kOnlyExact || (kTrials && (COUNT || NJ > 1));  // single exact jobs: kOnlyExact
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x;
@@ -1121,6 +1122,7 @@ enum WalkVariant : int {
   V_QUEUED,           // full warps that fetch from the queue
   V_QUEUED_TOGETHER,  // the same, with trials together
   V_QUEUED_WHOLE,     // the same, short eRVS rows scanned at once (node2vec; elsewhere V_QUEUED does that)
+  V_QUEUED_DENSE,     // the same, 5 blocks per SM (weighted; elsewhere V_QUEUED)
   V_SPREAD,           // walkers given by place
   V_SPREAD_TOGETHER,  // the same, with trials together
   V_SPREAD_SHARE,     // the same, with hub sharing
@@ -1138,6 +1140,7 @@ inline WalkKernel<NJ> walk_variant(int v) {
     case V_COUNTING: return walk_kernel<NJ, true, ALG>;
     case V_QUEUED_TOGETHER: return walk_kernel<NJ, false, ALG, false, false, true>;
     case V_QUEUED_WHOLE: return walk_kernel<NJ, false, ALG, false, false, false, ALG == ALGO_NODE2VEC ? kWhole : kAny>;
+    case V_QUEUED_DENSE: return walk_kernel<NJ, false, ALG, false, false, false, ALG == ALGO_WEIGHTED ? kDense : kAny>;
     case V_SPREAD: return walk_kernel<NJ, false, ALG, true>;
     case V_SPREAD_TOGETHER: return walk_kernel<NJ, false, ALG, true, false, true>;
     case V_SPREAD_SHARE: return walk_kernel<NJ, false, ALG, true, true>;
@@ -1212,6 +1215,18 @@ constexpr float kRareRatio = 1.5f;
 // 429 / 255; 430: 995 / 1,009, 1,855 / 2,190, 372 / 225; 1,246: 1,793 /
 // 2,573, 4,051 / 5,364, 557 / 490.
 constexpr double kShortScan = 250.0;
+// Queued weighted walks take 5 blocks per SM (48 registers) instead of 4 where
+// that hides memory latency: edge records beyond L2, weights whose
+// envelope is low (few trials per hop), walks that are not short, and
+// fewer turns of the resident lanes.  GB300, speed against the earlier queued
+// kernel with 5 / 4 blocks, x 30 hops, 500,000 walkers: U(0,1] s12 1.02 / 1.04,
+// s20 1.12 / 1.05, s22 1.11 / 1.05; lognormal s20 1.00 / 1.03, s22 0.97 / 1.00;
+// no weights s22 1.02 / 1.03; U(0,1] s20 300,000 walkers (two turns either way)
+// 0.98 / 1.05, 800,000 x 5 hops 0.85 / 1.02.  s22, one walker per node x 80
+// hops 7.04 / 7.21 ms; served queries on 8 streams 156 / 172 ms.
+constexpr long long kDenseRecords = 96ll << 20;  // bytes (s17: 118 MB; L2 holds 129 MB)
+constexpr double kDenseEnvelope = 2.0;
+constexpr int kDenseLength = 16;  // mean hops per walker
 struct LaunchShape {
   int variant;  // WalkVariant
   int grid, wpw;
@@ -1223,13 +1238,16 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
                               LaunchShape* s) {
   static_assert(kBlock == 32 * kShapeWarps, "place_walkers knows the block size");
   const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
-  bool scans = true, reservoir = true, exact = true, trials = false, rare = true;
+  bool scans = true, reservoir = true, exact = true, trials = false, rare = true, weighted = true;
+  long long hops = 0;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
     scans = scans && scan;
     reservoir = reservoir && jobs[i].mode == MODE_RVS;
     exact = exact && jobs[i].mode == MODE_EXACT;
     trials = trials || (!scan && jobs[i].weighted);
+    weighted = weighted && jobs[i].weighted;
+    hops += (long long)jobs[i].num_walkers * jobs[i].len;
     rare = rare && (jobs[i].mode == MODE_RJS || (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
   }
   int bps = 1;
@@ -1254,6 +1272,17 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
       s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
       if (e != cudaSuccess) return e;
+      if (ALG == ALGO_WEIGHTED && s->variant == V_QUEUED && weighted && 32ll * g->e >= kDenseRecords &&
+          g->envelope < kDenseEnvelope && hops >= total * kDenseLength) {
+        int dense = 1;
+        e = walk_blocks_per_sm<NJ, ALG>(V_QUEUED_DENSE, &dense);
+        if (e != cudaSuccess) return e;
+        auto turns = [&](int b) { return (total + (long long)g->num_sms * b * kBlock - 1) / ((long long)g->num_sms * b * kBlock); };
+        if (turns(dense) < turns(bps)) {
+          s->variant = V_QUEUED_DENSE;
+          bps = dense;
+        }
+      }
     }
   }
   if (!place.by_place)  // full warps, at most the resident blocks
