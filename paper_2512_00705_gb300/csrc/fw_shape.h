@@ -18,6 +18,29 @@ constexpr int kShapeWarps = 8;  // warps per block
 // 331, which keep less of a lone launch's gain on few streams.
 constexpr int kSharedWalkersJob = 16, kSharedWalkersTable = 2;
 
+// Walkers per warp of jobs that only scan rows, `row` entries long on average.
+// The warp scans one long row at a time, so that few walkers per warp leave no
+// warp with several hub rows at the end of a launch; short rows are their
+// lane's own work, and launches of more walkers than lanes (`many`) last long
+// enough to even out.  A histogram's walkers all scan one row.  GB300, R-MAT
+// s12 to s18, 5 hops, speed against full warps from a queue with 1 / 4 / 8 /
+// 16 / 32 walkers per warp: eRVS, weighted, 1,200,000 walkers, mean row 48
+// 0.56 / 0.79 / 0.90 / 1.00 / 1.05, 142 0.77 / 0.94 / 1.02 / 1.05 / 1.06, 745
+// 1.20 / 1.30 / 1.31 / 1.29 / 1.26; 60,000 walkers, row 192 1.63 / 1.65 / 1.68
+// (no more needed), 745 2.58 / 2.36 / 1.98; metapath (rows of a label's share)
+// 1,200,000 walkers, row 48 / 8 0.26 / 0.46 / 0.63 / 0.86 / 1.12.  Exact mode,
+// metapath, 1,200,000 walkers, row 48 0.67 / 0.84 / 0.95 / 1.04 / 1.09, 142
+// 0.92 / 1.00 / 1.05 / 1.06 / 1.08, 745 1.08 / 1.10 / 1.09 / 1.07 / 1.04;
+// 300,000 walkers, row 745 1.27 / 1.24 / 1.19 / 1.15 / 1.00; 60,000 walkers,
+// row 48 1.46 / 1.56 / 1.48 / 1.65, 250 2.20 / 1.88 / 1.67.
+constexpr double kTinyScan = 100.0, kShortScan = 250.0;
+inline int scan_walkers_per_warp(bool reservoir, bool histogram, double row, bool many) {
+  if (histogram) return 32;
+  if (row < kTinyScan) return reservoir ? 32 : 16;
+  if (row < kShortScan) return many || reservoir ? 8 : 1;
+  return many ? (reservoir ? 8 : 4) : 1;
+}
+
 struct WalkerPlacement {
   bool by_place;  // walkers are given to the warps by place; else they come from the queue, 32 per warp
   int wpw;        // walkers per warp

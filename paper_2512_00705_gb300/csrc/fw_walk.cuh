@@ -1188,10 +1188,9 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // spread over the resident warps before they share one -- wpw is the
 // smallest count with which they fit, and blocks fill before warps do.  No
 // queue counter is needed then.  Jobs that only scan rows (forced eRVS,
-// exact mode) keep one walker per warp at every size (eight where the rows
-// are short, see kShortScan), the rest in the queue:
-// the warp works for one walker at a time anyway, and a warp's lot of 14
-// walkers with hub rows made some warps run long after the others (65,536
+// exact mode) keep fewer walkers per warp (see scan_walkers_per_warp), the
+// rest in the queue: the warp works for one walker with a long row at a time
+// anyway, and a warp's lot of 14 made some warps run long after the others (65,536
 // walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
 // with 1, 8.2 in the variant that holds only eRVS; without exact mode's code
 // the others gain too: metapath s21 1.32 -> 1.31 ms, second-order PageRank
@@ -1207,14 +1206,6 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // 25.1, 1.5 28.0 / 27.6, 2 28.9 / 30.0, 4 33.7 / 40.8; s20 p = 4, q = 1/4 at
 // r = 1/4 4.80 / 4.20, 1 3.67 / 3.63, 1.5 3.90 / 4.05, 2 4.17 / 4.53.
 constexpr float kRareRatio = 1.5f;
-// Where eRVS rows are short (mean row of a walk below kShortScan; metapath: of
-// a label's share of it), most of them are their lane's own work and eight
-// walkers go to a warp.  60,000 walkers x 10 hops, 1 / 8 walkers per warp
-// (us): mean row 79 weighted 531 / 366, node2vec 876 / 624, metapath 312 /
-// 143; 142: 601 / 500, 1,018 / 901, 317 / 168; 241: 775 / 697, 1,243 / 1,280,
-// 429 / 255; 430: 995 / 1,009, 1,855 / 2,190, 372 / 225; 1,246: 1,793 /
-// 2,573, 4,051 / 5,364, 557 / 490.
-constexpr double kShortScan = 250.0;
 // Queued weighted walks take 5 blocks per SM (48 registers) instead of 4 where
 // that hides memory latency: edge records beyond L2, weights whose
 // envelope is low (few trials per hop), walks that are not short, and
@@ -1237,8 +1228,7 @@ template <int NJ, int ALG>
 inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                               LaunchShape* s) {
   static_assert(kBlock == 32 * kShapeWarps, "place_walkers knows the block size");
-  const double scanned = ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;
-  bool scans = true, reservoir = true, exact = true, trials = false, rare = true, weighted = true;
+  bool scans = true, reservoir = true, exact = true, trials = false, rare = true, weighted = true, histogram = true;
   long long hops = 0;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
@@ -1247,6 +1237,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     exact = exact && jobs[i].mode == MODE_EXACT;
     trials = trials || (!scan && jobs[i].weighted);
     weighted = weighted && jobs[i].weighted;
+    histogram = histogram && jobs[i].kind == JOB_HIST;
     hops += (long long)jobs[i].num_walkers * jobs[i].len;
     rare = rare && (jobs[i].mode == MODE_RJS || (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
   }
@@ -1267,7 +1258,10 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
     if (e != cudaSuccess) return e;
     const int fill = !scans && (ALG == ALGO_WEIGHTED || ALG == ALGO_METAPATH) ? kFirstOrderFill : kFillAll;
-    place = place_walkers(total, g->num_sms, bps, fill, scans, reservoir && scanned < kShortScan ? 8 : 1, NJ > 1, beside);
+    const double row = reservoir && ALG == ALGO_METAPATH ? g->mean_row / kLabelStats : g->mean_row;  // eRVS: a label's share
+    const bool many = total > (long long)g->num_sms * bps * kBlock;
+    place = place_walkers(total, g->num_sms, bps, fill, scans, scan_walkers_per_warp(reservoir, histogram, row, many),
+                          NJ > 1, beside);
     if (!place.by_place) {
       s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);

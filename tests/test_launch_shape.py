@@ -42,6 +42,12 @@ int main() {
           }
           if (!scan && beside > 1 && !p.by_place) CHECK(p.grid == (total + 255) / 256 || p.grid == blocks);
         }
+  // scans: full warps for short rows and histograms, few walkers per warp for long rows in small launches
+  CHECK3(fw::scan_walkers_per_warp(true, false, 48, true) == 32 && fw::scan_walkers_per_warp(false, false, 48, false) == 16);
+  CHECK3(fw::scan_walkers_per_warp(true, true, 5000, true) == 32 && fw::scan_walkers_per_warp(false, true, 5000, false) == 32);
+  CHECK3(fw::scan_walkers_per_warp(true, false, 1246, false) == 1 && fw::scan_walkers_per_warp(true, false, 1246, true) == 8);
+  CHECK3(fw::scan_walkers_per_warp(true, false, 150, false) == 8 && fw::scan_walkers_per_warp(false, false, 150, false) == 1);
+  CHECK3(fw::scan_walkers_per_warp(false, false, 150, true) == 8 && fw::scan_walkers_per_warp(false, false, 1246, true) == 4);
   // first-order: 60,000 walkers alone, 25 to a warp
   CHECK3(fw::place_walkers(60000, 152, 4, fw::kFirstOrderFill, false, 32, false, 1).wpw == 25);
   // 20,000 walkers on 152 SMs x 4 blocks: alone on every block, beside seven others in 79 blocks of full warps
