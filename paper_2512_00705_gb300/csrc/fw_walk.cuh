@@ -1217,7 +1217,7 @@ constexpr float kRareRatio = 1.5f;
 // hops 7.04 / 7.21 ms; served queries on 8 streams 156 / 172 ms.
 constexpr long long kDenseRecords = 96ll << 20;  // bytes (s17: 118 MB; L2 holds 129 MB)
 constexpr double kDenseEnvelope = 2.0;
-constexpr int kDenseLength = 16;  // mean hops per walker
+constexpr int kShortWalk = 16;  // walks of fewer hops (per walker, on average) are short
 struct LaunchShape {
   int variant;  // WalkVariant
   int grid, wpw;
@@ -1267,7 +1267,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
       if (e != cudaSuccess) return e;
       if (ALG == ALGO_WEIGHTED && s->variant == V_QUEUED && weighted && 32ll * g->e >= kDenseRecords &&
-          g->envelope < kDenseEnvelope && hops >= total * kDenseLength) {
+          g->envelope < kDenseEnvelope && hops >= total * kShortWalk) {
         int dense = 1;
         e = walk_blocks_per_sm<NJ, ALG>(V_QUEUED_DENSE, &dense);
         if (e != cudaSuccess) return e;
@@ -1291,18 +1291,26 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
 // a tuned rjs_batch as it is).  After a round the lanes that accepted move on
 // while the others wait, so a second trial pays where most lanes fail the
 // first: measured with 1 / 2 / 3 trials per round on GB300 (s20, ms), U(0,1]
-// weights q = 1/4 2.30 / 2.40 / 2.61 and q = 4 5.05 / 4.88 / 5.05, h = 1 q =
-// 1/4 1.80 / 1.95 / 1.99 and q = 4 3.74 / 3.81 / 4.10, metapath 1.52 / 1.43 /
-// 1.47; second-order PageRank 6.09 / 5.24 / 4.97 and 4.82 with 4; spread
-// launches, bound by latency, 0.369 / 0.331 / 0.326 and 0.318 with 4 (5,003
-// walkers), 57 / 48 / 46 and 45 with 4 (Pareto weights).  Queues of several
-// jobs mix lanes of q < 1 and q > 1 in a warp and keep 2 (64 mixed jobs: 8.54
-// ms, with 1 for q < 1 8.96); so do launches of whole scans (p = 4, q = 1/4, r
-// = 1/4 4.20, with 1 4.28).
-inline int32_t round_trials(const Job& J, int variant, int njobs) {
+// weights q = 1/4 2.30 / 2.40 / 2.61 and q = 4 5.05 / 4.88 / 5.05, metapath
+// 1.52 / 1.43 / 1.47; second-order PageRank 6.09 / 5.24 / 4.97 and 4.82 with 4;
+// spread launches, bound by latency, 0.369 / 0.331 / 0.326 and 0.318 with 4
+// (5,003 walkers), 57 / 48 / 46 and 45 with 4 (Pareto weights); mean speed of
+// 20,000 to 150,000 walkers x 5 hops with 4 / 3 / 2 against 2 from a queue:
+// node2vec 1.45 / 1.43 / 1.38, x 30 hops 1.38 / 1.38 / 1.37.  node2vec queues
+// with q < 1, 300,000 walkers, 1 / 2 against the earlier two: U(0,1] x 30 hops
+// 1.31 / 1.33 and at 160,000 to 1,000,000 1.44 / 1.37, x 5 hops 1.12 / 1.21; no
+// weights x 30 1.24 / 1.19, x 5 0.99 / 1.07; lognormal 1.16 / 1.34 and 0.95 /
+// 1.16: one for long walks and a low envelope only.  q = 4 without weights x
+// 30 hops 1.51 / 1.58: two.  Queues of several jobs mix lanes of q < 1 and q >
+// 1 in a warp and keep 2 (64 mixed jobs: 8.54 ms, with 1 for q < 1 8.96); so do
+// launches of whole scans (p = 4, q = 1/4, r = 1/4 4.20, with 1 4.28).
+constexpr double kOneTrialEnvelope = 2.0;
+inline int32_t round_trials(const fw_graph* g, const Job& J, int variant, int njobs) {
   if (J.round > 0) return J.round;
   if (variant >= V_SPREAD || J.algo == ALGO_PAGERANK2) return 4;
-  if (njobs == 1 && variant != V_QUEUED_WHOLE && J.algo == ALGO_NODE2VEC && J.need_member && (!J.weighted || J.inv_q > 1.0f)) return 1;
+  if (njobs == 1 && variant != V_QUEUED_WHOLE && J.algo == ALGO_NODE2VEC && J.inv_q > 1.0f &&
+      (!J.weighted || g->envelope < kOneTrialEnvelope) && J.len >= kShortWalk)
+    return 1;
   return kRjsBatchDefault;
 }
 
@@ -1317,7 +1325,7 @@ inline cudaError_t launch_walk_t(const fw_graph* g, const Job* jobs, int njobs, 
   JobTableN<NJ> tab;
   for (int i = 0; i < njobs; ++i) {
     tab.jobs[i] = jobs[i];
-    tab.jobs[i].round = round_trials(jobs[i], s.variant, njobs);
+    tab.jobs[i].round = round_trials(g, jobs[i], s.variant, njobs);
   }
   walk_variant<NJ, ALG>(s.variant)<<<s.grid, kBlock, 0, stream>>>(dev_graph(g), tab, njobs, total, s.wpw, qctr, g->d_err,
                                                                  g->d_cnt);
