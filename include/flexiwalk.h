@@ -170,7 +170,7 @@ typedef struct {
   float weight_scale;        /* largest per-node scale s_v after
                                 fw_graph_quantize_weights, else 0                */
   int32_t lane_max_degrees[4]; /* tuned launch shape per algorithm (fw_params)  */
-  int32_t rjs_batches[4];
+  int32_t rjs_batches[4];      /* (2 also where trials per round follow from the launch) */
   float trial_budgets[4];
 } fw_graph_info_t;
 
@@ -289,7 +289,7 @@ fw_status fw_graph_set_cost_ratio(fw_graph* graph, float ratio);
  *             3 % of the fastest time, keep the median
  *   method 2  method 1's sweep of r with 64-hop sample walks, then the launch
  *             shape one parameter at a time -- lane_max_degree in
- *             {1, 4, 8, 16, 32, 64}, rjs_batch in {1, 2, 3, 4, 6},
+ *             {1, 4, 8, 16, 32, 64}, rjs_batch in {default, 1, 2, 3, 4, 6},
  *             trial_budget in {0.25, 0.5, 1, 2, 4} -- each candidate kept
  *             only if its sample walk (best of three) is at least 2 %
  *             faster than the incumbent, then r swept again under the

@@ -135,8 +135,8 @@ fw_status make_job(const fw_graph* g, int32_t algo, const fw_params* params, uin
   }
   job->ratio = P.cost_ratio > 0.0f ? P.cost_ratio : g->ratio_algo[algo];
   job->lane_max = P.lane_max_degree > 0 ? P.lane_max_degree : g->lane_max_algo[algo];
-  job->rjs_batch = P.rjs_batch > 0 ? P.rjs_batch : g->rjs_batch_algo[algo];
-  job->round = P.rjs_batch > 0 || job->rjs_batch != kRjsBatchDefault ? job->rjs_batch : 0;
+  job->round = P.rjs_batch > 0 ? P.rjs_batch : g->rjs_batch_algo[algo];
+  job->rjs_batch = job->round > 0 ? job->round : kRjsBatchDefault;
   job->budget = P.trial_budget > 0.0f ? P.trial_budget : g->budget_algo[algo];
   job->key0 = (uint32_t)seed;
   job->key1 = (uint32_t)(seed >> 32);
@@ -517,7 +517,7 @@ extern "C" fw_status fw_graph_info(const fw_graph* g, fw_graph_info_t* info) {
   info->weight_scale = g->d_h8 ? g->hscale : 0.0f;
   for (int a = 0; a < 4; ++a) {
     info->lane_max_degrees[a] = g->lane_max_algo[a];
-    info->rjs_batches[a] = g->rjs_batch_algo[a];
+    info->rjs_batches[a] = g->rjs_batch_algo[a] > 0 ? g->rjs_batch_algo[a] : kRjsBatchDefault;
     info->trial_budgets[a] = g->budget_algo[a];
   }
   return FW_OK;

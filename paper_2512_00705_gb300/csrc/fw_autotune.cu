@@ -127,7 +127,8 @@ struct CacheKey {
   int method;
 };
 
-// A tuned result: r, and (method 2) the launch shape; 0 = not tuned.
+// A tuned result: r, and (method 2) the launch shape; 0 = not tuned
+// (rjs_batch: the launch's own rule was the fastest).
 struct Tuned {
   float r = 0.0f;
   int lane_max = 0, rjs_batch = 0;
@@ -149,7 +150,7 @@ bool cache_lookup(const char* path, const CacheKey& k, Tuned* t) {
                                 &fp, &algo, &p, &q, &gamma, &flags, &schema, &method, &rv, &lane, &batch, &budget);
     if ((got == 9 || got == 12) && fp == k.fp && algo == k.algo && p == k.p && q == k.q && gamma == k.gamma &&
         flags == k.flags && schema == k.schema && method == k.method && rv > 0.0f &&
-        (method != 2 || (got == 12 && lane >= 1 && lane <= 64 && batch >= 1 && batch <= 16 && budget > 0.0f))) {
+        (method != 2 || (got == 12 && lane >= 1 && lane <= 64 && batch >= 0 && batch <= 16 && budget > 0.0f))) {
       t->r = rv;
       t->lane_max = got == 12 ? lane : 0;
       t->rjs_batch = got == 12 ? batch : 0;
@@ -366,7 +367,7 @@ static fw_status sweep_shape(fw_graph* g, int32_t algo, const fw_params* params,
   if (g->e == 0) {
     out->r = 4.0f;
     out->lane_max = kLaneMaxDegree;
-    out->rjs_batch = kRjsBatchDefault;
+    out->rjs_batch = 0;
     out->budget = 1.0f;
     return FW_OK;
   }
@@ -375,7 +376,7 @@ static fw_status sweep_shape(fw_graph* g, int32_t algo, const fw_params* params,
   if (s != FW_OK) return s;
   fw_params P = sweep_params(params);
   P.lane_max_degree = kLaneMaxDegree;
-  P.rjs_batch = kRjsBatchDefault;
+  P.rjs_batch = 0;  // the launch's rule, so that what is timed is what an untuned or newly tuned walk runs
   P.trial_budget = 1.0f;
   P.cost_ratio = 4.0f;
   s = fw_walk(g, sm.starts, sm.w, sm.len, algo, &P, 7, sm.out, st);  // warm-up
@@ -440,7 +441,12 @@ extern "C" fw_status fw_autotune(fw_graph* g, int32_t algo, const fw_params* par
   if (!cached) {
     if (method == 0) s = profile_ratio(g, J, st, &t.r);
     else if (method == 1) s = sweep_ratio(g, algo, params, st, &t);
-    else s = sweep_shape(g, algo, params, st, &t);
+    else {
+      const int32_t installed = g->rjs_batch_algo[algo];
+      g->rjs_batch_algo[algo] = 0;  // an earlier tuning's value is no rule
+      s = sweep_shape(g, algo, params, st, &t);
+      g->rjs_batch_algo[algo] = installed;
+    }
     if (s != FW_OK) return s;
     if (!(t.r > 0.0f) || !std::isfinite(t.r)) return set_error(FW_ERR_CUDA, "profiling gave no usable ratio");
     if (cache_path && cache_path[0]) cache_store(cache_path, key, t);

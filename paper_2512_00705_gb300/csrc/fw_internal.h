@@ -50,8 +50,7 @@ struct fw_graph {
   float ratio_algo[4] = {4.0f, 4.0f, 4.0f, 4.0f};  // r of Eq. (runtime) per algorithm (fw_algo order)
   // launch shape per algorithm (fw_params lane_max_degree, rjs_batch, trial_budget), tuned by method 2
   int32_t lane_max_algo[4] = {fw::kLaneMaxDegree, fw::kLaneMaxDegree, fw::kLaneMaxDegree, fw::kLaneMaxDegree};
-  int32_t rjs_batch_algo[4] = {fw::kRjsBatchDefault, fw::kRjsBatchDefault, fw::kRjsBatchDefault,
-                               fw::kRjsBatchDefault};
+  int32_t rjs_batch_algo[4] = {0, 0, 0, 0};  // 0: by the launch's rule (round_trials)
   float budget_algo[4] = {1.0f, 1.0f, 1.0f, 1.0f};
   unsigned long long fingerprint = 0;
   double preprocess_ms = 0.0;
