@@ -560,8 +560,8 @@ struct Accept {
 // mass is (1/q) d + (1 - 1/q) d' < d, so fewer trials than the one-envelope
 // bound max(1, 1/q) h_MAX = h_MAX (B = h_MAX is passed in this case).
 //
-// Lane eRVS (rvs: a reservoir step over a row that the walker's own lane
-// scans, rvs_pick<1>): "trial" t is the scan's position t, so such a lane
+// Lane eRVS (rvs, node2vec only: a reservoir step over a row that the walker's
+// own lane scans, rvs_pick<1>): "trial" t is the scan's position t, so such a lane
 // moves in step with its warp's eRJS lanes instead of stalling them for the
 // whole row: its record load and membership test are the trials' own, its
 // Philox block is (wid, hop, 6, 0) for position 0 and (wid, hop, 2, t)
@@ -574,6 +574,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
                                            float& beta, int32_t& pos_ret, float h_ret, int32_t t0, int32_t nt,
                                            Accept& acc, LaneCounters& lc, bool csplit, float& beta2, bool grp,
                                            int32_t lane_rvs = kLaneNone) {
+  static_assert(!LANE_RVS || ALG == ALGO_NODE2VEC, "lane eRVS knows node2vec's weights and rows");
   const bool rvs = LANE_RVS && lane_rvs != kLaneNone;
   const bool keyed = LANE_RVS && lane_rvs == kLaneKeyed;
   const uint32_t d = (uint32_t)c.d;
@@ -600,7 +601,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
       break;
     }
     int4 a, b;  // {col, h, target row start, target degree}, {target h_MAX, target h_SUM, label, 0}
-    if ((FW_ALGO(J) == ALGO_METAPATH) && grp && !rvs) {
+    if ((FW_ALGO(J) == ALGO_METAPATH) && grp) {
       // metapath inside the required label's segment [c.ps, c.pe) of the grouped
       // arrays, every entry of w = 1, ordered by weight class: slot t of the
       // class envelope (class_slots) proposes an entry of class c in proportion
@@ -685,7 +686,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
     const int4* er;
     if (rvs) {
       ku = (uint32_t)t;
-      er = (FW_ALGO(J) == ALGO_METAPATH) && grp ? g.gerec + 2ll * (c.ps + t) : g.erec + 2ll * (c.s + t);
+      er = g.erec + 2ll * (c.s + t);
     } else if (c.n0 >= 0) {
       // three weight classes of bounds B, B / 2, B / 4 (h <= h_MAX / 2^c in class c): slot t of
       // 4 n0 + 2 n1 + n2 proposes an entry of class c in proportion to its bound
@@ -716,16 +717,14 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
     bool adj = false;
     if (second ? (u != c.vp && (rvs ? J.need_member != 0
                                     : !csplit && UB < __fmul_rn(J.whi1, hk) && UB >= __fmul_rn(J.wlo1, hk)))
-               : (pr2 && (rvs || (!split && UB < __fmul_rn(c.w1, hk) && UB >= __fmul_rn(c.w2, hk))))) {
+               : (pr2 && !split && UB < __fmul_rn(c.w1, hk) && UB >= __fmul_rn(c.w2, hk))) {
       uint32_t pb = 0;
       adj = prev_contains<ALG == ALGO_PAGERANK2>(g, J, c, u, pb);
       probes += pb;
     }
     if (rvs) {
-      float wt;
-      if (second) wt = __fmul_rn(u == c.vp ? J.inv_p : (adj || !J.need_member ? 1.0f : J.inv_q), hk);
-      else if (FW_ALGO(J) == ALGO_METAPATH) wt = grp || (uint8_t)b.z == want ? hk : 0.0f;
-      else wt = pr2 ? __fmul_rn(adj ? c.w1 : c.w2, hk) : hk;
+      const float wt =
+          second ? __fmul_rn(u == c.vp ? J.inv_p : (adj || !J.need_member ? 1.0f : J.inv_q), hk) : hk;
       if (COUNT) lc.rvs_items++;
       if (t == 0) {
         beta2 = -CUDART_INF_F;
@@ -746,8 +745,7 @@ __device__ __forceinline__ bool rjs_trials(const DevGraph& g, const Job& J, cons
           if (jump) beta = (beta2 < 0.0f) ? logf(u01_open(t == 0 ? x.w : x.z)) / beta2 : CUDART_INF_F;
         }
       }
-      const int32_t len = (FW_ALGO(J) == ALGO_METAPATH) && grp ? c.pe - c.ps : c.d;
-      if (t + 1 >= len) {
+      if (t + 1 >= c.d) {
         if (beta2 == -CUDART_INF_F) pos_ret = -1;
         found = true;
         break;
