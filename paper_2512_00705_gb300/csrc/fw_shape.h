@@ -74,7 +74,10 @@ constexpr int kFirstOrderFill = 2, kFillAll = 64;
 // them.  GB300, s22 x 40 hops on 8 streams, every launch spread over the GPU
 // -> its share of it (us per launch): node2vec 3,000 walkers 60 -> 32, 20,000
 // 184 -> 68, 60,000 313 -> 127 (full warps always: 59 / 75 / 169); batches of
-// 64 served queries 583 -> 463 ms.
+// 64 served queries 583 -> 463 ms.  The algorithms of one batch do not count:
+// a plan's parallel branches last as long as their longest, which gains more
+// from the whole GPU than the others lose (47 plans of 2 to 64 jobs, branches
+// sharing / alone: 1.62 / 1.89 times the speed of full warps).
 inline WalkerPlacement place_walkers(long long total, int sms, int bps, int fill, bool scans, int scan_wpw, bool table,
                                      int beside) {
   WalkerPlacement p;

@@ -66,7 +66,8 @@ cudaError_t launch_walk_mixed(const fw_graph* g, const Job* jobs, int njobs, boo
   for (int i = 0; i < np && e == cudaSuccess; ++i) {
     const int a = present[i];
     cudaStream_t st = (fork && i > 0) ? side[i - 1] : stream;
-    e = table_launches(a).launch(g, grp + firsts[a], counts[a], totals[a], count, fork ? beside * np : beside, qctr + a, st);
+    // the branches of one call are shaped as if alone: the longest decides when it ends (see fw_shape.h)
+    e = table_launches(a).launch(g, grp + firsts[a], counts[a], totals[a], count, beside, qctr + a, st);
   }
   if (fork) {  // `stream` waits for the helper streams
     for (int i = 1; i < np && e == cudaSuccess; ++i) {
