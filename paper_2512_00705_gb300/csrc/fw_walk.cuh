@@ -442,6 +442,23 @@ __device__ __forceinline__ int32_t hub_step(const DevGraph& g, const Job* sj, co
 template <int ALG>
 constexpr int32_t kTogetherFrom = ALG == ALGO_PAGERANK2 ? 16 : 8;
 constexpr double kTogetherEnvelope = 5.0, kTogetherPagerank = 2.5;
+// It pays where a launch ends with its longest steps; where all walkers' hops
+// outweigh them, the lanes' own trials are the faster ones.  The more so the
+// lower the envelope E: launches of up to kTogetherHops * E hops in all (and
+// metapath, whose steps see a label's share of a row, kTogetherHopsLeast).
+// GB300, speed against the earlier kernel, together / a lane's own: Pareto 2
+// (E = 5 to 8 on s16 / s18 / s20) node2vec p = 2, q = 1/2 2.0 M hops 1.14 /
+// 2.47 / 1.36 and 1.10 / 0.93 / 0.96, 3.6 M 0.84 / 1.21 / 1.00 and 1.31 / 1.31
+// / 1.25, 12 M 0.80 / 0.88 / 0.79 and 1.47 / 1.14 / 1.11, 45 M 0.76 / 0.71 /
+// 0.62 and 1.61 / 1.34 / 1.30; weighted 12 M 1.32 / 1.68 / 1.20 and 1.02 /
+// 0.97 / 1.00, 45 M 0.83 / 0.98 / 0.91 and 0.99 / 0.99 / 1.01; metapath 2.0 M
+// 1.12 / 1.92 / 1.46 and 1.02 / 0.98 / 0.98, 12 M 0.88 / 1.04 / 0.95 and 1.05
+// / 1.01 / 1.01.  Pareto 1 (E = 75 and more): node2vec 45 M 1.04 / 1.14 / 1.15
+// and 1.12 / 1.08 / 1.04, weighted 45 M 1.13 / 1.45 / 1.69 and 0.97 / 0.98 /
+// 0.97, metapath 12 M 0.85 / 1.29 / 1.96 and 1.00 / 0.99 / 0.97.
+template <int ALG>
+constexpr double kTogetherHops = ALG == ALGO_WEIGHTED ? 2.5e6 : ALG == ALGO_NODE2VEC ? 0.4e6 : 0.09e6;
+constexpr double kTogetherHopsLeast = 2.5e6;
 
 // The walk loop of one warp over one queue: take walkers, plan, sample and
 // write rows until the queue is exhausted and the warp holds no walker.
@@ -1248,8 +1265,10 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
   WalkerPlacement place = {false, 32, 0};
   s->variant = V_COUNTING;
   if (!count) {
+    const double most = std::max(kTogetherHops<ALG> * g->envelope, ALG == ALGO_METAPATH ? kTogetherHopsLeast : 0.0);
     const bool together = ALG == ALGO_PAGERANK2 ? !scans && (total <= lanes || g->envelope >= kTogetherPagerank)
-                                                : trials && g->envelope >= kTogetherEnvelope;
+                                                : trials && g->envelope >= kTogetherEnvelope &&
+                                                      (double)hops <= most;
     s->variant = hub_share_pays(g, jobs, njobs, total, lanes) ? V_SPREAD_SHARE
                  : reservoir                                  ? V_SPREAD_RVS
                  : exact                                      ? V_SPREAD_EXACT
