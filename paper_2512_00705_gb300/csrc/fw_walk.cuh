@@ -1222,6 +1222,12 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
 // in step / whole (ms), s22 p = 1/4, q = 4 at r = 1/4 26.6 / 24.1, 1 27.2 /
 // 25.1, 1.5 28.0 / 27.6, 2 28.9 / 30.0, 4 33.7 / 40.8; s20 p = 4, q = 1/4 at
 // r = 1/4 4.80 / 4.20, 1 3.67 / 3.63, 1.5 3.90 / 4.05, 2 4.17 / 4.53.
+// So do walks with q = 1, whose scans need no membership test, at any ratio:
+// 200,000 to 2,000,000 walkers x 4 / 10 / 30 hops, s12 to s21, r = 4, speed
+// against the earlier kernel, in step and whole: p = 4 no weights 0.82 / 0.87 /
+// 0.90 and 1.13 / 1.11 / 1.08, U(0,1] 1.02 / 1.07 / 1.07 and 1.14 / 1.17 / 1.15;
+// p = 1/2 no weights 1.02 / 1.04 / 1.06 and 1.40 / 1.37 / 1.32, 8-bit weights
+// 0.99 / 0.98 / 0.98 and 1.17 / 1.17 / 1.15.
 constexpr float kRareRatio = 1.5f;
 // Queued weighted walks take 5 blocks per SM (48 registers) instead of 4 where
 // that hides memory latency: edge records beyond L2, weights whose
@@ -1245,7 +1251,7 @@ template <int NJ, int ALG>
 inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, long long total, bool count, int beside,
                               LaunchShape* s) {
   static_assert(kBlock == 32 * kShapeWarps, "place_walkers knows the block size");
-  bool scans = true, reservoir = true, exact = true, trials = false, rare = true, weighted = true, histogram = true;
+  bool scans = true, reservoir = true, exact = true, trials = false, whole = true, weighted = true, histogram = true;
   long long hops = 0;
   for (int i = 0; i < njobs; ++i) {
     const bool scan = jobs[i].mode == MODE_RVS || jobs[i].mode == MODE_EXACT;
@@ -1256,7 +1262,8 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     weighted = weighted && jobs[i].weighted;
     histogram = histogram && jobs[i].kind == JOB_HIST;
     hops += (long long)jobs[i].num_walkers * jobs[i].len;
-    rare = rare && (jobs[i].mode == MODE_RJS || (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
+    whole = whole && (!jobs[i].need_member || jobs[i].mode == MODE_RJS ||
+                      (jobs[i].mode == MODE_AUTO && jobs[i].ratio < kRareRatio));
   }
   int bps = 1;
   cudaError_t e = walk_blocks_per_sm<NJ, ALG>(count ? V_COUNTING : V_QUEUED, &bps);
@@ -1282,7 +1289,7 @@ inline cudaError_t walk_shape(const fw_graph* g, const Job* jobs, int njobs, lon
     place = place_walkers(total, g->num_sms, bps, fill, scans, scan_walkers_per_warp(reservoir, histogram, row, many),
                           NJ > 1, beside);
     if (!place.by_place) {
-      s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && rare ? V_QUEUED_WHOLE : V_QUEUED;
+      s->variant = together ? V_QUEUED_TOGETHER : ALG == ALGO_NODE2VEC && whole ? V_QUEUED_WHOLE : V_QUEUED;
       e = walk_blocks_per_sm<NJ, ALG>(s->variant, &bps);
       if (e != cudaSuccess) return e;
       if (ALG == ALGO_WEIGHTED && s->variant == V_QUEUED && weighted && 32ll * g->e >= kDenseRecords &&

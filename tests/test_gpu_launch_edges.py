@@ -26,12 +26,12 @@ def graph(request):
     G.close()
 
 
-ALGOS = [("weighted", 1.0, 1.0), ("node2vec", 2.0, 0.5), ("node2vec", 0.25, 4.0), ("metapath", 1.0, 1.0),
-         ("pagerank2", 1.0, 1.0)]
+ALGOS = [("weighted", 1.0, 1.0), ("node2vec", 2.0, 0.5), ("node2vec", 0.25, 4.0), ("node2vec", 4.0, 1.0),
+         ("node2vec", 0.5, 1.0), ("metapath", 1.0, 1.0), ("pagerank2", 1.0, 1.0)]
 
 
 @pytest.mark.parametrize("algo,p,q", ALGOS)
-@pytest.mark.parametrize("mode,ratio", [("auto", 4.0), ("auto", 8.0), ("auto", 0.5), ("rjs", 0.0)])
+@pytest.mark.parametrize("mode,ratio", [("auto", 4.0), ("auto", 8.0), ("auto", 0.5), ("rjs", 0.0), ("random", 0.0)])
 def test_lanes_run_out(graph, algo, p, q, mode, ratio):
     g, G, sms, starts = graph
     kw = dict(p=p, q=q, mode=mode, cost_ratio=ratio, schema=[0, 1, 2] if algo == "metapath" else None, seed=8)
