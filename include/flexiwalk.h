@@ -553,6 +553,10 @@ fw_status fw_gather_ceiling(void* table, uint64_t table_bytes, double* rate_out,
 /* Number of kernel launches this library has issued (process-wide). */
 uint64_t fw_launch_count(void);
 
+/* Number of times this library has taken queue counters from a graph's pool
+ * (process-wide): walks whose walkers come from a queue, and batches. */
+uint64_t fw_counter_allocation_count(void);
+
 /* Message of the last failing call of this thread ("" if none); the
  * pointer stays valid until this thread's next call into the library. */
 const char* fw_last_error(void);

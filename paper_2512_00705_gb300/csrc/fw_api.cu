@@ -14,6 +14,7 @@
 namespace fw {
 
 std::atomic<unsigned long long> g_launches{0};
+static std::atomic<unsigned long long> g_counter_allocs{0};
 
 static thread_local std::string t_last_error;
 
@@ -73,6 +74,7 @@ static void create_counter_pool(fw_graph* g) {
 }
 
 cudaError_t alloc_counters(const fw_graph* g, int count, unsigned long long** out, cudaStream_t st) {
+  g_counter_allocs.fetch_add(1);
   const size_t bytes = sizeof(unsigned long long) * (size_t)count;
   void** p = reinterpret_cast<void**>(out);
   cudaError_t e = g->counter_pool ? cudaMallocFromPoolAsync(p, bytes, g->counter_pool, st) : cudaMallocAsync(p, bytes, st);
@@ -352,6 +354,8 @@ extern "C" const char* fw_status_string(fw_status s) {
 }
 
 extern "C" uint64_t fw_launch_count(void) { return g_launches.load(); }
+
+extern "C" uint64_t fw_counter_allocation_count(void) { return g_counter_allocs.load(); }
 
 // Host-side CSR validation (runs before any CUDA call).
 static fw_status validate_host_csr(const int32_t* off, const int32_t* col, const float* h, int32_t n, int64_t e) {
