@@ -51,8 +51,8 @@ def _inputs_digest() -> str:
 
 # The files that define the walk kernel and the device data it reads (records,
 # filters, label-grouped view): profiles of the kernel are keyed to their digest.
-WALK_KERNEL_FILES = ["fw_device.cuh", "fw_walk.cuh", "fw_kernels.cu", "fw_walk_mixed.cu", "fw_preprocess.cu", "fw_internal.h",
-                     "fw_api.cu"]
+WALK_KERNEL_FILES = ["fw_device.cuh", "fw_walk.cuh", "fw_shape.h", "fw_kernels.cu", "fw_walk_mixed.cu", "fw_preprocess.cu",
+                     "fw_rows.h", "fw_internal.h", "fw_api.cu"]
 
 
 def _code_only(text: str) -> str:

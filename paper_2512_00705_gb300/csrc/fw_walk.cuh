@@ -1,6 +1,6 @@
-// fw_walk.cuh -- the walk kernel: its loop, the kernel template and its
-// launcher, instantiated for single jobs (fw_kernels.cu) and for tables of
-// up to 64 jobs of one algorithm (fw_walk_mixed.cu).
+// fw_walk.cuh -- the walk kernel: its loop, the kernel template, its variants
+// and their launcher, instantiated for single jobs (fw_walk_single_*.cu) and
+// for tables of up to 64 jobs of one algorithm (fw_walk_table_*.cu).
 //
 // One warp runs the loop over one walker queue [Sec. 5.3]:
 //   * query fetch   lanes without a walker take the next global walker
@@ -1198,25 +1198,26 @@ inline bool hub_share_pays(const fw_graph* g, const Job* jobs, int njobs, long l
   return rvs;
 }
 
-// The shape of one launch.  While every walker can have a lane of its own
-// (`spread`), walkers go to their warps by place, `wpw` to a warp (the other
-// lanes stay idle): a warp pays for the longest of its lanes' paths in every
-// iteration and scans its lanes' long rows one after another, so walkers are
-// spread over the resident warps before they share one -- wpw is the
-// smallest count with which they fit, and blocks fill before warps do.  No
-// queue counter is needed then.  Jobs that only scan rows (forced eRVS,
-// exact mode) keep fewer walkers per warp (see scan_walkers_per_warp), the
-// rest in the queue: the warp works for one walker with a long row at a time
-// anyway, and a warp's lot of 14 made some warps run long after the others (65,536
-// walkers x 20 hops, s18: 12.9 ms with wpw 14, 11.8 with 4, 11.2 with 2, 10.9
-// with 1, 8.2 in the variant that holds only eRVS; without exact mode's code
-// the others gain too: metapath s21 1.32 -> 1.31 ms, second-order PageRank
-// s20 4.36 -> 4.24, 5,003 walkers 351 -> 338 us).  Other launches with more
-// walkers than lanes: full warps that fetch from the queue.  Measured on GB300 (R-MAT s18 / s20, one launch of
-// full warps from a queue -> spread): 37 walkers x 10 hops 86 -> 28 us, 5,003
-// x 63 hops 1,152 -> 388 us, 65,536 x 20 hops of eRVS 22.4 -> 13.5 ms.  A
-// kernel variant of its own, because the same choice made inside the queued
-// kernel's fetch cost the whole-graph walks 1 to 3 %.
+// The shape of one launch.  While every walker can have a lane of its own, and
+// no other launches run beside, walkers go to their warps by place, `wpw` to a
+// warp (the other lanes stay idle): a warp pays for the longest of its lanes'
+// paths in every iteration and scans its lanes' long rows one after another, so
+// walkers are spread over the resident warps before they share one, and blocks
+// fill before warps do (place_walkers).  No queue counter is needed then.
+// Jobs that only scan rows (forced eRVS, exact mode) keep fewer walkers per
+// warp (see scan_walkers_per_warp), the rest in the queue: the warp works for
+// one walker with a long row at a time anyway, and a warp's lot of 14 made some
+// warps run long after the others (65,536 walkers x 20 hops, s18: 12.9 ms with
+// wpw 14, 11.8 with 4, 11.2 with 2, 10.9 with 1, 8.2 in the variant that holds
+// only eRVS; without exact mode's code the others gain too: metapath s21 1.32
+// -> 1.31 ms, second-order PageRank s20 4.36 -> 4.24, 5,003 walkers 351 -> 338
+// us).  Other launches: full warps that fetch from the queue.  Measured on
+// GB300 (R-MAT s18 / s20, one launch of full warps from a queue -> spread): 37
+// walkers x 10 hops 86 -> 28 us, 5,003 x 63 hops 1,152 -> 388 us, 65,536 x 20
+// hops of eRVS 22.4 -> 13.5 ms.  A kernel variant of its own, because the same
+// choice made inside the queued kernel's fetch cost the whole-graph walks 1 to
+// 3 %.
+//
 // Below this cost ratio, as tuning picks it, eRVS steps are rare and node2vec
 // keeps whole scans, as the code of scans in step costs the trials registers:
 // in step / whole (ms), s22 p = 1/4, q = 4 at r = 1/4 26.6 / 24.1, 1 27.2 /
