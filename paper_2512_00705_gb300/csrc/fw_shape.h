@@ -73,8 +73,9 @@ constexpr int kFirstOrderFill = 2, kFillAll = 64;
 // next launch.  So a launch takes its share of the blocks only and fills
 // them.  GB300, s22 x 40 hops on 8 streams, every launch spread over the GPU
 // -> its share of it (us per launch): node2vec 3,000 walkers 60 -> 32, 20,000
-// 184 -> 68, 60,000 313 -> 127 (full warps always: 59 / 75 / 169); batches of
-// 64 served queries 583 -> 463 ms.  The algorithms of one batch do not count:
+// 185 -> 64, 60,000 315 -> 127 (full warps always: 53 / 72 / 169), weighted 42
+// -> 19, 109 -> 30, 155 -> 61 (25 / 31 / 63); batches of 64 served queries 583
+// -> 463 ms.  The algorithms of one batch do not count:
 // a plan's parallel branches last as long as their longest, which gains more
 // from the whole GPU than the others lose (47 plans of 2 to 64 jobs, branches
 // sharing / alone: 1.62 / 1.89 times the speed of full warps).
